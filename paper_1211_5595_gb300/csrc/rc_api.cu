@@ -875,6 +875,13 @@ static rc_status ensure_occupancy(rc_context *ctx, rc_volume *v, int f) {
     return RC_OK;
 }
 
+// What a render's empty-space skipping reads: the occupancy masks for
+// compositing, the block maxima for MIP and the first-hit functions.
+static rc_status ensure_skip(rc_context *ctx, rc_volume *v, const rc_render_params *p) {
+    if (!p->skip || p->func == RC_FUNC_AVERAGE || p->func == RC_FUNC_XRAY) return RC_OK;
+    return p->func == RC_FUNC_COMPOSITE ? ensure_occupancy(ctx, v, p->filter) : ensure_grid(ctx, v, p->filter);
+}
+
 // Copies the device counters into *stats (synchronises the stream). The
 // importance kernels count fallback rays in the first slot.
 // Zeroes the statistics counters and marks the start of a call's device work
@@ -942,6 +949,13 @@ static MarchArgs march_args(rc_context *ctx, const rc_volume *v, const rc_render
     a.p.filter = p->filter;
     a.occ = v->d_occ[p->filter];
     a.fine = v->d_fine[p->filter];
+    a.mx = v->d_mx[p->filter];
+    a.mx4 = v->d_mx4[p->filter];
+    for (int i = 0; i < 2; i++) a.c4[i] = (v->n[i] - 1 + 3) / 4;
+    // FP32 reconstruction rounds by less than 2^-18 of full scale; FP16 codes
+    // beyond 12 bits are stored to within 2^-12 of the offset
+    a.slack = (float)v->vmax * (1.0f / 65536.0f) +
+              (v->storage == RC_STORE_F16 && v->vmax > 4096 ? o * (1.0f / 2048.0f) : 0.0f);
     a.out = reinterpret_cast<float4 *>(out);
     a.stats = nullptr;
     a.cams = nullptr;
@@ -956,10 +970,8 @@ rc_status rc_render(rc_context *ctx, const rc_volume *vol, const rc_render_param
     if (st != RC_OK) return st;
     DeviceScope ds(ctx->device);
     rc_volume *v = const_cast<rc_volume *>(vol);
-    if (p->skip && p->func == RC_FUNC_COMPOSITE) {
-        st = ensure_occupancy(ctx, v, p->filter);
-        if (st != RC_OK) return st;
-    }
+    st = ensure_skip(ctx, v, p);
+    if (st != RC_OK) return st;
     st = prepare_filter(ctx, v, p);
     if (st != RC_OK) return st;
     MarchArgs a = march_args(ctx, v, p, out_rgba);
@@ -981,10 +993,8 @@ rc_status rc_render_views(rc_context *ctx, const rc_volume *vol, const rc_render
     if (st != RC_OK) return st;
     DeviceScope ds(ctx->device);
     rc_volume *v = const_cast<rc_volume *>(vol);
-    if (p->skip && p->func == RC_FUNC_COMPOSITE) {
-        st = ensure_occupancy(ctx, v, p->filter);
-        if (st != RC_OK) return st;
-    }
+    st = ensure_skip(ctx, v, p);
+    if (st != RC_OK) return st;
     st = prepare_filter(ctx, v, p);
     if (st != RC_OK) return st;
     CamRec first;
@@ -1075,10 +1085,8 @@ rc_status rc_render_views_host(rc_context *ctx, const rc_volume *vol, const rc_r
             return fail(ctx, RC_ERR_INVALID_ARG, "%s: host_rgba is device memory (use rc_render_views)", who);
     }
     rc_volume *v = const_cast<rc_volume *>(vol);
-    if (p->skip && p->func == RC_FUNC_COMPOSITE) {
-        st = ensure_occupancy(ctx, v, p->filter);
-        if (st != RC_OK) return st;
-    }
+    st = ensure_skip(ctx, v, p);
+    if (st != RC_OK) return st;
     st = prepare_filter(ctx, v, p);
     if (st != RC_OK) return st;
     CamRec first;

@@ -106,6 +106,12 @@ struct MarchArgs {
     MarchParams p;
     const uint8_t *occ;            // cell-brick occupancy (1 = may be non-empty)
     const unsigned long long *fine;   // compositing: per cell-brick, one bit per 4^3 sub-block (or null)
+    // ray functions that skip by block maxima: largest code of each cell-brick
+    // and of each 4^3 sub-block (c4[0] x c4[1] x ceil((n-1)/4) of them), and
+    // the margin in code units by which a value may exceed its block's maximum
+    const uint16_t *mx, *mx4;
+    int c4[2];
+    float slack;
     float4 *out;                   // H x W RGBA (view-major for several views)
     unsigned long long *stats;     // dense, evaluated, hit, total (or null)
     const CamRec *cams;            // one record per view (blockIdx.z), or null: cam

@@ -101,13 +101,48 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     if (a.stats) add_stats(a.stats, (unsigned)min(k, nsamp), evald, hit ? 1u : 0u, inimg ? 1u : 0u);
 }
 
+// Ray function groups: the functions of one group share a loop.
+enum : int { kFnMip = 0, kFnSum = 1, kFnFirst = 2 };    // MIP | average, x-ray | isosurface, threshold
+
+// The largest block around cell c (brick b) whose codes cannot matter to a
+// search for values above `need` (code units): 4 for the cell-brick, 2 for the
+// 4^3 sub-block, -1 when the sample has to be evaluated. A block's maximum
+// code bounds every value reconstructed in it up to FP32 rounding (and, for
+// FP16 storage of more than 12 bits, the rounding of the stored values);
+// a.slack covers both many times over, so a skipped sample is strictly below
+// `need`.
+__device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int b, float need) {
+    const int j = ((c.i[2] >> 2) * a.c4[1] + (c.i[1] >> 2)) * a.c4[0] + (c.i[0] >> 2);
+    if ((float)__ldg(a.mx4 + j) + a.slack > need) return -1;
+    return (float)__ldg(a.mx + b) + a.slack > need ? 2 : 4;
+}
+
 // The other ray functions of Sec. 4.1 (MIP, average, x-ray, isosurface,
 // threshold); output channels as documented in rc.h. CUBIC: B-spline values
 // and analytic gradient instead of trilinear values and central differences.
-template <int ST, bool CUBIC>
+//
+// MIP and the first-hit functions march the block maxima instead of every
+// sample: a sample in a 4^3 sub-block or cell-brick whose largest code cannot
+// exceed the ray's maximum so far (or reach the iso-value) changes nothing, so
+// the ray jumps over the block (the compositing march's exact jump, verified
+// on the sample grid). A warp jumps only when none of its lanes has to
+// evaluate: in noise the lanes' blocks alternate, and a jump costs more than
+// the sample it saves. The maximum does not depend on the order, so MIP first
+// takes samples eight voxels apart and so starts from nearly the ray's
+// maximum, with the space in front of the brightest tissue to skip as well.
+// The value before a first hit is reconstructed once, when the hit is found.
+// Average and x-ray sum every sample.
+// Instruction issue bounds it (76% with every sample evaluated, L1 54%, DRAM
+// 3%). 256x256x180 phantom at 1024^2: 4 isosurface views 0.725 -> 0.283 ms,
+// 8 MIP views 2.44 -> 2.15 ms (the noise around the head has block maxima
+// above any value reconstructed in it, so 60% of the samples stay; jumping
+// lane by lane instead of by warp 2.55, with samples four voxels apart first
+// 2.60).
+template <int ST, bool CUBIC, int FN>
 __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs a) {
     extern __shared__ float4 s_tf[];
-    if (a.p.func == RC_FUNC_THRESHOLD) {   // the only one that classifies (1-D table)
+    const int func = a.p.func;
+    if (FN == kFnFirst && func == RC_FUNC_THRESHOLD) {   // the only one that classifies (1-D table)
         load_tf(a.tf, s_tf);
         __syncthreads();
     }
@@ -119,60 +154,119 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
     Ray R;
     const bool hit = inimg && setup_ray(cam, a.vol, a.p.step_vox, x, y, R);
     const int nsamp = hit ? R.nsamp : 0;
-    const int func = a.p.func;
     float4 out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float acc = 0.0f, prev_v = 0.0f, prev_t = 0.0f;
+    float acc = FN == kFnMip ? -__int_as_float(0x7f800000) : 0.0f;
     int k = 0;
-    bool found = false;
-    for (; k < nsamp; k++) {
-        float t = sample_t(R, k), p[3];
-        position_at(R, t, p);
-        Cell c;
+    unsigned evald = 0;
+    int hit_k = -1;
+    auto value = [&](const Cell &c) { return CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c); };
+    // thresholds in code units: FP16 storage holds h = code / o - 1
+    auto in_codes = [&](float v) { return ST == RC_STORE_F16 ? (v + 1.0f) * a.vol.f16o : v; };
+    float need = FN == kFnFirst ? in_codes(a.p.iso) : acc;
+    auto cell_at = [&](int j, Cell &c) {
+        float p[3];
+        position_at(R, sample_t(R, j), p);
         cell_of(a.vol, p, c);
-        float v = CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c);
-        if (func == RC_FUNC_MIP) {
-            acc = k == 0 ? v : fmaxf(acc, v);
-        } else if (func == RC_FUNC_AVERAGE || func == RC_FUNC_XRAY) {
-            acc += v;
-        } else if (v >= a.p.iso) {
-            found = true;
-            if (func == RC_FUNC_THRESHOLD) {
-                float4 e = classify(s_tf, a.tf.K, tf_coord<ST>(v, a.tf.ucoef), nullptr, nullptr, RC_DBG_ERR(a.vol));
-                out = make_float4(e.x, e.y, e.z, 1.0f);
-            } else {
-                float ts = k > 0 ? prev_t + (t - prev_t) * ((a.p.iso - prev_v) / (v - prev_v)) : t;
-                float g[3], sf, spec;
-                if (CUBIC) bspline_grad<ST>(a.vol, c, g);
-                else value_grad<ST>(a.vol, c, g);
-                shade_factor(a.p, a.vol, g, R.dir, sf, spec);
-                out = make_float4(ts, fminf(1.0f, sf + spec), (float)k, 1.0f);
+    };
+    if (FN == kFnMip && a.p.skip) {
+        const int stride = (int)fminf(8.0f / a.p.step_vox, 4096.0f);
+        for (int j = stride >> 1; stride > 1 && j < nsamp; j += stride) {
+            Cell c;
+            cell_at(j, c);
+            if (low_block(a, c, brick_of(a.vol, c), need) >= 0) continue;
+            const float v = value(c);
+            evald++;
+            if (v > acc) {
+                acc = v;
+                need = in_codes(v);
             }
-            k++;
-            break;
         }
-        prev_v = v;
-        prev_t = t;
     }
-    if (!found && nsamp > 0) {
+    bool active = nsamp > 0;
+    while (__any_sync(kFull, active)) {
+        Cell c0, c1;
+        if (active) cell_at(k, c0);
+        if (FN != kFnSum && a.p.skip) {
+            const int s = active ? low_block(a, c0, brick_of(a.vol, c0), need) : 4;
+            if (!__any_sync(kFull, s < 0)) {
+                if (active) {
+                    k = jump_block(R, a.vol, c0, k, s);
+                    active = k < nsamp;
+                }
+                continue;
+            }
+        }
+        if (!active) continue;
+        // two samples per turn; a second one past the end is clamped into the
+        // volume and ignored
+        cell_at(k + 1, c1);
+        const float v0 = value(c0), v1 = value(c1);
+        const bool two = k + 1 < nsamp;
+        if (FN == kFnMip) {
+            acc = fmaxf(acc, v0);
+            if (two) acc = fmaxf(acc, v1);
+            need = in_codes(acc);
+        } else if (FN == kFnSum) {
+            acc += v0;
+            if (two) acc += v1;
+        } else if (v0 >= a.p.iso || (two && v1 >= a.p.iso)) {
+            if (!(v0 >= a.p.iso)) {
+                k++;
+                evald++;
+            }
+            evald++;
+            hit_k = k++;
+            active = false;
+            continue;
+        }
+        k += 2;
+        evald += two ? 2 : 1;
+        active = k < nsamp;
+    }
+    if (FN == kFnFirst && hit_k >= 0) {
+        // the hit's value again, and for an isosurface the value before it
+        const float t = sample_t(R, hit_k);
+        Cell c;
+        cell_at(hit_k, c);
+        const float v = value(c);
+        if (func == RC_FUNC_THRESHOLD) {
+            float4 e = classify(s_tf, a.tf.K, tf_coord<ST>(v, a.tf.ucoef), nullptr, nullptr, RC_DBG_ERR(a.vol));
+            out = make_float4(e.x, e.y, e.z, 1.0f);
+        } else {
+            float ts = t;
+            if (hit_k > 0) {
+                const float prev_t = sample_t(R, hit_k - 1);
+                Cell cp;
+                cell_at(hit_k - 1, cp);
+                const float prev_v = value(cp);
+                ts = prev_t + (t - prev_t) * ((a.p.iso - prev_v) / (v - prev_v));
+            }
+            float g[3], sf, spec;
+            if (CUBIC) bspline_grad<ST>(a.vol, c, g);
+            else value_grad<ST>(a.vol, c, g);
+            shade_factor(a.p, a.vol, g, R.dir, sf, spec);
+            out = make_float4(ts, fminf(1.0f, sf + spec), (float)hit_k, 1.0f);
+        }
+    }
+    k = min(k, nsamp);
+    if (FN != kFnFirst && nsamp > 0) {
         // over full scale; FP16 values h = (code - o) / o are shifted by 1 first
         // (code / vmax = (h + 1) / vscale)
-        float m = 0.0f;
-        bool have = true;
+        float m;
         if (ST == RC_STORE_F16) {
-            if (func == RC_FUNC_MIP) m = (acc + 1.0f) / a.vol.vscale;
+            if (FN == kFnMip) m = (acc + 1.0f) / a.vol.vscale;
             else if (func == RC_FUNC_AVERAGE) m = (acc / (float)nsamp + 1.0f) / a.vol.vscale;
-            else if (func == RC_FUNC_XRAY) m = (acc + (float)nsamp) * R.ds / a.vol.vscale;
-            else have = false;
+            else m = (acc + (float)nsamp) * R.ds / a.vol.vscale;
         } else {
-            if (func == RC_FUNC_MIP) m = acc / a.vol.vscale;
+            if (FN == kFnMip) m = acc / a.vol.vscale;
             else if (func == RC_FUNC_AVERAGE) m = acc / (float)nsamp / a.vol.vscale;
-            else if (func == RC_FUNC_XRAY) m = acc * R.ds / a.vol.vscale;
-            else have = false;
+            else m = acc * R.ds / a.vol.vscale;
         }
-        if (have) out = make_float4(m, m, m, 1.0f);
+        out = make_float4(m, m, m, 1.0f);
     }
     if (inimg) outp[(size_t)y * cam.W + x] = out;
-    if (a.stats) add_stats(a.stats, (unsigned)k, (unsigned)k, hit ? 1u : 0u, inimg ? 1u : 0u);
+    // a sample that MIP took in its first pass too counts once
+    if (a.stats) add_stats(a.stats, (unsigned)k, min(evald, (unsigned)k), hit ? 1u : 0u, inimg ? 1u : 0u);
 }
 
 template <typename K>
@@ -210,13 +304,23 @@ static cudaError_t launch_composite(const MarchArgs &a, int nviews, cudaStream_t
     }
 }
 
-template <bool CUBIC>
-static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t s) {
+template <bool CUBIC, int FN>
+static cudaError_t launch_function_group(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = a.p.func == RC_FUNC_THRESHOLD;
     switch (a.vol.storage) {
-        case RC_STORE_F32: return launch_kernel(function_kernel<RC_STORE_F32, CUBIC>, a, nviews, smem, s);
-        case RC_STORE_F16: return launch_kernel(function_kernel<RC_STORE_F16, CUBIC>, a, nviews, smem, s);
-        default: return launch_kernel(function_kernel<RC_STORE_U16, CUBIC>, a, nviews, smem, s);
+        case RC_STORE_F32: return launch_kernel(function_kernel<RC_STORE_F32, CUBIC, FN>, a, nviews, smem, s);
+        case RC_STORE_F16: return launch_kernel(function_kernel<RC_STORE_F16, CUBIC, FN>, a, nviews, smem, s);
+        default: return launch_kernel(function_kernel<RC_STORE_U16, CUBIC, FN>, a, nviews, smem, s);
+    }
+}
+
+template <bool CUBIC>
+static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t s) {
+    switch (a.p.func) {
+        case RC_FUNC_MIP: return launch_function_group<CUBIC, kFnMip>(a, nviews, s);
+        case RC_FUNC_AVERAGE:
+        case RC_FUNC_XRAY: return launch_function_group<CUBIC, kFnSum>(a, nviews, s);
+        default: return launch_function_group<CUBIC, kFnFirst>(a, nviews, s);
     }
 }
 
