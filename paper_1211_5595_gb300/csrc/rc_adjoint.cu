@@ -210,9 +210,8 @@ __global__ void __launch_bounds__(TF2 ? 32 * kWarps2D : 32 * kAdjWarps) adjoint_
             position_at(R, sample_t(R, k), p);
             Cell c;
             cell_of(a.vol, p, c);
-            const int b = brick_of(a.vol, c);
-            const int s = a.fine ? empty_block(__ldg(a.fine + b), c) : (__ldg(a.occ + b) ? -1 : 4);
-            if (s >= 0) {
+            const int s = empty_level(a, a.lvl, c);
+            if (s) {
                 k = jump_block(R, a.vol, c, k, s);
                 continue;
             }

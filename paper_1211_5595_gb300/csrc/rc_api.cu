@@ -97,9 +97,9 @@ struct rc_volume {
     // min/max grid and occupancy mask per reconstruction filter (index rc_filter)
     uint16_t *d_mn[2] = {nullptr, nullptr}, *d_mx[2] = {nullptr, nullptr};
     uint8_t *d_occ[2] = {nullptr, nullptr};
-    // 4^3 sub-block min/max grid and the fine mask of the trilinear compositing march
+    // 4^3 sub-block min/max grid and the empty levels of the compositing march
     uint16_t *d_mn4[2] = {nullptr, nullptr}, *d_mx4[2] = {nullptr, nullptr};
-    unsigned long long *d_fine[2] = {nullptr, nullptr};
+    uint8_t *d_lvl[2] = {nullptr, nullptr};
     bool uploaded = false;
     uint64_t data_version = 0;
     uint64_t grid_data_version[2] = {~0ull, ~0ull};
@@ -310,7 +310,7 @@ static void volume_free(rc_volume *v) {
     for (int f = 0; f < 2; f++) {
         cudaFree(v->d_mn4[f]);
         cudaFree(v->d_mx4[f]);
-        cudaFree(v->d_fine[f]);
+        cudaFree(v->d_lvl[f]);
     }
 }
 
@@ -362,10 +362,10 @@ rc_status rc_volume_create(rc_context *ctx, int nx, int ny, int nz, float sx, fl
         dev_alloc(&v->d_occ[1], v->nbricks) != cudaSuccess ||
         dev_alloc(&v->d_mn4[0], n4 * sizeof(uint16_t)) != cudaSuccess ||
         dev_alloc(&v->d_mx4[0], n4 * sizeof(uint16_t)) != cudaSuccess ||
-        dev_alloc(&v->d_fine[0], v->nbricks * sizeof(unsigned long long)) != cudaSuccess ||
+        dev_alloc(&v->d_lvl[0], n4) != cudaSuccess ||
         dev_alloc(&v->d_mn4[1], n4 * sizeof(uint16_t)) != cudaSuccess ||
         dev_alloc(&v->d_mx4[1], n4 * sizeof(uint16_t)) != cudaSuccess ||
-        dev_alloc(&v->d_fine[1], v->nbricks * sizeof(unsigned long long)) != cudaSuccess) {
+        dev_alloc(&v->d_lvl[1], n4) != cudaSuccess) {
         cudaGetLastError();
         volume_free(v);
         delete v;
@@ -868,8 +868,7 @@ static rc_status ensure_occupancy(rc_context *ctx, rc_volume *v, int f) {
     TFDev tf = tf_dev(ctx, v);
     const int f16o = v->storage == RC_STORE_F16 ? f16_offset(v->vmax) : 0;
     RC_CUDA(ctx, launch_occupancy(v->d_mn[f], v->d_mx[f], v->nbricks, v->vmax, f16o, tf, v->d_occ[f], ctx->stream));
-    RC_CUDA(ctx, launch_finemask(v->d_mn4[f], v->d_mx4[f], v->n, v->cb, v->vmax, f16o, tf, v->d_fine[f],
-                                 ctx->stream));
+    RC_CUDA(ctx, launch_levels(v->d_mn4[f], v->d_mx4[f], v->n, v->cb, f16o, tf, v->d_lvl[f], ctx->stream));
     v->occ_tf_version[f] = ctx->tf_version;
     v->occ_data_version[f] = v->data_version;
     return RC_OK;
@@ -948,10 +947,10 @@ static MarchArgs march_args(rc_context *ctx, const rc_volume *v, const rc_render
     a.p.rmode = a.p.ratio == 1.0f ? 0 : a.p.ratio == 0.5f ? 1 : a.p.ratio == 0.25f ? 2 : 3;
     a.p.filter = p->filter;
     a.occ = v->d_occ[p->filter];
-    a.fine = v->d_fine[p->filter];
+    a.lvl = v->d_lvl[p->filter];
     a.mx = v->d_mx[p->filter];
     a.mx4 = v->d_mx4[p->filter];
-    for (int i = 0; i < 2; i++) a.c4[i] = (v->n[i] - 1 + 3) / 4;
+    for (int i = 0; i < 3; i++) a.c4[i] = (v->n[i] - 1 + 3) / 4;
     // FP32 reconstruction rounds by less than 2^-18 of full scale; FP16 codes
     // beyond 12 bits are stored to within 2^-12 of the offset
     a.slack = (float)v->vmax * (1.0f / 65536.0f) +
@@ -1156,8 +1155,7 @@ rc_status rc_render_batch(rc_context *ctx, const rc_volume *const *vols, int nvo
     BatchVol *recs = new (std::nothrow) BatchVol[nvols];
     if (!recs) return fail(ctx, RC_ERR_OOM, "%s: host allocation", who);
     for (int i = 0; i < nvols; i++)
-        recs[i] = BatchVol{vols[i]->d_data, vols[i]->d_vg, vol_dev(vols[i]).pairs, vols[i]->d_occ[p->filter],
-                           vols[i]->d_fine[p->filter]};
+        recs[i] = BatchVol{vols[i]->d_data, vols[i]->d_vg, vol_dev(vols[i]).pairs, vols[i]->d_lvl[p->filter]};
     cudaError_t ce = cudaMemcpyAsync(ctx->d_batch, recs, (size_t)nvols * sizeof(BatchVol), cudaMemcpyHostToDevice,
                                      ctx->stream);
     delete[] recs;

@@ -756,6 +756,25 @@ __device__ __forceinline__ void composite_add(const float4 &e, float &C0, float 
     T = T * (1.0f - e.w);
 }
 
+// About the distance at which the ray leaves the block of 2^s cells per axis
+// around cell c; false when the block reaches the volume's far sides. An
+// estimate: the jumps verify the sample they land on, so the divisions need
+// not round exactly.
+__device__ __forceinline__ bool block_exit(const Ray &R, const VolDev &v, const Cell &c, int s, float &texit) {
+    texit = __int_as_float(0x7f800000);
+    bool leaves = false;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const int lo = (c.i[a] >> s) << s, hi = lo + (1 << s);
+        const bool up = R.d[a] > 0.0f;
+        if (up ? hi <= v.n[a] - 2 : (R.d[a] < 0.0f && lo > 0)) {
+            texit = fminf(texit, __fdividef((float)(up ? hi : lo) - R.o[a], R.d[a]));
+            leaves = true;
+        }
+    }
+    return leaves;
+}
+
 // Jump over an empty axis-aligned block of 2^s cells per axis containing
 // cell c (s = 4: the cell-brick; 3 and 2: its octants and 4^3 sub-blocks).
 // Returns the index of the first sample that may lie outside the block: the
@@ -765,18 +784,9 @@ __device__ __forceinline__ void composite_add(const float4 &e, float &C0, float 
 // k and m is then inside too. Falls back to k + 1 when the check fails, so
 // the exit estimate needs no exact rounding.
 __device__ __forceinline__ int jump_block(const Ray &R, const VolDev &v, const Cell &c, int k, int s) {
-    const float INF = __int_as_float(0x7f800000);
-    float texit = INF;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const int lo = (c.i[a] >> s) << s, hi = lo + (1 << s);
-        if (R.d[a] > 0.0f && hi <= v.n[a] - 2)
-            texit = fminf(texit, __fdiv_rn((float)hi - R.o[a], R.d[a]));
-        else if (R.d[a] < 0.0f && lo > 0)
-            texit = fminf(texit, __fdiv_rn((float)lo - R.o[a], R.d[a]));
-    }
-    if (texit == INF) return R.nsamp;
-    float fm = floorf(__fdiv_rn(texit - R.tn, R.ds));
+    float texit;
+    if (!block_exit(R, v, c, s, texit)) return R.nsamp;
+    const float fm = floorf(__fdividef(texit - R.tn, R.ds));
     int m = fm >= (float)R.nsamp ? R.nsamp - 1 : (int)fm;
     if (m <= k) return k + 1;
 #pragma unroll 1
@@ -791,20 +801,18 @@ __device__ __forceinline__ int jump_block(const Ray &R, const VolDev &v, const C
     return k + 1;
 }
 
-// The empty block around cell c by the fine mask of its cell-brick (one bit
-// per 4^3 sub-block, bit sz*16 + sy*4 + sx): 4 when the whole brick is empty,
-// 3 when its octant is, 2 when the sub-block is, -1 when the sample may have
-// non-zero opacity.
-// The sub-block's own bit is tested first: most evaluated samples lie in an
-// occupied sub-block and need nothing else.
-__device__ __forceinline__ int empty_block(unsigned long long m, const Cell &c) {
-    const int bit = ((c.i[0] >> 2) & 3) | (c.i[1] & 12) | ((c.i[2] & 12) << 2);   // sz*16 + sy*4 + sx
-    const unsigned half = (bit & 32) ? (unsigned)(m >> 32) : (unsigned)m;
-    if ((half >> (bit & 31)) & 1u) return -1;
-    if (m == 0ull) return 4;
-    const int oct = bit & 0x2A;                                          // bit of the octant's first sub-block
-    if (((m >> oct) & 0x330033ull) == 0ull) return 3;                   // sub-blocks {0,1} x {0,1} x {0,1} of it
-    return 2;
+// The empty block around cell c: 4 when its whole cell-brick holds no visible
+// sub-block, 3 when its 8^3 octant does not, 2 when its 4^3 sub-block is
+// empty, 0 when the sample may have non-zero opacity. One byte per sub-block,
+// x fastest, so a sample costs three shifts, two multiply-adds, the load and
+// the test. (A 64-bit mask per cell-brick needs the brick index first and then
+// the bit's position, half and shift: RC_LVL_MS.)
+__device__ __forceinline__ int empty_level(const MarchArgs &a, const uint8_t *lvl, const Cell &c) {
+    int j = ((c.i[2] >> 2) * a.c4[1] + (c.i[1] >> 2)) * a.c4[0] + (c.i[0] >> 2);
+#ifdef RC_DEBUG
+    j = dbg_index(j, a.c4[0] * a.c4[1] * a.c4[2], a.vol.dbg_err, kSiteBrick);
+#endif
+    return __ldg(lvl + j);
 }
 
 }  // namespace rc

@@ -95,8 +95,7 @@ struct BatchVol {
     const void *data;
     const void *vg;
     const void *pairs;
-    const uint8_t *occ;
-    const unsigned long long *fine;
+    const uint8_t *lvl;
 };
 
 struct MarchArgs {
@@ -105,12 +104,12 @@ struct MarchArgs {
     TFDev tf;
     MarchParams p;
     const uint8_t *occ;            // cell-brick occupancy (1 = may be non-empty)
-    const unsigned long long *fine;   // compositing: per cell-brick, one bit per 4^3 sub-block (or null)
+    const uint8_t *lvl;            // compositing: empty level of each 4^3 sub-block (see empty_level)
     // ray functions that skip by block maxima: largest code of each cell-brick
-    // and of each 4^3 sub-block (c4[0] x c4[1] x ceil((n-1)/4) of them), and
+    // and of each 4^3 sub-block (c4[0] x c4[1] x c4[2] of them, x fastest), and
     // the margin in code units by which a value may exceed its block's maximum
     const uint16_t *mx, *mx4;
-    int c4[2];
+    int c4[3];
     float slack;
     float4 *out;                   // H x W RGBA (view-major for several views)
     unsigned long long *stats;     // dense, evaluated, hit, total (or null)
@@ -222,12 +221,12 @@ cudaError_t launch_minmax(const uint16_t *stage, const int n[3], const int cb[3]
 cudaError_t launch_occupancy(const uint16_t *mn, const uint16_t *mx, int nbricks, int vmax,
                              int f16o, TFDev tf, uint8_t *occ, cudaStream_t s);
 // 4^3 sub-block min/max grid of a filter (cells 4j..4j+3; footprint voxels
-// 4j..4j+4, or 4j-1..4j+5 for the B-spline, clamped) and the fine mask built
-// from it: per cell-brick one bit per sub-block.
+// 4j..4j+4, or 4j-1..4j+5 for the B-spline, clamped) and the empty
+// levels built from it: one byte per sub-block.
 cudaError_t launch_minmax4(const uint16_t *stage, const int n[3], int vmax, int filter, uint16_t *mn, uint16_t *mx,
                            cudaStream_t s);
-cudaError_t launch_finemask(const uint16_t *mn4, const uint16_t *mx4, const int n[3], const int cb[3], int vmax,
-                            int f16o, TFDev tf, unsigned long long *fine, cudaStream_t s);
+cudaError_t launch_levels(const uint16_t *mn4, const uint16_t *mx4, const int n[3], const int cb[3], int f16o,
+                          TFDev tf, uint8_t *lvl, cudaStream_t s);
 cudaError_t launch_march(const MarchArgs &a, int nviews, cudaStream_t s);
 cudaError_t launch_march_cubic(const MarchArgs &a, int nviews, cudaStream_t s);   // filter = B-spline
 cudaError_t launch_march_tf2(const MarchArgs &a, int nviews, cudaStream_t s);     // trilinear, 2-D table

@@ -49,8 +49,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     }
     // a batch of volumes: the volume's own data and masks, the shared record
     VolDev vol = a.vol;
-    const uint8_t *occ = a.occ;
-    const unsigned long long *fine = a.fine;
+    const uint8_t *lvl = a.lvl;
     int view = blockIdx.z;
     if (a.batch) {
         const int vi = blockIdx.z / a.views;
@@ -59,8 +58,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
         vol.data = bv.data;
         vol.vg = bv.vg;
         vol.pairs = bv.pairs;
-        occ = bv.occ;
-        fine = bv.fine;
+        lvl = bv.lvl;
     }
     const CamRec cam = a.cams ? a.cams[view] : a.cam;
     float4 *out = a.out + (size_t)blockIdx.z * cam.W * cam.H;
@@ -81,11 +79,10 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
         Cell c;
         cell_of(vol, p, c);
         if (a.p.skip) {
-            // the largest empty block around the sample: with the fine mask
-            // the cell-brick, its octant or its 4^3 sub-block; else the brick
-            const int b = brick_of(vol, c);
-            const int s = fine ? empty_block(__ldg(fine + b), c) : (__ldg(occ + b) ? -1 : 4);
-            if (s >= 0) {
+            // the largest empty block around the sample: the cell-brick, its
+            // octant or its 4^3 sub-block
+            const int s = empty_level(a, lvl, c);
+            if (s) {
                 k = jump_block(R, vol, c, k, s);
                 active = k < nsamp;
                 continue;

@@ -67,14 +67,13 @@ __global__ void __launch_bounds__(kMarchThreads) staged_kernel(const MarchArgs a
             float p[3];
             position_at(R, sample_t(R, k), p);
             cell_of(vol, p, c);
-            const int b = brick_of(vol, c);
-            const int s = a.fine ? empty_block(__ldg(a.fine + b), c) : (__ldg(a.occ + b) ? -1 : 4);
-            if (s >= 0) {
+            const int s = empty_level(a, a.lvl, c);
+            if (s) {
                 k = jump_block(R, vol, c, k, s);
                 active = k < nsamp;
                 continue;
             }
-            mine = (unsigned)b;
+            mine = (unsigned)brick_of(vol, c);
             break;
         }
         // the CTA's next brick: the smallest any ray needs
@@ -125,7 +124,7 @@ __global__ void __launch_bounds__(kMarchThreads) staged_kernel(const MarchArgs a
                 cell_of(vol, p, c);
                 const int b = brick_of(vol, c);
                 if ((unsigned)b != bmin) break;
-                if ((a.fine ? empty_block(__ldg(a.fine + b), c) : (__ldg(a.occ + b) ? -1 : 4)) >= 0) break;
+                if (empty_level(a, a.lvl, c)) break;
             }
         }
         __syncthreads();      // the brick and s_min are read before the next stage replaces them

@@ -54,10 +54,7 @@ __global__ void __launch_bounds__(128) profiles_kernel(const MarchArgs a, float 
             position_at(R, __fmaf_rn((float)k + 0.5f, delta, R.tn), p);
             Cell c;
             cell_of(a.vol, p, c);
-            if (a.p.skip) {                                                   // opacity exactly 0
-            const int b = brick_of(a.vol, c);
-            if (a.fine ? empty_block(__ldg(a.fine + b), c) >= 0 : !__ldg(a.occ + b)) continue;
-        }
+            if (a.p.skip && empty_level(a, a.lvl, c)) continue;               // opacity exactly 0
             float4 e = eval_sample<ST, false>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio);
             acc = __fmaf_rn(T, e.w, acc);
             T = T * (1.0f - e.w);
@@ -488,9 +485,8 @@ __device__ __forceinline__ void plain_ray(const MarchArgs &a, const float4 *s_tf
         Cell c;
         cell_of(a.vol, p, c);
         if (a.p.skip) {
-            const int b = brick_of(a.vol, c);
-            const int s = a.fine ? empty_block(__ldg(a.fine + b), c) : (__ldg(a.occ + b) ? -1 : 4);
-            if (s >= 0) {
+            const int s = empty_level(a, a.lvl, c);
+            if (s) {
                 k = jump_block(R, a.vol, c, k, s);
                 continue;
             }
@@ -562,18 +558,9 @@ __device__ __forceinline__ void range_of(const MarchArgs &a, const Ray &R, const
 // Falls back to j + 1 when the check fails.
 __device__ __forceinline__ int jump_block_grid(const Ray &R, const VolDev &v, const Cell &c, int j, int s, float ta,
                                                float seg, int n) {
-    const float INF = __int_as_float(0x7f800000);
-    float texit = INF;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const int lo = (c.i[a] >> s) << s, hi = lo + (1 << s);
-        if (R.d[a] > 0.0f && hi <= v.n[a] - 2)
-            texit = fminf(texit, __fdiv_rn((float)hi - R.o[a], R.d[a]));
-        else if (R.d[a] < 0.0f && lo > 0)
-            texit = fminf(texit, __fdiv_rn((float)lo - R.o[a], R.d[a]));
-    }
-    if (texit == INF) return n;
-    const float fm = floorf(__fsub_rn(__fdiv_rn(texit - ta, seg), 0.5f));
+    float texit;
+    if (!block_exit(R, v, c, s, texit)) return n;
+    const float fm = floorf(__fsub_rn(__fdividef(texit - ta, seg), 0.5f));
     int m = fm >= (float)n ? n - 1 : (int)fm;
     if (m <= j) return j + 1;
 #pragma unroll 1
@@ -609,9 +596,8 @@ __device__ __forceinline__ void march_range(const ImportanceArgs &A, const float
         Cell c;
         cell_of(a.vol, p, c);
         if (a.p.skip) {          // opacity exactly 0: past the largest empty block around the sample
-            const int b = brick_of(a.vol, c);
-            const int s = a.fine ? empty_block(__ldg(a.fine + b), c) : (__ldg(a.occ + b) ? -1 : 4);
-            if (s >= 0) {
+            const int s = empty_level(a, a.lvl, c);
+            if (s) {
                 j = JUMP ? jump_block_grid(R, a.vol, c, j, s, ta, seg, A.nimp) : j + 1;
                 continue;
             }
@@ -669,12 +655,7 @@ __device__ __forceinline__ void march_invcdf(const ImportanceArgs &A, const floa
         position_at(R, tj, p);
         Cell c;
         cell_of(a.vol, p, c);
-        bool empty = false;
-        if (a.p.skip) {                                                   // opacity exactly 0
-            const int bb = brick_of(a.vol, c);
-            empty = a.fine ? empty_block(__ldg(a.fine + bb), c) >= 0 : !__ldg(a.occ + bb);
-        }
-        if (!empty) {
+        if (!(a.p.skip && empty_level(a, a.lvl, c))) {                    // empty: opacity exactly 0
             const float ratio = __fdiv_rn(len, a.vol.smin);
             float4 e = eval_sample<ST, SHADE>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio);
             composite_add(e, C0, C1, C2, T);

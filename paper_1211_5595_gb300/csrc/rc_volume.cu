@@ -305,35 +305,44 @@ __device__ __forceinline__ bool range_visible(float vmn, float vmx, int f16o, co
     return false;
 }
 
-// One thread per sub-block, 64 per cell-brick: bit t = sz*16 + sy*4 + sx of
-// the brick's mask is set when sub-block (4*bx + sx, 4*by + sy, 4*bz + sz)
-// exists and may hold non-zero opacity; each warp's ballot is one 32-bit half.
-__global__ void __launch_bounds__(128) finemask_kernel(const uint16_t *mn4, const uint16_t *mx4, int c0, int c1,
-                                                       int c2, int cb0, int cb1, int nbricks, int f16o,
-                                                       TFDev tf, uint32_t *fine) {
+// One thread per sub-block, 64 per cell-brick (two cell-bricks per block):
+// sub-block t = sz*16 + sy*4 + sx of brick b is (4*bx + sx, 4*by + sy,
+// 4*bz + sz). The ballots of a brick's two warps form its 64-bit visibility
+// mask, from which each thread writes its sub-block's empty level: 0 visible,
+// 2 empty, 3 the octant (sub-blocks {0,1} x {0,1} x {0,1} of it) empty,
+// 4 the whole brick empty.
+__global__ void __launch_bounds__(128) levels_kernel(const uint16_t *mn4, const uint16_t *mx4, int c0, int c1, int c2,
+                                                     int cb0, int cb1, int nbricks, int f16o, TFDev tf, uint8_t *lvl) {
+    __shared__ uint32_t s_bits[4];
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int b = (int)(e >> 6), t = (int)(e & 63);
-    bool vis = false;
+    bool exists = false, vis = false;
+    int j = 0;
     if (b < nbricks) {
         const int bx = b % cb0, by = (b / cb0) % cb1, bz = b / (cb0 * cb1);
         const int jx = 4 * bx + (t & 3), jy = 4 * by + ((t >> 2) & 3), jz = 4 * bz + (t >> 4);
-        if (jx < c0 && jy < c1 && jz < c2) {
-            const int j = (jz * c1 + jy) * c0 + jx;
+        exists = jx < c0 && jy < c1 && jz < c2;
+        if (exists) {
+            j = (jz * c1 + jy) * c0 + jx;
             vis = range_visible((float)mn4[j], (float)mx4[j], f16o, tf);
         }
     }
     const unsigned bits = __ballot_sync(0xffffffffu, vis);
-    if ((threadIdx.x & 31) == 0 && b < nbricks) fine[2 * b + (t >> 5)] = bits;
+    if ((threadIdx.x & 31) == 0) s_bits[threadIdx.x >> 5] = bits;
+    __syncthreads();
+    if (!exists) return;
+    const int w = (threadIdx.x >> 6) * 2;
+    const unsigned long long m = (unsigned long long)s_bits[w] | ((unsigned long long)s_bits[w + 1] << 32);
+    lvl[j] = vis ? 0 : m == 0ull ? 4 : ((m >> (t & 0x2A)) & 0x330033ull) == 0ull ? 3 : 2;
 }
 
-cudaError_t launch_finemask(const uint16_t *mn4, const uint16_t *mx4, const int n[3], const int cb[3], int vmax,
-                            int f16o, TFDev tf, unsigned long long *fine, cudaStream_t s) {
+cudaError_t launch_levels(const uint16_t *mn4, const uint16_t *mx4, const int n[3], const int cb[3], int f16o,
+                          TFDev tf, uint8_t *lvl, cudaStream_t s) {
     const int c0 = (n[0] - 1 + 3) / 4, c1 = (n[1] - 1 + 3) / 4, c2 = (n[2] - 1 + 3) / 4;
     const int nb = cb[0] * cb[1] * cb[2];
     const long long threads = (long long)nb * 64;
-    (void)vmax;
-    finemask_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(mn4, mx4, c0, c1, c2, cb[0], cb[1], nb, f16o,
-                                                                      tf, reinterpret_cast<uint32_t *>(fine));
+    levels_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(mn4, mx4, c0, c1, c2, cb[0], cb[1], nb, f16o, tf,
+                                                                    lvl);
     return cudaGetLastError();
 }
 
