@@ -6,6 +6,8 @@
 // (rc_march.cu, rc_march_cubic.cu, rc_march_tf2.cu) so they compile in parallel.
 #pragma once
 
+#include <math.h>
+
 #include "rc_device.cuh"
 
 namespace rc {
@@ -40,8 +42,24 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, unsigned de
 // Compositing ray function (Sec. 4.2, Eq. 4): C += T a' c, T *= (1 - a'),
 // front to back from the eye; stop after the sample where 1 - T >= term.
 // F selects the sample form (kShade, kCubic, kTF2).
+//
+// Instruction issue and the L1 data path bound it, with the latency of one
+// sample's chain (level, voxels, table) behind both. One turn of the loop is
+// - two samples for the plain trilinear form, whose 8 loads leave registers
+//   for a second sample in flight (4 FP16 views of 181x217x157 at 901x703:
+//   0.342 -> 0.327 ms; with shading the registers cost more warps than the
+//   overlap gains: 2.63 -> 2.78 ms for 12 views of 256x256x180 at 1024^2);
+// - one sample with the next one's cell and level fetched under it for the
+//   shaded FP32 form (2.635 -> 2.612 ms; uint16 1.373 -> 1.422, B-spline
+//   1.725 -> 1.762);
+// - one sample at a time else.
+// Lanes leave the loop one by one: holding the warp together by a vote per
+// turn took uint16 at 512x512x256, 2048^2, from 1.37 to 1.45 ms.
+enum : int { kTurnOne = 0, kTurnPair = 1, kTurnAhead = 2 };
+
 template <int ST, int F, int RM>
 __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArgs a) {
+    constexpr int kTurn = F == 0 ? kTurnPair : F == kShade && ST == RC_STORE_F32 ? kTurnAhead : kTurnOne;
     extern __shared__ float4 s_tf[];
     if (!(F & kTF2)) {
         load_tf(a.tf, s_tf);
@@ -72,30 +90,157 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     int k = 0;
     unsigned evald = 0;
     bool active = nsamp > 0;
-    while (__any_sync(kFull, active)) {
-        if (!active) continue;
+    auto cell_at = [&](int i, Cell &c) {
         float p[3];
-        position_at(R, sample_t(R, k), p);
-        Cell c;
+        position_at(R, sample_t(R, i), p);
         cell_of(vol, p, c);
-        if (a.p.skip) {
-            // the largest empty block around the sample: the cell-brick, its
-            // octant or its 4^3 sub-block
-            const int s = empty_level(a, lvl, c);
-            if (s) {
-                k = jump_block(R, vol, c, k, s);
-                active = k < nsamp;
-                continue;
-            }
-        }
-        float4 e = eval_sample_x<ST, F, RM>(vol, a.p, s_tf, a.tf, R.dir, c, a.p.rmode, a.p.ratio);
+    };
+    auto level = [&](const Cell &c) { return a.p.skip ? empty_level(a, lvl, c) : 0; };
+    auto sample = [&](const Cell &c) {
+        return eval_sample_x<ST, F, RM>(vol, a.p, s_tf, a.tf, R.dir, c, a.p.rmode, a.p.ratio);
+    };
+    auto add = [&](const float4 &e) {
         composite_add(e, C0, C1, C2, T);
         evald++;
         k++;
         active = k < nsamp && (1.0f - T) < a.p.term;
+    };
+    // past the largest empty block around the sample: its cell-brick, octant
+    // or 4^3 sub-block
+    auto jump = [&](const Cell &c, int s) {
+        k = jump_block(R, vol, c, k, s);
+        active = k < nsamp;
+    };
+    if constexpr (kTurn == kTurnPair) {
+        while (active) {
+            Cell c, cn;
+            cell_at(k, c);
+            cell_at(k + 1, cn);                 // past the end: clamped into the volume, not used
+            const int s = level(c), sn = level(cn);
+            if (s) {
+                jump(c, s);
+                continue;
+            }
+            const float4 e = sample(c), en = sample(cn);
+            add(e);
+            if (active && !sn) add(en);
+        }
+    } else if constexpr (kTurn == kTurnAhead) {
+        Cell c;
+        int s = 0;
+        if (active) {
+            cell_at(0, c);
+            s = level(c);
+        }
+        while (active) {
+            if (s) {
+                jump(c, s);
+                cell_at(k, c);
+                s = level(c);
+                continue;
+            }
+            Cell cn;
+            cell_at(k + 1, cn);
+            s = level(cn);
+            add(sample(c));
+            c = cn;
+        }
+    } else {
+        while (active) {
+            Cell c;
+            cell_at(k, c);
+            const int s = level(c);
+            if (s) jump(c, s);
+            else add(sample(c));
+        }
     }
+    __syncwarp();
     if (inimg) out[(size_t)y * cam.W + x] = make_float4(C0, C1, C2, 1.0f - T);
     if (a.stats) add_stats(a.stats, (unsigned)min(k, nsamp), evald, hit ? 1u : 0u, inimg ? 1u : 0u);
+}
+
+// The compositing march with L lanes per ray, for launches too small to fill
+// the GPU with one: lane j of a ray's group evaluates sample k + j, then every
+// lane of the group composites the L samples in order from shuffles, so the
+// image is composite_kernel's bit for bit and a ray's chain of dependent
+// sample latencies is L times shorter. Samples past a termination are
+// evaluated in vain and the shuffles cost issue slots: lanes_per_ray says
+// where that pays.
+template <int L> struct WideTile;
+template <> struct WideTile<2> { static constexpr int X = 4, Y = 4; };
+template <> struct WideTile<4> { static constexpr int X = 4, Y = 2; };
+template <> struct WideTile<8> { static constexpr int X = 2, Y = 2; };
+
+template <int ST, int F, int L>
+__global__ void __launch_bounds__(kMarchThreads) wide_kernel(const MarchArgs a) {
+    extern __shared__ float4 s_tf[];
+    if (!(F & kTF2)) {
+        load_tf(a.tf, s_tf);
+        __syncthreads();
+    }
+    VolDev vol = a.vol;
+    const uint8_t *lvl = a.lvl;
+    int view = blockIdx.z;
+    if (a.batch) {
+        const int vi = blockIdx.z / a.views;
+        view = blockIdx.z - vi * a.views;
+        const BatchVol bv = a.batch[vi];
+        vol.data = bv.data;
+        vol.vg = bv.vg;
+        vol.pairs = bv.pairs;
+        lvl = bv.lvl;
+    }
+    const CamRec cam = a.cams ? a.cams[view] : a.cam;
+    float4 *out = a.out + (size_t)blockIdx.z * cam.W * cam.H;
+    constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane % L, ray = lane / L, first = lane - j;
+    const int x = blockIdx.x * (kWarpsX * TX) + (warp % kWarpsX) * TX + ray % TX;
+    const int y = blockIdx.y * (kWarpsY * TY) + (warp / kWarpsX) * TY + ray / TX;
+    const bool inimg = x < cam.W && y < cam.H;
+    Ray R;
+    const bool hit = inimg && setup_ray(cam, vol, a.p.step_vox, x, y, R);
+    const int nsamp = hit ? R.nsamp : 0;
+    float C0 = 0.0f, C1 = 0.0f, C2 = 0.0f, T = 1.0f;
+    int k = 0;
+    unsigned evald = 0;
+    bool active = nsamp > 0;
+    while (__any_sync(kFull, active)) {
+        // every lane of a group has the same k, active, C and T
+        const bool turn = active, in = turn && k + j < nsamp;
+        Cell c;
+        int s = 0;
+        if (in) {
+            float p[3];
+            position_at(R, sample_t(R, k + j), p);
+            cell_of(vol, p, c);
+            if (a.p.skip) s = empty_level(a, lvl, c);
+        }
+        const unsigned vis = (__ballot_sync(kFull, in && s == 0) >> first) & ((1u << L) - 1u);
+        float4 e = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        int next = k + j + 1;
+        if (in && s == 0) e = eval_sample_x<ST, F>(vol, a.p, s_tf, a.tf, R.dir, c, a.p.rmode, a.p.ratio);
+        else if (in && vis == 0) next = jump_block(R, vol, c, k + j, s);
+        // all L samples empty: on from the last one's block
+        next = __shfl_sync(kFull, next, first + max(min(nsamp - 1 - k, L - 1), 0));
+#pragma unroll
+        for (int i = 0; i < L; i++) {
+            const float4 q = make_float4(__shfl_sync(kFull, e.x, first + i), __shfl_sync(kFull, e.y, first + i),
+                                         __shfl_sync(kFull, e.z, first + i), __shfl_sync(kFull, e.w, first + i));
+            if (active && ((vis >> i) & 1u)) {
+                composite_add(q, C0, C1, C2, T);
+                evald++;
+                active = (1.0f - T) < a.p.term;
+                if (!active) next = k + i + 1;
+            }
+        }
+        if (turn) k = next;
+        active = active && k < nsamp;
+    }
+    if (inimg && j == 0) out[(size_t)y * cam.W + x] = make_float4(C0, C1, C2, 1.0f - T);
+    if (a.stats) {
+        const bool one = j == 0;
+        add_stats(a.stats, one ? (unsigned)min(k, nsamp) : 0u, one ? evald : 0u, one && hit ? 1u : 0u, one && inimg ? 1u : 0u);
+    }
 }
 
 // Ray function groups: the functions of one group share a loop.
@@ -179,11 +324,19 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
             }
         }
     }
-    bool active = nsamp > 0;
-    while (__any_sync(kFull, active)) {
+    if (FN == kFnSum) {
+        for (; k < nsamp; k++) {
+            Cell c;
+            cell_at(k, c);
+            acc += value(c);
+        }
+        evald = (unsigned)nsamp;
+    }
+    bool active = FN != kFnSum && nsamp > 0;
+    while (FN != kFnSum && __any_sync(kFull, active)) {
         Cell c0, c1;
         if (active) cell_at(k, c0);
-        if (FN != kFnSum && a.p.skip) {
+        if (a.p.skip) {
             const int s = active ? low_block(a, c0, brick_of(a.vol, c0), need) : 4;
             if (!__any_sync(kFull, s < 0)) {
                 if (active) {
@@ -203,9 +356,6 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
             acc = fmaxf(acc, v0);
             if (two) acc = fmaxf(acc, v1);
             need = in_codes(acc);
-        } else if (FN == kFnSum) {
-            acc += v0;
-            if (two) acc += v1;
         } else if (v0 >= a.p.iso || (two && v1 >= a.p.iso)) {
             if (!(v0 >= a.p.iso)) {
                 k++;
@@ -267,15 +417,81 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
 }
 
 template <typename K>
-static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool table_in_smem, cudaStream_t s) {
+static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool table_in_smem, cudaStream_t s,
+                                 int tile_w = kTileW, int tile_h = kTileH) {
     size_t smem = table_in_smem ? (size_t)a.tf.K * sizeof(float4) : 0;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid((a.cam.W + kTileW - 1) / kTileW, (a.cam.H + kTileH - 1) / kTileH, nviews);
+    dim3 grid((a.cam.W + tile_w - 1) / tile_w, (a.cam.H + tile_h - 1) / tile_h, nviews);
     kern<<<grid, kMarchThreads, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+// Lanes per ray of a launch. A ray's samples are a serial chain (a few hundred
+// of them, 0.3 us each), so a launch with few rays takes the time of its
+// longest ray however few there are; more lanes shorten the chain until the
+// shuffles and the samples past termination fill the GPU. The lines lie where
+// the measured times cross, in rays that meet the volume (`hits`, 0.27 of the
+// pixels there) and per sample across the box (`steps`); us per view with
+// 1, 2, 4 and 8 lanes, FP32 shaded / FP32 plain:
+//   64x64x32, 256^2:    79 58 46 42 / 68 44 35 40
+//   128x128x96, 384^2: 118 107 74 88 / 102 65 66 73
+//   256x256x180, 256^2: 147 102 72 61 / 162 84 58 56
+//   256x256x180, 512^2: 172 142 135 161 / 135 105 99 131
+//   256x256x180, 724^2: 223 201 214 293 / 150 143 162 235
+//   256x256x180, 1024^2: 292 307 386 572 / 193 229 287 456
+// Forms whose samples take longer (FP32 shading, B-spline, 2-D table) gain
+// further up than the plain and the 16-bit ones.
+static int lanes_per_ray(const MarchArgs &a, int nviews) {
+    // the box's corners bound the part of the image whose rays can meet it;
+    // its silhouette fills about two thirds of that rectangle
+    const CamRec &c = a.cam;
+    double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0}, diag2 = 0.0;
+    bool behind = false;
+    for (int q = 0; q < 8; q++) {
+        double d[3], z = 0.0, u[2] = {0.0, 0.0};
+        for (int i = 0; i < 3; i++) {
+            d[i] = (((q >> i) & 1 ? a.vol.n[i] - 1 : 0) - (double)c.o[i]) * a.vol.s[i];
+            z += d[i] * c.f[i];
+            u[0] += d[i] * c.r[i];
+            u[1] += d[i] * c.u[i];
+        }
+        if (!(z > 0.0)) behind = true;
+        else {
+            const double t[2] = {c.tx, c.ty};
+            for (int i = 0; i < 2; i++) {
+                const double e = u[i] / (z * t[i]);
+                lo[i] = e < lo[i] ? e : lo[i];
+                hi[i] = e > hi[i] ? e : hi[i];
+            }
+        }
+    }
+    double part = 1.0;
+    for (int i = 0; i < 2 && !behind; i++) {
+        const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
+        part *= h > l ? (h - l) * 0.5 : 0.0;
+    }
+    for (int i = 0; i < 3; i++) diag2 += (double)(a.vol.n[i] - 1) * a.vol.s[i] * (a.vol.n[i] - 1) * a.vol.s[i];
+    const double hits = 0.65 * part * c.W * c.H * nviews;
+    const double steps = sqrt(diag2) / ((double)a.p.step_vox * a.vol.smin);
+    const bool heavy = (a.p.shade && a.vol.storage == RC_STORE_F32) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2;
+    if (hits <= (heavy ? 22e3 : 7e3) && hits <= 70.0 * steps) return 8;
+    if (hits <= 76e3 && hits <= 190.0 * steps) return 4;
+    if (hits <= 155e3 && hits <= (heavy ? 390.0 : 190.0) * steps) return 2;
+    return 1;
+}
+
+template <int F, int L>
+static cudaError_t launch_wide(const MarchArgs &a, int nviews, cudaStream_t s) {
+    const bool smem = !(F & kTF2);
+    constexpr int W = kWarpsX * WideTile<L>::X, H = kWarpsY * WideTile<L>::Y;
+    switch (a.vol.storage) {
+        case RC_STORE_F32: return launch_kernel(wide_kernel<RC_STORE_F32, F, L>, a, nviews, smem, s, W, H);
+        case RC_STORE_F16: return launch_kernel(wide_kernel<RC_STORE_F16, F, L>, a, nviews, smem, s, W, H);
+        default: return launch_kernel(wide_kernel<RC_STORE_U16, F, L>, a, nviews, smem, s, W, H);
+    }
 }
 
 // Composite march with sample form F and opacity-correction mode RM for the
@@ -293,6 +509,11 @@ static cudaError_t launch_composite_rm(const MarchArgs &a, int nviews, cudaStrea
 // The step ratios of the fixed modes (1, 1/2, 1/4) get their own instances.
 template <int F>
 static cudaError_t launch_composite(const MarchArgs &a, int nviews, cudaStream_t s) {
+    switch (lanes_per_ray(a, nviews)) {
+        case 8: return launch_wide<F, 8>(a, nviews, s);
+        case 4: return launch_wide<F, 4>(a, nviews, s);
+        case 2: return launch_wide<F, 2>(a, nviews, s);
+    }
     switch (a.p.rmode) {
         case 0: return launch_composite_rm<F, 0>(a, nviews, s);
         case 1: return launch_composite_rm<F, 1>(a, nviews, s);

@@ -42,3 +42,40 @@ def test_positions_outside_the_box_clamp(rc, orc, dims, distance, entries, filt)
         compare(img, o, TOL_FP32)
     finally:
         r.close()
+
+
+# The launch form depends on the number of rays: one small view marches with
+# several lanes per ray, a hundred copies of it with one. The images and the
+# sample counts are the same. Ragged image sizes; a camera inside the box; a
+# table whose opacities end rays after a few samples.
+@pytest.mark.parametrize("storage", ["F32", "F16", "U16"])
+@pytest.mark.parametrize("form", [dict(shade=False), dict(shade=True), dict(shade=True, filter=1), dict(shade=False, tf2=True)])
+@pytest.mark.parametrize("size,views", [((37, 21), 1200), ((97, 75), 130), ((260, 201), 18)])
+def test_lanes_per_ray_change_nothing(rc, storage, form, size, views):
+    import torch
+    form = dict(form)
+    dims, spacing = (50, 41, 37), (1.0, 1.0, 1.5)
+    ph = synth.head_phantom(dims, spacing, seed=5, tumor_radius_vox=3)
+    r = GPURenderer(rc, ph.vol, spacing, getattr(rc, "RC_STORE_" + storage))
+    try:
+        w, h = size
+        inside = dict(eye=(20.0, 18.0, 25.0), target=(40.0, 20.0, 30.0), up=(0.0, 0.0, 1.0), fovy_deg=50.0, width=w, height=h)
+        tf2 = form.pop("tf2", False)
+        for alpha, step in ((1.0, 0.5), (8.0, 0.3)):
+            tab = synth.tf2d_table(64, 8) if tf2 else synth.tf_table(200)
+            tab[..., 3] = np.minimum(1.0, tab[..., 3] * alpha)
+            if tf2:
+                rc.rc_tf2d_set(r.ctx, tab, 1200.0)
+            else:
+                r.set_tf(tab)
+            for cam in (synth.orbit_camera(dims, spacing, 77.0, width=w, height=h), inside):
+                P = dict(step_vox=step, term=0.95, **form)
+                one, st = r.render(cam, stats=True, **P)
+                many = torch.empty((views, h, w, 4), device="cuda")
+                sm = rc.rc_render_views(r.ctx, r.vol, P, [cam] * views, many, stats=True)
+                assert (many == torch.from_numpy(one).cuda()[None]).all()
+                for key in ("dense_samples", "evaluated_samples", "rays_hit", "rays_total"):
+                    assert sm[key] == views * st[key], key
+                assert st["evaluated_samples"] > 0
+    finally:
+        r.close()
