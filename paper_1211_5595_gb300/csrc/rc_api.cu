@@ -1192,7 +1192,6 @@ rc_status rc_render_backward(rc_context *ctx, const rc_volume *vol, const rc_ren
     a.m.p.skip = 0;
     a.dimg = reinterpret_cast<const float4 *>(dL_dimage);
     a.acc = reinterpret_cast<long long *>(ctx->d_scratch);
-    a.acc_scale = 0.0f;
     a.fimg = nullptr;
     RC_CUDA(ctx, launch_adjoint(a, 1, dL_dtf, ctx->stream));
     return RC_OK;
@@ -1243,7 +1242,6 @@ static rc_status backward_views(rc_context *ctx, const rc_volume *vol, const rc_
     a.m.cams = ctx->d_cams;
     a.dimg = reinterpret_cast<const float4 *>(dL_dimages);
     a.acc = reinterpret_cast<long long *>(ctx->d_scratch);
-    a.acc_scale = 0.0f;
     a.fimg = reinterpret_cast<const float4 *>(images);
     RC_CUDA(ctx, launch_adjoint(a, nviews, dL_dtf, ctx->stream));
     return RC_OK;
@@ -1315,7 +1313,6 @@ rc_status rc_render_backward_noalloc(rc_context *ctx, const rc_volume *vol, cons
     a.m.p.skip = 0;
     a.dimg = reinterpret_cast<const float4 *>(dL_dimage);
     a.acc = scratch;            // cleared on the stream before the kernel runs
-    a.acc_scale = 0.0f;
     a.fimg = nullptr;
     RC_CUDA(ctx, launch_adjoint(a, 1, dL_dtf, ctx->stream));
     return RC_OK;

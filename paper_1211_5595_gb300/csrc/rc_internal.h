@@ -124,7 +124,7 @@ struct AdjointArgs {
     const float4 *dimg;            // H x W dL/dI
     const float4 *fimg;            // the forward images (C, 1 - T) of the same views, or null: recomputed
     long long *acc;                // K x 4 fixed-point accumulators (scratch)
-    float acc_scale;               // fixed-point units per unit of gradient
+    unsigned *next;                // chunk queue of a 2-D table's launch (set by launch_adjoint)
 };
 
 // ---- learned proposal ----------------------------------------------------
@@ -230,7 +230,7 @@ cudaError_t launch_levels(const uint16_t *mn4, const uint16_t *mx4, const int n[
 cudaError_t launch_march(const MarchArgs &a, int nviews, cudaStream_t s);
 cudaError_t launch_march_cubic(const MarchArgs &a, int nviews, cudaStream_t s);   // filter = B-spline
 cudaError_t launch_march_tf2(const MarchArgs &a, int nviews, cudaStream_t s);     // trilinear, 2-D table
-cudaError_t launch_adjoint(const AdjointArgs &a, int nviews, float *dL_dtf, cudaStream_t s);
+cudaError_t launch_adjoint(AdjointArgs a, int nviews, float *dL_dtf, cudaStream_t s);
 cudaError_t launch_absmax(const float *x, long long n, float *out, cudaStream_t s);
 cudaError_t launch_profiles(const MarchArgs &a, float *out, cudaStream_t s);
 cudaError_t launch_features(const MarchArgs &a, float *out, cudaStream_t s);
