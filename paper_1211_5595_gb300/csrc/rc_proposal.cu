@@ -27,41 +27,94 @@ __device__ __forceinline__ void tile_pixel(int &x, int &y) {
 // opacity profiles: 512 samples at the centres of 512 equal segments of the
 // chord, no termination; weights T_k a'_k summed 16 per bin; T at the end
 // ---------------------------------------------------------------------------
+// Four lanes per ray: lane j evaluates samples 4i + j of a bin, then the group
+// runs the bin's recurrence in sample order from shuffles (an empty sample has
+// opacity exactly 0 and changes nothing, so the values are those of one lane
+// marching alone). A ray's 512 samples are a serial chain and only the rays that
+// meet the volume have one, so one lane per ray left the GPU waiting on latency
+// (256x256x180, 256^2 view 240 us, 512^2 257, 1024^2 602; now 68, 136 and 398).
+// When a whole bin is empty, the bins up to the exit of the last sample's block
+// are too. Rows are staged in shared memory and written 132 contiguous bytes
+// per ray.
+constexpr int kProfLanes = 4, kProfTileX = 8, kProfTileY = 4;      // pixels per CTA of 4 warps (4 x 2 per warp)
+
+__device__ __forceinline__ int jump_block_grid(const Ray &R, const VolDev &v, const Cell &c, int j, int s, float ta,
+                                               float seg, int n);
+
 template <int ST>
 __global__ void __launch_bounds__(128) profiles_kernel(const MarchArgs a, float *out) {
     extern __shared__ float4 s_tf[];
+    __shared__ float s_row[4][32 / kProfLanes][kOutUsed];
     load_tf(a.tf, s_tf);
     __syncthreads();
-    int x, y;
-    tile_pixel(x, y);
-    if (x >= a.cam.W || y >= a.cam.H) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane % kProfLanes, ray = lane / kProfLanes,
+              first = lane - j;
+    const int x0 = blockIdx.x * kProfTileX + (warp & 1) * 4, y0 = blockIdx.y * kProfTileY + (warp >> 1) * 2;
+    const int x = x0 + (ray & 3), y = y0 + (ray >> 2);
     Ray R;
-    const bool hit = setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
-    float *o = out + ((size_t)y * a.cam.W + x) * kOutUsed;
-    if (!hit) {
-        for (int b = 0; b < kBins; b++) o[b] = 0.0f;
-        o[kBins] = 1.0f;
-        return;
-    }
-    const float delta = __fdiv_rn(__fsub_rn(R.tf, R.tn), (float)kProfSamples);
-    const float ratio = __fdiv_rn(delta, a.vol.smin);
+    const bool hit = x < a.cam.W && y < a.cam.H && setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
+    float *row = s_row[warp][ray];
+    for (int b = j; b < kBins; b += kProfLanes) row[b] = 0.0f;
+    __syncwarp();
     float T = 1.0f;
-    for (int b = 0; b < kBins; b++) {
-        float acc = 0.0f;
-        for (int kk = 0; kk < kProfSamples / kBins; kk++) {
-            const int k = b * (kProfSamples / kBins) + kk;
-            float p[3];
-            position_at(R, __fmaf_rn((float)k + 0.5f, delta, R.tn), p);
+    if (__any_sync(0xffffffffu, hit)) {
+        constexpr int kPerBin = kProfSamples / kBins, kPerLane = kPerBin / kProfLanes;
+        const float delta = hit ? __fdiv_rn(__fsub_rn(R.tf, R.tn), (float)kProfSamples) : 0.0f;
+        const float ratio = __fdiv_rn(delta, a.vol.smin);
+        int b = hit ? 0 : kBins;
+        while (__any_sync(0xffffffffu, b < kBins)) {
+            const bool on = b < kBins;
+            float al[kPerLane];
             Cell c;
-            cell_of(a.vol, p, c);
-            if (a.p.skip && empty_level(a, a.lvl, c)) continue;               // opacity exactly 0
-            float4 e = eval_sample<ST, false>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio);
-            acc = __fmaf_rn(T, e.w, acc);
-            T = T * (1.0f - e.w);
+            int s = 0;
+            unsigned some = 0;
+#pragma unroll
+            for (int i = 0; i < kPerLane; i++) {
+                al[i] = 0.0f;
+                if (on) {
+                    float p[3];
+                    position_at(R, __fmaf_rn((float)(b * kPerBin + i * kProfLanes + j) + 0.5f, delta, R.tn), p);
+                    cell_of(a.vol, p, c);
+                    s = a.p.skip ? empty_level(a, a.lvl, c) : 0;
+                    if (!s) {
+                        al[i] = eval_sample<ST, false>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio).w;
+                        some = 1;
+                    }
+                }
+            }
+            float acc = 0.0f;
+            if (__any_sync(0xffffffffu, some)) {
+#pragma unroll
+                for (int k = 0; k < kPerBin; k++) {
+                    const float w = __shfl_sync(0xffffffffu, al[k / kProfLanes], first + k % kProfLanes);
+                    acc = __fmaf_rn(T, w, acc);
+                    T = T * (1.0f - w);
+                }
+            }
+            const unsigned in_group = (__ballot_sync(0xffffffffu, some) >> first) & ((1u << kProfLanes) - 1u);
+            int next = b + 1;
+            if (on && in_group == 0) {
+                // the sample after the block of each lane's last sample; the
+                // bins wholly before the last lane's stay zero
+                const int k = jump_block_grid(R, a.vol, c, b * kPerBin + kPerBin - kProfLanes + j, s, R.tn, delta, kProfSamples);
+                next = max(next, k / kPerBin);
+            }
+            next = __shfl_sync(0xffffffffu, next, first + kProfLanes - 1);
+            if (on) {
+                if (j == 0 && in_group) row[b] = acc;
+                b = next;
+            }
         }
-        o[b] = acc;
     }
-    o[kBins] = T;
+    if (j == 0) row[kBins] = T;
+    __syncwarp();
+    // two image rows of up to four rays, contiguous in the output
+    const int rays = min(4, a.cam.W - x0);
+    for (int r = 0; r < 2 && y0 + r < a.cam.H; r++) {
+        float *o = out + ((size_t)(y0 + r) * a.cam.W + x0) * kOutUsed;
+        const float *src = s_row[warp][4 * r];
+        for (int e = lane; e < rays * kOutUsed; e += 32) o[e] = src[e];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -133,17 +186,43 @@ __device__ __forceinline__ uint32_t ray_features(const VolDev &v, const uint8_t 
     return mask;
 }
 
+// One thread per ray. A warp's 32 rows are staged in shared memory (rows padded
+// to 116 floats: eight lanes' 16-byte stores then hit eight different bank
+// groups) and written as four runs of contiguous rows. VEC: the output is
+// 16-byte aligned. Bound by the stores: 262144 rays (117 MB) 151 us with each
+// thread writing its own row by 4-byte stores, 40 by 16-byte stores, 25
+// staged (17 at the copy rate); 1048576 rays 768, 303 and 79 (69).
+constexpr int kFeatRow = kFeat + 4;
+constexpr int kFeatSmem = 4 * 32 * kFeatRow * (int)sizeof(float);
+
+template <bool VEC>
 __global__ void __launch_bounds__(128) features_kernel(const MarchArgs a, float *out) {
+    extern __shared__ float4 s_tf[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *rows = reinterpret_cast<float *>(s_tf) + warp * 32 * kFeatRow;
     int x, y;
     tile_pixel(x, y);
-    if (x >= a.cam.W || y >= a.cam.H) return;
     Ray R;
-    const bool hit = setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
-    float *o = out + ((size_t)y * a.cam.W + x) * kFeat;
+    const bool hit = x < a.cam.W && y < a.cam.H && setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
+    float4 *mine = reinterpret_cast<float4 *>(rows + lane * kFeatRow);
     ray_features(a.vol, a.occ, R, hit, [&](int chunk, const float (&v)[8]) {
-#pragma unroll
-        for (int i = 0; i < 8; i++) o[8 * chunk + i] = v[i];
+        mine[2 * chunk] = make_float4(v[0], v[1], v[2], v[3]);
+        mine[2 * chunk + 1] = make_float4(v[4], v[5], v[6], v[7]);
     });
+    __syncwarp();
+    const int x0 = x - (lane & 7), y0 = y - (lane >> 3);
+    const int n = min(8, a.cam.W - x0);                       // rays of a run (none when the tile is outside)
+    for (int r = 0; r < 4 && y0 + r < a.cam.H; r++) {
+        float *o = out + ((size_t)(y0 + r) * a.cam.W + x0) * kFeat;
+        const float *src = rows + 8 * r * kFeatRow;
+        if (VEC) {
+            for (int e = lane; e < n * (kFeat / 4); e += 32)
+                reinterpret_cast<float4 *>(o)[e] =
+                    *reinterpret_cast<const float4 *>(src + (e / (kFeat / 4)) * kFeatRow + 4 * (e % (kFeat / 4)));
+        } else {
+            for (int e = lane; e < n * kFeat; e += 32) o[e] = src[(e / kFeat) * kFeatRow + e % kFeat];
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1118,11 +1197,12 @@ static dim3 image_grid(const CamRec &c) { return dim3((c.W + 15) / 16, (c.H + 7)
 cudaError_t launch_profiles(const MarchArgs &a, float *out, cudaStream_t s) {
     const size_t smem = (size_t)a.tf.K * sizeof(float4);
     auto go = [&](auto kern) -> cudaError_t {
-        if (smem > 48 * 1024) {
+        if (smem > 40 * 1024) {       // the staged rows take 4.2 KB of the 48 KB beside it
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<image_grid(a.cam), 128, smem, s>>>(a, out);
+        const dim3 grid((a.cam.W + kProfTileX - 1) / kProfTileX, (a.cam.H + kProfTileY - 1) / kProfTileY);
+        kern<<<grid, 128, smem, s>>>(a, out);
         return cudaGetLastError();
     };
     switch (a.vol.storage) {
@@ -1133,7 +1213,10 @@ cudaError_t launch_profiles(const MarchArgs &a, float *out, cudaStream_t s) {
 }
 
 cudaError_t launch_features(const MarchArgs &a, float *out, cudaStream_t s) {
-    features_kernel<<<image_grid(a.cam), 128, 0, s>>>(a, out);
+    auto kern = (reinterpret_cast<uintptr_t>(out) & 15u) == 0 ? features_kernel<true> : features_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFeatSmem);
+    if (e != cudaSuccess) return e;
+    kern<<<image_grid(a.cam), 128, kFeatSmem, s>>>(a, out);
     return cudaGetLastError();
 }
 
