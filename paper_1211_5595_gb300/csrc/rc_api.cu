@@ -1373,7 +1373,7 @@ static rc_status net_alloc(rc_context *ctx) {
     uint8_t *f = nullptr;
     if (dev_alloc(&p, kParams * sizeof(float)) != cudaSuccess || dev_alloc(&m, kParams * sizeof(float)) != cudaSuccess ||
         dev_alloc(&v, kParams * sizeof(float)) != cudaSuccess || dev_alloc(&g, kParams * sizeof(float)) != cudaSuccess ||
-        dev_alloc(&f, kUmmaAllBytes) != cudaSuccess) {
+        dev_alloc(&f, kUmmaBytes) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p);
         cudaFree(m);
@@ -1509,7 +1509,7 @@ rc_status rc_proposal_forward(rc_context *ctx, const float *features, int64_t n,
 }
 
 static rc_status net_grad(rc_context *ctx, const float *features, const float *targets, int64_t n, float *grad,
-                          float *loss) {
+                          float *loss, const AdamArgs *step) {
     const int grid = train_grid(n);
     if (ctx->partial_blocks < grid) {
         float *pp = nullptr, *lp = nullptr;
@@ -1537,7 +1537,7 @@ static rc_status net_grad(rc_context *ctx, const float *features, const float *t
     a.inv_n = (float)(1.0 / (double)n);
     a.budget = wait_budget(&a.issue_mma);
     a.err = error_word(ctx);
-    RC_CUDA(ctx, launch_train_grad(a, grid, grad, loss, ctx->stream));
+    RC_CUDA(ctx, launch_train_grad(a, grid, grad, loss, step, ctx->stream));
     return RC_OK;
 }
 
@@ -1547,7 +1547,7 @@ rc_status rc_proposal_grad(rc_context *ctx, const float *features, const float *
     if (st != RC_OK) return st;
     if (!grad) return fail(ctx, RC_ERR_INVALID_ARG, "rc_proposal_grad: grad is NULL");
     DeviceScope ds(ctx->device);
-    return net_grad(ctx, features, targets, n, grad, loss);
+    return net_grad(ctx, features, targets, n, grad, loss, nullptr);
 }
 
 rc_status rc_proposal_train_step(rc_context *ctx, const float *features, const float *targets, int64_t n, float lr,
@@ -1556,11 +1556,12 @@ rc_status rc_proposal_train_step(rc_context *ctx, const float *features, const f
     if (st != RC_OK) return st;
     if (!(lr > 0.0f) || !isfinite(lr)) return fail(ctx, RC_ERR_INVALID_ARG, "rc_proposal_train_step: lr %g", (double)lr);
     DeviceScope ds(ctx->device);
-    st = net_grad(ctx, features, targets, n, ctx->d_grad, loss);
+    const double t = (double)(ctx->adam_step + 1);
+    const AdamArgs step{ctx->d_param, ctx->d_m, ctx->d_v, ctx->d_umma, lr, (float)(1.0 - pow(0.9, t)),
+                        (float)(1.0 - pow(0.999, t))};
+    st = net_grad(ctx, features, targets, n, ctx->d_grad, loss, &step);
     if (st != RC_OK) return st;
     ctx->adam_step++;
-    RC_CUDA(ctx, launch_adam(ctx->d_param, ctx->d_m, ctx->d_v, ctx->d_grad, ctx->adam_step, lr, ctx->stream));
-    RC_CUDA(ctx, launch_pack(ctx->d_param, ctx->d_umma, ctx->stream));
     return RC_OK;
 }
 

@@ -822,288 +822,402 @@ __global__ void __launch_bounds__(128) importance_kernel(const ImportanceArgs A)
 // weight gradient (rays as K, accumulated in TMEM over the CTA's tiles) and
 // the input gradient (rays as M)
 // ---------------------------------------------------------------------------
-// Weight gradient of layer l: dW_l = H_{l-1}^T dZ_l over the tile's 128 rays,
-// an M = 128, K = 128 MMA that reads both operands MN-major: A = H^T from H
-// itself (rays x inputs, the forward's K-major operand, whose ones column
-// gives the D row of the bias gradient sum_rays dZ, zero columns after it)
-// and B = dZ^T from dZ (rays x outputs): no transposed copies. Input gradient:
-// dH_{l-1} = dZ_l W_l^T, A = dZ (rays x outputs, K-major), B = W_l (inputs x
-// outputs). All operands BF16 (dZ rounded once), FP32 accumulation. (Writing
-// H^T and dZ^T as separate transposed operands took 1.062 ms per 1 M rays
-// against 0.764 with the MN-major reads; the gradients are identical bit for
-// bit.)
+// A CTA runs two groups of 128 threads (thread = ray = TMEM lane), each on its
+// own tiles of 128 rays, and one thread that issues every MMA of both: while one
+// group's MMAs run, the other group's threads work on their accumulators. The
+// issuing order is fixed (step by step, group 0 then group 1, tiles in ascending
+// order), so the groups share the weight-gradient accumulators and the sums do
+// not depend on timing.
+//
+// Weight gradient of layer l: dW_l = H_{l-1}^T dZ_l over the tile's 128 rays, an
+// M = 128, K = 128 MMA that reads both operands MN-major straight from the
+// forward's K-major ones: A starts at H_{l-1} (or at the ones chunk before it)
+// and covers 16 chunks of 8 columns; the row of the ones column is the bias
+// gradient, and rows that fall on whatever lies beyond H_{l-1} are never read
+// back. Input gradient: dH_{l-1} = dZ_l W_l^T, whose B operand is the forward's
+// weight operand read MN-major. dZ_l overwrites H_l in place (its readers, the
+// MMAs of step l + 1, have completed). Shared memory per group, in chunks of
+// 8 columns x 128 rays (2 KB): X 14 | ones | H1 8 | H2 8 | ones | H3 8 | dZ4 6.
+// All operands BF16 (dZ rounded once), FP32 accumulation.
+//
+// Bound: the chain of eight dependent MMA steps per tile with the threads' work
+// between them. 1048576 rays 746 us with one group of 128 threads per SM that
+// issued for itself and kept 128-column operands, RC_TRAIN_US now (131 us at the
+// issue rate, 90 us at the copy rate for the features and targets).
+constexpr int kChX = 0, kChOne0 = 14, kChH1 = 15, kChH2 = 23, kChOne1 = 31, kChH3 = 32, kChDz4 = 40, kChunks = 46;
+constexpr int kChunkBytes = 2048;
+constexpr int kTrainThreads = 2 * kGroupThreads + 32;      // two groups and the issuing warp
 struct TrainSmem {
-    uint8_t w[kUmmaAllBytes];              // forward and backward B operands
-    uint8_t x[128 * 128 * 2];              // features (rays x 112), ones column 112, zero columns after it
-    uint8_t h[3][128 * 128 * 2];           // H1..H3 (rays x 64), ones column 64, zero columns after it
-    uint8_t adz[128 * kHid * 2];           // dZ (rays x outputs)
+    uint8_t op[2][kChunks * kChunkBytes];  // operands of the groups (the last A operand reads one chunk into what follows)
+    uint8_t w[kUmmaBytes];                 // the four layers' weight operands
     float bias[3 * kHid + kN4];
-    float wloss[4];
-    unsigned long long bar_w, bar_m;
+    float wloss[8];
+    unsigned long long bar_w, ready[2], done[2];
     uint32_t tmem;
 };
-constexpr int kTrainCols = 512;            // D (64) | dW4 (48) | dW3 | dW2 | dW1 (64 each)
-constexpr uint32_t kColD = 0, kColW4 = 64, kColW3 = 128, kColW2 = 192, kColW1 = 256;
+constexpr int kTrainCols = 512;
+constexpr uint32_t kColD = 0, kColW = 128;                 // D of group g at 64 g; dW of layer l at 128 + 64 l
 
-// D (+)= A B^T over K / 16 MMAs, A with `rows_a` rows, B with n rows.
-__device__ __forceinline__ void issue_mma(uint32_t a0, int rows_a, uint32_t b0, int n, int K, uint32_t tmem_d,
-                                          bool accumulate) {
-    const uint32_t lbo_a = (uint32_t)(rows_a / 8) * 128, lbo_b = (uint32_t)(n / 8) * 128;
-    const uint32_t idesc = tc::idesc_bf16_f32(128, n);
-    for (int ks = 0; ks < K / 16; ks++)
-        tc::mma_bf16(tmem_d, tc::smem_desc(a0 + ks * 2 * lbo_a, lbo_a, 128), tc::smem_desc(b0 + ks * 2 * lbo_b, lbo_b, 128),
-                     idesc, accumulate || ks > 0);
+// First chunk of the layer input H_l (l = 0: the features), of the weight
+// gradient's A operand of layer l, and its accumulator row of input 0 and of
+// the bias.
+__device__ __forceinline__ int input_chunk(int l) { return l == 0 ? kChX : l == 1 ? kChH1 : l == 2 ? kChH2 : kChH3; }
+__device__ __forceinline__ int grad_chunk(int l) { return l == 0 ? kChX : l == 1 ? kChOne0 : l == 2 ? kChH2 : kChOne1; }
+__device__ __forceinline__ int grad_row0(int l) { return l == 1 || l == 3 ? 8 : 0; }
+__device__ __forceinline__ int bias_row(int l) { return l == 0 ? kFeat : l == 2 ? kHid : 0; }
+
+// One layer of the forward: D = A W^T, or of the backward: the weight gradient
+// into its accumulator, then (l > 0) the input gradient into D; with a commit.
+__device__ __forceinline__ void issue_forward(uint32_t op, uint32_t w, int l, uint32_t tmem_d) {
+    const NetLayer L = net_layer(l);
+    const uint32_t a0 = op + input_chunk(l) * kChunkBytes, b0 = w + L.b_off, lbo_b = (uint32_t)(L.N / 8) * 128;
+    const uint32_t idesc = tc::idesc_bf16_f32(128, L.N);
+    for (int ks = 0; ks < L.K / 16; ks++)
+        tc::mma_bf16(tmem_d, tc::smem_desc(a0 + ks * 2 * kChunkBytes, kChunkBytes, 128),
+                     tc::smem_desc(b0 + ks * 2 * lbo_b, lbo_b, 128), idesc, ks > 0);
 }
 
-// D (+)= A B^T over K = 128 rays with A and B read MN-major from operands
-// stored rays x M and rays x N (core matrices of 8 rays x 8 elements; the
-// K-adjacent cores 128 bytes apart, the M- or N-adjacent ones 2048): the
-// weight gradient straight from the forward's operands.
-__device__ __forceinline__ void issue_mma_mn(uint32_t a0, uint32_t b0, int n, uint32_t tmem_d, bool accumulate) {
-    const uint32_t idesc = tc::idesc_bf16_f32(128, n) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
-    for (int ks = 0; ks < 8; ks++)
-        tc::mma_bf16(tmem_d, tc::smem_desc(a0 + ks * 256, 128, 2048), tc::smem_desc(b0 + ks * 256, 128, 2048), idesc,
-                     accumulate || ks > 0);
+__device__ __forceinline__ void issue_backward(uint32_t op, uint32_t w, int l, uint32_t tmem_w, uint32_t tmem_d,
+                                               bool accumulate) {
+    const NetLayer L = net_layer(l);
+    const uint32_t dz = op + (l == 3 ? kChDz4 : input_chunk(l + 1)) * kChunkBytes;
+    const uint32_t a0 = op + grad_chunk(l) * kChunkBytes;
+    const uint32_t id_w = tc::idesc_bf16_f32(128, L.N) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
+    for (int ks = 0; ks < 8; ks++)         // 16 rays each
+        tc::mma_bf16(tmem_w, tc::smem_desc(a0 + ks * 256, 128, kChunkBytes), tc::smem_desc(dz + ks * 256, 128, kChunkBytes),
+                     id_w, accumulate || ks > 0);
+    if (l == 0) return;
+    const uint32_t id_d = tc::idesc_bf16_f32(128, kHid) | tc::kIdescMnMajorB;
+    for (int ks = 0; ks < L.N / 16; ks++)  // 16 outputs each
+        tc::mma_bf16(tmem_d, tc::smem_desc(dz + ks * 2 * kChunkBytes, kChunkBytes, 128),
+                     tc::smem_desc(w + L.b_off + ks * 256, 128, (uint32_t)(L.N / 8) * 128), id_d, ks > 0);
 }
 
-// A bounded wait for the CTA's committed MMAs (all 128 threads).
-__device__ __forceinline__ bool train_sync_mma(const TrainArgs &A, uint32_t bar, uint32_t &phase) {
-    const bool ok = __syncthreads_and(tc::bar_wait(bar, phase, A.budget));
-    if (ok) phase ^= 1u;
-    tc::fence_after();
-    return ok;
-}
-
-__device__ __forceinline__ void operands_ready() {
-    tc::fence_async_smem();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-}
-
-// One BF16 value at (row, k) of a K-major operand with `rows` rows.
-__device__ __forceinline__ void put_bf16(uint8_t *M, int row, int k, int rows, float v) {
-    *reinterpret_cast<__nv_bfloat16 *>(M + tc::core_offset(row, k, rows)) = __float2bfloat16_rn(v);
-}
-
-__device__ __forceinline__ float get_bf16(const uint8_t *M, int row, int k, int rows) {
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(M + tc::core_offset(row, k, rows)));
-}
-
-// dZ of this thread's ray (n values, zeros up to k_pad) as row t of the dZ
-// operand, 8 values per 16-byte store.
-__device__ __forceinline__ void put_dz(TrainSmem &S, const float (&dz)[kHid], int n, int k_pad, int t) {
+// dZ of this thread's ray (N values, zeros up to a multiple of 8) as row t of a
+// K-major operand, 8 values per 16-byte store.
+template <int N>
+__device__ __forceinline__ void put_dz(uint8_t *A, const float (&dz)[N], int t) {
 #pragma unroll
-    for (int j0 = 0; j0 < kHid; j0 += 8) {
-        if (j0 >= k_pad) break;
+    for (int j0 = 0; j0 < N; j0 += 8) {
         uint4 q;
         uint32_t *w = reinterpret_cast<uint32_t *>(&q);
 #pragma unroll
         for (int h = 0; h < 4; h++) {
-            const float lo = j0 + 2 * h < n ? dz[j0 + 2 * h] : 0.0f, hi = j0 + 2 * h + 1 < n ? dz[j0 + 2 * h + 1] : 0.0f;
-            __nv_bfloat162 b2 = __floats2bfloat162_rn(lo, hi);
+            __nv_bfloat162 b2 = __floats2bfloat162_rn(dz[j0 + 2 * h], dz[j0 + 2 * h + 1]);
             w[h] = *reinterpret_cast<uint32_t *>(&b2);
         }
-        *reinterpret_cast<uint4 *>(S.adz + tc::core_offset(t, j0, 128)) = q;
+        *reinterpret_cast<uint4 *>(A + tc::core_offset(t, j0, 128)) = q;
     }
 }
 
-__global__ void __launch_bounds__(128) tc_train_kernel(const TrainArgs A) {
+__global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem_raw);
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const uint32_t bar_w = tc::smem_addr(&S.bar_w), bar_m = tc::smem_addr(&S.bar_m);
-    if (warp == 0) tc::tmem_alloc<kTrainCols>(tc::smem_addr(&S.tmem));
-    if (t == 0) {
-        tc::bar_init(bar_w, 1);
-        tc::bar_init(bar_m, 1);
+    const int tid = threadIdx.x, g = tid / kGroupThreads, t = tid % kGroupThreads;     // g = 2: the issuing warp
+    const int warp = t >> 5, lane = t & 31;
+    if (tid < 32) tc::tmem_alloc<kTrainCols>(tc::smem_addr(&S.tmem));
+    if (tid == 0) {
+        tc::bar_init(tc::smem_addr(&S.bar_w), 1);
+        for (int i = 0; i < 2; i++) {
+            tc::bar_init(tc::smem_addr(&S.ready[i]), kGroupThreads);
+            tc::bar_init(tc::smem_addr(&S.done[i]), 1);
+        }
     }
-    for (int i = t; i < 3 * kHid + kN4; i += blockDim.x) {
+    for (int i = tid; i < 3 * kHid + kN4; i += blockDim.x) {
         const int l = i / kHid, j = i % kHid;
         float b = 0.0f;
         if (l < 3) b = A.params[(l == 0 ? kOffB1 : l == 1 ? kOffB2 : kOffB3) + j];
         else if (j < kOut) b = A.params[kOffB4 + j];
         S.bias[i] = b;
     }
-    // features and hidden layers all zero, then their ones columns (constant:
-    // the tiles rewrite the value columns only)
-    for (int i = t; i < 4 * 128 * 128 * 2 / 16; i += blockDim.x) reinterpret_cast<uint4 *>(S.x)[i] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    put_bf16(S.x, t, kFeat, 128, 1.0f);
-    for (int l = 0; l < 3; l++) put_bf16(S.h[l], t, kHid, 128, 1.0f);
+    if (g < 2) {
+        const uint4 one = make_uint4(0x3F80u, 0u, 0u, 0u);          // BF16 1, then seven zeros
+        *reinterpret_cast<uint4 *>(S.op[g] + kChOne0 * kChunkBytes + t * 16) = one;
+        *reinterpret_cast<uint4 *>(S.op[g] + kChOne1 * kChunkBytes + t * 16) = one;
+    }
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = S.tmem;
-    if (t == 0) tc::bulk_g2s(tc::smem_addr(S.w), A.umma, kUmmaAllBytes, bar_w);
-    bool ok = __syncthreads_and(tc::bar_wait(bar_w, 0, A.budget));
-    if (!ok) tc::bar_wait(bar_w, 0, A.budget);
-    uint32_t phase = 0;
-    bool mma_waited_out = false, first = true;
-    float loss_sum = 0.0f;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);      // this warp's lanes
+    if (tid == 0) tc::bulk_g2s(tc::smem_addr(S.w), A.umma, kUmmaBytes, tc::smem_addr(&S.bar_w));
+    bool ok = __syncthreads_and(tc::bar_wait(tc::smem_addr(&S.bar_w), 0, A.budget));
+    if (!ok) tc::bar_wait(tc::smem_addr(&S.bar_w), 0, A.budget);     // the copy may still be in flight
     const long long ntiles = (A.n + 127) / 128;
+    float loss_sum = 0.0f;
+    if (ok && tid == 2 * kGroupThreads) {
+        // the issuing thread: steps 0-3 the forward layers, 4-7 the backward
+        // ones, for the tiles i = 2 pair + group of this CTA
+        const uint32_t w = tc::smem_addr(S.w);
+        uint32_t phase[2] = {0u, 0u};
+        bool issued[2] = {false, false};
+        for (long long pair = 0; ok && blockIdx.x + 2 * pair * gridDim.x < ntiles; pair++) {
 #pragma unroll 1
-    for (long long tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-        const long long r0 = tile * 128, r = r0 + t;
-        const bool valid = r < A.n;
-        // the CTA's next tile (features and targets) into L2
-        const long long nt = tile + gridDim.x;
-        if (t == 0 && nt < ntiles) {
-            const long long nrows = min((long long)128, A.n - nt * 128);
-            tc::prefetch_l2(A.feat + nt * 128 * kFeat, (uint32_t)(nrows * kFeat * sizeof(float)));
-            tc::prefetch_l2(A.target + nt * 128 * kOutUsed, (uint32_t)((nrows * kOutUsed * sizeof(float)) & ~15ull));
-        }
-        // features: coalesced float4 loads of the contiguous tile -> BF16
-        {
-            const float4 *src = reinterpret_cast<const float4 *>(A.feat + r0 * kFeat);
-            const long long nvalid = min((long long)128, A.n - r0);
-#pragma unroll 7
-            for (int i = 0; i < 128 * kFeat / 4 / 128; i++) {
-                const int e = i * 128 + t, row = e / (kFeat / 4), k = (e % (kFeat / 4)) * 4;
-                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (row < nvalid) v = __ldg(src + e);
-                __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-                uint2 q;
-                q.x = *reinterpret_cast<uint32_t *>(&lo);
-                q.y = *reinterpret_cast<uint32_t *>(&hi);
-                *reinterpret_cast<uint2 *>(S.x + tc::core_offset(row, k, 128)) = q;
+            for (int step = 0; step < 8 && ok; step++) {
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    if (blockIdx.x + (2 * pair + q) * gridDim.x >= ntiles || !ok) continue;
+                    ok = tc::bar_wait(tc::smem_addr(&S.ready[q]), phase[q], A.budget);
+                    if (!ok) continue;
+                    phase[q] ^= 1u;
+                    tc::fence_after();
+                    if (!A.issue_mma) continue;
+                    const uint32_t op = tc::smem_addr(S.op[q]), d = tmem + kColD + 64u * q;
+                    if (step < 4) issue_forward(op, w, step, d);
+                    else issue_backward(op, w, 7 - step, tmem + kColW + 64u * (7 - step), d, pair > 0 || q > 0);
+                    tc::commit(tc::smem_addr(&S.done[q]));
+                    issued[q] = true;
+                }
             }
         }
-        // forward: layers 1-3 into H1..H3, layer 4 -> logits
-        float z[kN4];
+        // every commit but the last of each group was waited for by the group
+        // before it made the next step ready
+        for (int q = 0; q < 2; q++)
+            if (issued[q]) tc::bar_wait(tc::smem_addr(&S.done[q]), phase[q] ^ 1u, A.budget);
+        if (!ok) atomicOr(A.err, 1);
+    } else if (ok && g < 2) {
+        const uint32_t ready = tc::smem_addr(&S.ready[g]), done = tc::smem_addr(&S.done[g]);
+        uint8_t *op = S.op[g];
+        const uint32_t taddr = tmem + kColD + 64u * g + ((uint32_t)(warp * 32) << 16);     // this warp's lanes of D
+        uint32_t phase = 0;
+        // makes the operands just written (and D, if read) available to the
+        // issuing thread
+        auto hand_over = [&]() {
+            tc::fence_async_smem();
+            tc::fence_before();
+            tc::bar_arrive(ready);
+        };
+        // the group's MMAs of the step are complete; the same answer in every
+        // thread of the group, and a barrier of it
+        auto wait_done = [&]() {
+            ok = group_sync_and(g, tc::bar_wait(done, phase, A.budget));
+            phase ^= 1u;
+            tc::fence_after();
+            return ok;
+        };
 #pragma unroll 1
-        for (int l = 0; l < 4 && ok; l++) {
-            operands_ready();
-            const NetLayer L = net_layer(l);
-            const uint8_t *Ain = l == 0 ? S.x : S.h[l - 1];
-            if (t == 0 && A.issue_mma) {
-                issue_mma(tc::smem_addr(Ain), 128, tc::smem_addr(S.w) + L.b_off, L.N, L.K, tmem + kColD, false);
-                tc::commit(bar_m);
+        for (long long tile = blockIdx.x + (long long)g * gridDim.x; ok && tile < ntiles; tile += 2ll * gridDim.x) {
+            const long long r0 = tile * 128;
+            const int nvalid = (int)min((long long)128, A.n - r0);
+            const bool valid = t < nvalid;
+            // the group's next tile (features and targets) into L2
+            const long long nt = tile + 2ll * gridDim.x;
+            if (t == 0 && nt < ntiles) {
+                const long long nrows = min((long long)128, A.n - nt * 128);
+                tc::prefetch_l2(A.feat + nt * 128 * kFeat, (uint32_t)(nrows * kFeat * sizeof(float)));
+                tc::prefetch_l2(A.target + nt * 128 * kOutUsed, (uint32_t)((nrows * kOutUsed * sizeof(float)) & ~15ull));
             }
-            ok = train_sync_mma(A, bar_m, phase);
-            if (!ok) {
-                mma_waited_out = true;
-                break;
+            // features: coalesced float4 loads of the contiguous tile, all in
+            // flight at once -> BF16
+            {
+                const float4 *src = reinterpret_cast<const float4 *>(A.feat + r0 * kFeat);
+                constexpr int kLoads = 128 * kFeat / 4 / 128;
+                float4 v[kLoads];
+#pragma unroll
+                for (int i = 0; i < kLoads; i++) {
+                    const int e = i * 128 + t;
+                    v[i] = e / (kFeat / 4) < nvalid ? __ldg(src + e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+#pragma unroll
+                for (int i = 0; i < kLoads; i++) {
+                    const int e = i * 128 + t, row = e / (kFeat / 4), k = (e % (kFeat / 4)) * 4;
+                    __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x, v[i].y), hi = __floats2bfloat162_rn(v[i].z, v[i].w);
+                    uint2 q;
+                    q.x = *reinterpret_cast<uint32_t *>(&lo);
+                    q.y = *reinterpret_cast<uint32_t *>(&hi);
+                    *reinterpret_cast<uint2 *>(op + kChX * kChunkBytes + tc::core_offset(row, k, 128)) = q;
+                }
             }
-            if (l < 3) {
-                store_hidden<true>(S.h[l], taddr + kColD, S.bias + l * kHid, t);
-            } else {
+            hand_over();
+            // forward: layers 1-3 into H1..H3
+#pragma unroll 1
+            for (int l = 0; l < 3; l++) {
+                if (!wait_done()) break;
+                store_hidden<true>(op + input_chunk(l + 1) * kChunkBytes, taddr, S.bias + l * kHid, t);
+                hand_over();
+            }
+            if (!ok) break;
+            // while layer 4 runs: this warp's targets, read coalesced and turned
+            // through the dZ4 operand's memory (2 KB per warp, free until dZ4 is
+            // written after the group's next barrier) in two passes of 17 columns
+            float y[kOutUsed + 1];
+            {
+                float *stage = reinterpret_cast<float *>(op + kChDz4 * kChunkBytes) + warp * (32 * 17);
+                const float *src = A.target + (r0 + warp * 32) * kOutUsed;
+                const int rows = max(0, min(32, nvalid - warp * 32));
+#pragma unroll
+                for (int half = 0; half < 2; half++) {
+                    const int c0 = 17 * half, nc = half ? 16 : 17;
+                    float v[17];
+#pragma unroll
+                    for (int i = 0; i < 17; i++) {
+                        const int e = i * 32 + lane, row = e / nc, c = e % nc;
+                        v[i] = i < nc && row < rows ? __ldg(src + row * kOutUsed + c0 + c) : 0.0f;
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 17; i++) {
+                        const int e = i * 32 + lane;
+                        if (i < nc) stage[(e / nc) * 17 + e % nc] = v[i];
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 17; c++) y[c0 + c] = c < nc ? stage[lane * 17 + c] : 0.0f;
+                }
+            }
+            if (!wait_done()) break;
+            // loss per ray: w KL(q || p) + (T^ - T)^2, q = bins / w, w = sum(bins):
+            // w q (log q - log p) = y (log y - log w - log p); dZ4 = dL/dz / n with
+            // w (p - q) = w p - y
+            {
+                float dz[kN4];
                 float v[64];
-                tc::tmem_ld64(taddr + kColD, v);       // the 48 used of the 64 D columns, one round trip
+                tc::tmem_ld64(taddr, v);               // the 48 used of the 64 D columns, one round trip
 #pragma unroll
-                for (int j = 0; j < kN4; j++) z[j] = v[j] + S.bias[3 * kHid + j];
-            }
-        }
-        if (!ok) break;
-        // loss per ray: w KL(q || p) + (T^ - T)^2, q = bins / w, w = sum(bins);
-        // dZ4 = dL/dz scaled by 1/n
-        float dz[kHid];
-        float loss = 0.0f;
+                for (int j = 0; j < kN4; j++) dz[j] = v[j] + S.bias[3 * kHid + j];
+                float loss = 0.0f, mx = dz[0], W = 0.0f, se = 0.0f;
 #pragma unroll
-        for (int j = 0; j < kN4; j++) dz[j] = 0.0f;
-        if (valid) {
-            const float *y = A.target + r * kOutUsed;
-            float mx = z[0], W = 0.0f;
-#pragma unroll
-            for (int b = 0; b < kBins; b++) {
-                mx = fmaxf(mx, z[b]);
-                W += y[b];
-            }
-            float se = 0.0f;
-#pragma unroll
-            for (int b = 0; b < kBins; b++) se += expf(z[b] - mx);
-            const float lse = mx + logf(se);
-#pragma unroll
-            for (int b = 0; b < kBins; b++) {
-                const float p = expf(z[b] - lse);
-                if (W > 0.0f) {
-                    const float q = y[b] / W;
-                    dz[b] = W * (p - q) * A.inv_n;
-                    if (q > 0.0f) loss += W * q * (logf(q) - (z[b] - lse));
+                for (int b = 0; b < kBins; b++) {
+                    mx = fmaxf(mx, dz[b]);
+                    W += y[b];
                 }
+#pragma unroll
+                for (int b = 0; b < kBins; b++) {
+                    v[b] = expf(dz[b] - mx);
+                    se += v[b];
+                }
+                const float lse = mx + logf(se), wp = W / se, lw = W > 0.0f ? logf(W) : 0.0f;
+#pragma unroll
+                for (int b = 0; b < kBins; b++) {
+                    if (W > 0.0f && y[b] > 0.0f) loss += y[b] * ((logf(y[b]) - lw) - (dz[b] - lse));
+                    dz[b] = W > 0.0f && valid ? (wp * v[b] - y[b]) * A.inv_n : 0.0f;
+                }
+                const float th = 1.0f / (1.0f + expf(-dz[kBins]));
+                const float dt = th - y[kBins];
+                loss += dt * dt;
+                dz[kBins] = valid ? 2.0f * dt * th * (1.0f - th) * A.inv_n : 0.0f;
+#pragma unroll
+                for (int j = kOutUsed; j < kN4; j++) dz[j] = 0.0f;
+                if (valid) loss_sum += loss;
+                put_dz(op + kChDz4 * kChunkBytes, dz, t);
             }
-            const float th = 1.0f / (1.0f + expf(-z[kBins]));
-            const float dt = th - y[kBins];
-            loss += dt * dt;
-            dz[kBins] = 2.0f * dt * th * (1.0f - th) * A.inv_n;
-        }
-        loss_sum += loss;
-        // backward, layer 4 .. 1
+            hand_over();
+            // backward: dZ_l = dH_l * [H_l > 0] over H_l, layers 3..1
 #pragma unroll 1
-        for (int l = 3; l >= 0 && ok; l--) {
-            const int n_out = l == 3 ? kN4 : kHid;
-            put_dz(S, dz, l == 3 ? kOut : kHid, n_out, t);
-            operands_ready();
-            const uint32_t wcol = l == 3 ? kColW4 : l == 2 ? kColW3 : l == 1 ? kColW2 : kColW1;
-            if (t == 0 && A.issue_mma) {
-                issue_mma_mn(tc::smem_addr(l == 0 ? S.x : S.h[l - 1]), tc::smem_addr(S.adz), n_out, tmem + wcol, !first);
-                if (l > 0) {
-                    const uint32_t bb = l == 3 ? kUmmaB4 : l == 2 ? kUmmaB3 : kUmmaB2;
-                    issue_mma(tc::smem_addr(S.adz), 128, tc::smem_addr(S.w) + bb, kHid, n_out, tmem + kColD, false);
-                }
-                tc::commit(bar_m);
-            }
-            ok = train_sync_mma(A, bar_m, phase);
-            if (!ok) {
-                mma_waited_out = true;
-                break;
-            }
-            if (l > 0) {
-                // dZ_{l-1} = dH * [H_{l-1} > 0]
+            for (int l = 3; l > 0; l--) {
+                if (!wait_done()) break;
+                uint8_t *H = op + input_chunk(l) * kChunkBytes;
                 float v[kHid];
-                tc::tmem_ld64(taddr + kColD, v);
+                tc::tmem_ld64(taddr, v);
 #pragma unroll
-                for (int j = 0; j < kHid; j++) dz[j] = get_bf16(S.h[l - 1], t, j, 128) > 0.0f ? v[j] : 0.0f;
+                for (int j0 = 0; j0 < kHid; j0 += 8) {
+                    const uint4 q = *reinterpret_cast<const uint4 *>(H + tc::core_offset(t, j0, 128));
+                    const uint32_t h[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {          // a ReLU output is positive unless its bits are zero
+                        if ((h[i] & 0x7FFFu) == 0u) v[j0 + 2 * i] = 0.0f;
+                        if ((h[i] & 0x7FFF0000u) == 0u) v[j0 + 2 * i + 1] = 0.0f;
+                    }
+                }
+                put_dz(H, v, t);
+                hand_over();
             }
+            // the last step reads X and dZ1, which the next tile overwrites
+            if (!ok || !wait_done()) break;
         }
-        first = false;
+        if (!ok && t == 0) atomicOr(A.err, 1);
     }
-    if (!ok) {
-        if (t == 0) atomicOr(A.err, 1);
-        if (mma_waited_out && A.issue_mma) tc::bar_wait(bar_m, phase, A.budget);
-    }
-    // the CTA's gradient: lane = input row (or the bias at row n_in), column = output
-    float *part = A.partial + (size_t)blockIdx.x * kParams;
-    const int row = warp * 32 + lane;
+    // the CTA's gradient: accumulator row = input (or the bias), column = output;
+    // group 0 reads layers 1 and 2, group 1 layers 3 and 4
+    tc::fence_before();
+    ok = __syncthreads_and(ok);
+    tc::fence_after();
+    if (g < 2) {
+        float *part = A.partial + (size_t)blockIdx.x * kParams;
+        const int acc_row = warp * 32 + lane;
 #pragma unroll 1
-    for (int l = 0; l < 4; l++) {
-        const int n_in = l == 0 ? kFeat : kHid, n_out = l == 3 ? kOut : kHid, n_cols = l == 3 ? kN4 : kHid;
-        const uint32_t wcol = l == 3 ? kColW4 : l == 2 ? kColW3 : l == 1 ? kColW2 : kColW1;
-        const int offW = l == 0 ? kOffW1 : l == 1 ? kOffW2 : l == 2 ? kOffW3 : kOffW4;
-        const int offB = l == 0 ? kOffB1 : l == 1 ? kOffB2 : l == 2 ? kOffB3 : kOffB4;
-        for (int c = 0; c < n_cols; c += 16) {
-            float v[16];
-            tc::tmem_ld16(taddr + wcol + c, v);
-            for (int j = 0; j < 16 && c + j < n_out; j++) {
-                const float g = (first || !ok) ? 0.0f : v[j];
-                if (row < n_in) part[offW + row * n_out + c + j] = g;
-                else if (row == n_in) part[offB + c + j] = g;
-            }
+        for (int l = 2 * g; l < 2 * g + 2; l++) {
+            const int n_in = l == 0 ? kFeat : kHid, n_out = l == 3 ? kOut : kHid;
+            const int offW = l == 0 ? kOffW1 : l == 1 ? kOffW2 : l == 2 ? kOffW3 : kOffW4;
+            const int offB = l == 0 ? kOffB1 : l == 1 ? kOffB2 : l == 2 ? kOffB3 : kOffB4;
+            const int row = acc_row - grad_row0(l);
+            float *dst = acc_row == bias_row(l) ? part + offB : row >= 0 && row < n_in ? part + offW + row * n_out : nullptr;
+            float v[kHid];
+            tc::tmem_ld64(tmem + kColW + 64u * l + ((uint32_t)(warp * 32) << 16), v);
+            if (!dst) continue;
+#pragma unroll
+            for (int c = 0; c < kHid; c += 4)
+                if (c < n_out)
+                    *reinterpret_cast<float4 *>(dst + c) =
+                        ok ? make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
+        // loss: per-warp sums in a fixed order, then the CTA's
+        for (int o = 16; o > 0; o >>= 1) loss_sum += __shfl_xor_sync(0xffffffffu, loss_sum, o);
+        if (lane == 0) S.wloss[4 * g + warp] = loss_sum;
     }
-    // loss: per-warp sums in a fixed order, then the CTA's
-    for (int o = 16; o > 0; o >>= 1) loss_sum += __shfl_xor_sync(0xffffffffu, loss_sum, o);
-    if (lane == 0) S.wloss[warp] = loss_sum;
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (t == 0) A.loss_partial[blockIdx.x] = ((S.wloss[0] + S.wloss[1]) + S.wloss[2]) + S.wloss[3];
-    if (warp == 0) tc::tmem_free<kTrainCols>(tmem);
+    if (tid == 0) {
+        float sum = S.wloss[0];
+        for (int i = 1; i < 8; i++) sum += S.wloss[i];
+        A.loss_partial[blockIdx.x] = sum;
+    }
+    if (tid < 32) tc::tmem_free<kTrainCols>(tmem);
 }
 
-__global__ void reduce_grad_kernel(const float *partial, const float *loss_partial, int nblocks, float inv_n,
-                                   float *grad, float *loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kParams) {
-        float s = 0.0f;
-        for (int b = 0; b < nblocks; b++) s += partial[(size_t)b * kParams + i];
-        grad[i] = s;
+// Byte of parameter i's BF16 copy in the packed B operands (element (n, k) of
+// layer l is W_l[k][n], core-matrix layout), or -1 for a bias.
+__device__ __forceinline__ int operand_offset(int i) {
+    int off, nw, N;
+    unsigned base;
+    if (i < kOffB1) { off = i; nw = N = kHid; base = kUmmaL1; }
+    else if (i < kOffW2) return -1;
+    else if (i < kOffB2) { off = i - kOffW2; nw = N = kHid; base = kUmmaL2; }
+    else if (i < kOffW3) return -1;
+    else if (i < kOffB3) { off = i - kOffW3; nw = N = kHid; base = kUmmaL3; }
+    else if (i < kOffW4) return -1;
+    else if (i < kOffB4) { off = i - kOffW4; nw = kOut; N = kN4; base = kUmmaL4; }
+    else return -1;
+    return (int)(base + tc::core_offset(off % nw, off / nw, N));
+}
+
+// Sums the CTAs' partials: 32 parameters per block, eight threads on each
+// (every eighth partial, then a fixed order), so that the loads are whole lines
+// and eight chains of them run side by side (152 partials: 12.5 us with one
+// thread per parameter, RC_REDUCE_US). STEP: the Adam update (beta1 0.9, beta2
+// 0.999, eps 1e-8) of the FP32 parameters and their BF16 operands follows in
+// the same thread.
+template <bool STEP>
+__global__ void __launch_bounds__(256) reduce_grad_kernel(const float *partial, const float *loss_partial, int nblocks,
+                                                          float inv_n, float *grad, float *loss, AdamArgs P) {
+    __shared__ float s_sum[8][32];
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    float s = 0.0f;
+    if (i < kParams)
+        for (int b = seg; b < nblocks; b += 8) s += partial[(size_t)b * kParams + i];
+    s_sum[seg][lane] = s;
+    __syncthreads();
+    if (seg == 0 && i < kParams) {
+        float gi = s_sum[0][lane];
+#pragma unroll
+        for (int q = 1; q < 8; q++) gi += s_sum[q][lane];
+        grad[i] = gi;
+        if (STEP) {
+            const float mi = 0.9f * P.m[i] + 0.1f * gi;
+            const float vi = 0.999f * P.v[i] + 0.001f * gi * gi;
+            P.m[i] = mi;
+            P.v[i] = vi;
+            const float pi = P.params[i] - P.lr * (mi / P.c1) / (sqrtf(vi / P.c2) + 1e-8f);
+            P.params[i] = pi;
+            const int o = operand_offset(i);
+            if (o >= 0) *reinterpret_cast<__nv_bfloat16 *>(P.umma + o) = __float2bfloat16_rn(pi);
+        }
     }
-    if (i == 0 && loss) {
-        float s = 0.0f;
-        for (int b = 0; b < nblocks; b++) s += loss_partial[b];
-        *loss = s * inv_n;
+    if (loss && blockIdx.x == 0 && seg == 1) {
+        float q = 0.0f;
+        for (int b = lane; b < nblocks; b += 32) q += loss_partial[b];
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) *loss = q * inv_n;
     }
 }
 
@@ -1114,34 +1228,16 @@ int train_grid(long long n) {
     return (int)max(1ll, min((long long)sms, tiles));
 }
 
-cudaError_t launch_train_grad(const TrainArgs &a, int grid, float *grad, float *loss, cudaStream_t s) {
+cudaError_t launch_train_grad(const TrainArgs &a, int grid, float *grad, float *loss, const AdamArgs *step, cudaStream_t s) {
     const int smem = (int)sizeof(TrainSmem);
     cudaError_t e = cudaFuncSetAttribute(tc_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    tc_train_kernel<<<grid, 128, smem, s>>>(a);
+    tc_train_kernel<<<grid, kTrainThreads, smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    reduce_grad_kernel<<<(kParams + 255) / 256, 256, 0, s>>>(a.partial, a.loss_partial, grid, a.inv_n, grad, loss);
-    return cudaGetLastError();
-}
-
-// Adam (beta1 0.9, beta2 0.999, eps 1e-8) on the FP32 master parameters.
-__global__ void adam_kernel(float *p, float *m, float *v, const float *g, float lr, float c1, float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kParams) return;
-    const float gi = g[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi;
-    const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
-}
-
-cudaError_t launch_adam(float *params, float *m, float *v, const float *grad, long long step, float lr,
-                        cudaStream_t s) {
-    const float c1 = (float)(1.0 - pow(0.9, (double)step));
-    const float c2 = (float)(1.0 - pow(0.999, (double)step));
-    adam_kernel<<<(kParams + 255) / 256, 256, 0, s>>>(params, m, v, grad, lr, c1, c2);
+    const int blocks = (kParams + 31) / 32;
+    if (step) reduce_grad_kernel<true><<<blocks, 256, 0, s>>>(a.partial, a.loss_partial, grid, a.inv_n, grad, loss, *step);
+    else reduce_grad_kernel<false><<<blocks, 256, 0, s>>>(a.partial, a.loss_partial, grid, a.inv_n, grad, loss, AdamArgs{});
     return cudaGetLastError();
 }
 
@@ -1162,30 +1258,9 @@ __global__ void pack_umma_kernel(const float *params, uint8_t *umma) {
     *reinterpret_cast<__nv_bfloat16 *>(umma + boff + tc::core_offset(n, k, N)) = __float2bfloat16_rn(w);
 }
 
-// B operands of the training backward: element (n, k) of layer l is
-// bf16(W_l[n][k]) (inputs x outputs, as stored; 0 for the padding outputs
-// k >= 40 of layer 4).
-__global__ void pack_umma_back_kernel(const float *params, uint8_t *umma) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    constexpr int n4 = kHid * kN4, n3 = kHid * kHid;
-    if (idx >= n4 + 2 * n3) return;
-    int r, K, nw, woff;
-    unsigned boff;
-    if (idx < n4) { r = idx; K = kN4; nw = kOut; woff = kOffW4; boff = kUmmaB4; }
-    else if (idx < n4 + n3) { r = idx - n4; K = kHid; nw = kHid; woff = kOffW3; boff = kUmmaB3; }
-    else { r = idx - n4 - n3; K = kHid; nw = kHid; woff = kOffW2; boff = kUmmaB2; }
-    const int n = r / K, k = r % K;
-    const float w = k < nw ? params[woff + n * nw + k] : 0.0f;
-    *reinterpret_cast<__nv_bfloat16 *>(umma + boff + tc::core_offset(n, k, kHid)) = __float2bfloat16_rn(w);
-}
-
 cudaError_t launch_pack(const float *params, uint8_t *umma, cudaStream_t s) {
     constexpr int total = kHid * kFeat + 2 * kHid * kHid + kN4 * kHid;
     pack_umma_kernel<<<(total + 255) / 256, 256, 0, s>>>(params, umma);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    constexpr int back = kHid * kN4 + 2 * kHid * kHid;
-    pack_umma_back_kernel<<<(back + 255) / 256, 256, 0, s>>>(params, umma);
     return cudaGetLastError();
 }
 
