@@ -841,9 +841,12 @@ __global__ void __launch_bounds__(128) importance_kernel(const ImportanceArgs A)
 // All operands BF16 (dZ rounded once), FP32 accumulation.
 //
 // Bound: the chain of eight dependent MMA steps per tile with the threads' work
-// between them. 1048576 rays 746 us with one group of 128 threads per SM that
-// issued for itself and kept 128-column operands, RC_TRAIN_US now (131 us at the
-// issue rate, 90 us at the copy rate for the features and targets).
+// between them (the loss is the longest stretch). 1048576 rays 746 us with one
+// group of 128 threads per SM that issued for itself and kept 128-column
+// operands, 421 with two groups, 388 with the input gradient committed before
+// the weight gradient and the targets fetched under the forward (features and
+// targets: 90 us at the copy rate). Fetching the next tile's features under the
+// backward as well: 384, and 1.5 us more for a batch of 8192.
 constexpr int kChX = 0, kChOne0 = 14, kChH1 = 15, kChH2 = 23, kChOne1 = 31, kChH3 = 32, kChDz4 = 40, kChunks = 46;
 constexpr int kChunkBytes = 2048;
 constexpr int kTrainThreads = 2 * kGroupThreads + 32;      // two groups and the issuing warp
@@ -852,7 +855,7 @@ struct TrainSmem {
     uint8_t w[kUmmaBytes];                 // the four layers' weight operands
     float bias[3 * kHid + kN4];
     float wloss[8];
-    unsigned long long bar_w, ready[2], done[2];
+    unsigned long long bar_w, ready[2], done[2], done_w[2];
     uint32_t tmem;
 };
 constexpr int kTrainCols = 512;
@@ -866,8 +869,7 @@ __device__ __forceinline__ int grad_chunk(int l) { return l == 0 ? kChX : l == 1
 __device__ __forceinline__ int grad_row0(int l) { return l == 1 || l == 3 ? 8 : 0; }
 __device__ __forceinline__ int bias_row(int l) { return l == 0 ? kFeat : l == 2 ? kHid : 0; }
 
-// One layer of the forward: D = A W^T, or of the backward: the weight gradient
-// into its accumulator, then (l > 0) the input gradient into D; with a commit.
+// One layer of the forward: D = A W^T.
 __device__ __forceinline__ void issue_forward(uint32_t op, uint32_t w, int l, uint32_t tmem_d) {
     const NetLayer L = net_layer(l);
     const uint32_t a0 = op + input_chunk(l) * kChunkBytes, b0 = w + L.b_off, lbo_b = (uint32_t)(L.N / 8) * 128;
@@ -877,20 +879,25 @@ __device__ __forceinline__ void issue_forward(uint32_t op, uint32_t w, int l, ui
                      tc::smem_desc(b0 + ks * 2 * lbo_b, lbo_b, 128), idesc, ks > 0);
 }
 
+// Backward of layer l: the input gradient first (the group works on it while
+// the weight gradient runs), each with its own commit.
 __device__ __forceinline__ void issue_backward(uint32_t op, uint32_t w, int l, uint32_t tmem_w, uint32_t tmem_d,
-                                               bool accumulate) {
+                                               bool accumulate, uint32_t done, uint32_t done_w) {
     const NetLayer L = net_layer(l);
     const uint32_t dz = op + (l == 3 ? kChDz4 : input_chunk(l + 1)) * kChunkBytes;
     const uint32_t a0 = op + grad_chunk(l) * kChunkBytes;
+    if (l > 0) {
+        const uint32_t id_d = tc::idesc_bf16_f32(128, kHid) | tc::kIdescMnMajorB;
+        for (int ks = 0; ks < L.N / 16; ks++)  // 16 outputs each
+            tc::mma_bf16(tmem_d, tc::smem_desc(dz + ks * 2 * kChunkBytes, kChunkBytes, 128),
+                         tc::smem_desc(w + L.b_off + ks * 256, 128, (uint32_t)(L.N / 8) * 128), id_d, ks > 0);
+        tc::commit(done);
+    }
     const uint32_t id_w = tc::idesc_bf16_f32(128, L.N) | tc::kIdescMnMajorA | tc::kIdescMnMajorB;
-    for (int ks = 0; ks < 8; ks++)         // 16 rays each
+    for (int ks = 0; ks < 8; ks++)             // 16 rays each
         tc::mma_bf16(tmem_w, tc::smem_desc(a0 + ks * 256, 128, kChunkBytes), tc::smem_desc(dz + ks * 256, 128, kChunkBytes),
                      id_w, accumulate || ks > 0);
-    if (l == 0) return;
-    const uint32_t id_d = tc::idesc_bf16_f32(128, kHid) | tc::kIdescMnMajorB;
-    for (int ks = 0; ks < L.N / 16; ks++)  // 16 outputs each
-        tc::mma_bf16(tmem_d, tc::smem_desc(dz + ks * 2 * kChunkBytes, kChunkBytes, 128),
-                     tc::smem_desc(w + L.b_off + ks * 256, 128, (uint32_t)(L.N / 8) * 128), id_d, ks > 0);
+    tc::commit(done_w);
 }
 
 // dZ of this thread's ray (N values, zeros up to a multiple of 8) as row t of a
@@ -921,6 +928,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
         for (int i = 0; i < 2; i++) {
             tc::bar_init(tc::smem_addr(&S.ready[i]), kGroupThreads);
             tc::bar_init(tc::smem_addr(&S.done[i]), 1);
+            tc::bar_init(tc::smem_addr(&S.done_w[i]), 1);
         }
     }
     for (int i = tid; i < 3 * kHid + kN4; i += blockDim.x) {
@@ -949,7 +957,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
         // ones, for the tiles i = 2 pair + group of this CTA
         const uint32_t w = tc::smem_addr(S.w);
         uint32_t phase[2] = {0u, 0u};
-        bool issued[2] = {false, false};
+        int issued[2] = {-1, -1};                    // last step issued
+        uint32_t tiles_done[2] = {0u, 0u};
         for (long long pair = 0; ok && blockIdx.x + 2 * pair * gridDim.x < ntiles; pair++) {
 #pragma unroll 1
             for (int step = 0; step < 8 && ok; step++) {
@@ -961,24 +970,35 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                     phase[q] ^= 1u;
                     tc::fence_after();
                     if (!A.issue_mma) continue;
+                    if (step == 0 && issued[q] == 7) tiles_done[q]++;
                     const uint32_t op = tc::smem_addr(S.op[q]), d = tmem + kColD + 64u * q;
-                    if (step < 4) issue_forward(op, w, step, d);
-                    else issue_backward(op, w, 7 - step, tmem + kColW + 64u * (7 - step), d, pair > 0 || q > 0);
-                    tc::commit(tc::smem_addr(&S.done[q]));
-                    issued[q] = true;
+                    const uint32_t done = tc::smem_addr(&S.done[q]);
+                    if (step < 4) {
+                        issue_forward(op, w, step, d);
+                        tc::commit(done);
+                    } else {
+                        issue_backward(op, w, 7 - step, tmem + kColW + 64u * (7 - step), d, pair > 0 || q > 0, done,
+                                       tc::smem_addr(&S.done_w[q]));
+                    }
+                    issued[q] = step;
                 }
             }
         }
-        // every commit but the last of each group was waited for by the group
-        // before it made the next step ready
-        for (int q = 0; q < 2; q++)
-            if (issued[q]) tc::bar_wait(tc::smem_addr(&S.done[q]), phase[q] ^ 1u, A.budget);
+        // every commit but the last step's was waited for by the group before it
+        // made the next step ready; wait (bounded) for those still in flight.
+        // Steps 0-6 of a tile commit to `done` (7 per tile), 4-7 to `done_w` (4).
+        for (int q = 0; q < 2; q++) {
+            const uint32_t n = tiles_done[q] * 7u + (uint32_t)min(issued[q] + 1, 7);
+            const uint32_t nw = tiles_done[q] * 4u + (uint32_t)max(issued[q] - 3, 0);
+            if (n) tc::bar_wait(tc::smem_addr(&S.done[q]), (n - 1u) & 1u, A.budget);
+            if (nw) tc::bar_wait(tc::smem_addr(&S.done_w[q]), (nw - 1u) & 1u, A.budget);
+        }
         if (!ok) atomicOr(A.err, 1);
     } else if (ok && g < 2) {
-        const uint32_t ready = tc::smem_addr(&S.ready[g]), done = tc::smem_addr(&S.done[g]);
+        const uint32_t ready = tc::smem_addr(&S.ready[g]), done = tc::smem_addr(&S.done[g]), done_w = tc::smem_addr(&S.done_w[g]);
         uint8_t *op = S.op[g];
         const uint32_t taddr = tmem + kColD + 64u * g + ((uint32_t)(warp * 32) << 16);     // this warp's lanes of D
-        uint32_t phase = 0;
+        uint32_t phase = 0, phase_w = 0;
         // makes the operands just written (and D, if read) available to the
         // issuing thread
         auto hand_over = [&]() {
@@ -992,6 +1012,11 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
             ok = group_sync_and(g, tc::bar_wait(done, phase, A.budget));
             phase ^= 1u;
             tc::fence_after();
+            return ok;
+        };
+        auto wait_done_w = [&]() {
+            ok = group_sync_and(g, tc::bar_wait(done_w, phase_w, A.budget));
+            phase_w ^= 1u;
             return ok;
         };
 #pragma unroll 1
@@ -1028,6 +1053,18 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                 }
             }
             hand_over();
+            // this warp's targets, 17 and 16 columns of its 32 rows, in flight
+            // under the forward
+            float yc[kOutUsed];
+            {
+                const float *src = A.target + (r0 + warp * 32) * kOutUsed;
+                const int rows = max(0, min(32, nvalid - warp * 32));
+#pragma unroll
+                for (int i = 0; i < kOutUsed; i++) {
+                    const int nc = i < 17 ? 17 : 16, e = (i < 17 ? i : i - 17) * 32 + lane, row = e / nc;
+                    yc[i] = row < rows ? __ldg(src + row * kOutUsed + (i < 17 ? 0 : 17) + e % nc) : 0.0f;
+                }
+            }
             // forward: layers 1-3 into H1..H3
 #pragma unroll 1
             for (int l = 0; l < 3; l++) {
@@ -1036,32 +1073,25 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                 hand_over();
             }
             if (!ok) break;
-            // while layer 4 runs: this warp's targets, read coalesced and turned
-            // through the dZ4 operand's memory (2 KB per warp, free until dZ4 is
-            // written after the group's next barrier) in two passes of 17 columns
+            // while layer 4 runs: the targets turned from the coalesced order to
+            // one ray per lane, through the dZ4 operand's memory (2 KB per warp,
+            // free until dZ4 is written after the group's next barrier), 17
+            // columns at a time
             float y[kOutUsed + 1];
             {
                 float *stage = reinterpret_cast<float *>(op + kChDz4 * kChunkBytes) + warp * (32 * 17);
-                const float *src = A.target + (r0 + warp * 32) * kOutUsed;
-                const int rows = max(0, min(32, nvalid - warp * 32));
 #pragma unroll
                 for (int half = 0; half < 2; half++) {
-                    const int c0 = 17 * half, nc = half ? 16 : 17;
-                    float v[17];
-#pragma unroll
-                    for (int i = 0; i < 17; i++) {
-                        const int e = i * 32 + lane, row = e / nc, c = e % nc;
-                        v[i] = i < nc && row < rows ? __ldg(src + row * kOutUsed + c0 + c) : 0.0f;
-                    }
+                    const int nc = half ? 16 : 17;
                     __syncwarp();
 #pragma unroll
-                    for (int i = 0; i < 17; i++) {
+                    for (int i = 0; i < nc; i++) {
                         const int e = i * 32 + lane;
-                        if (i < nc) stage[(e / nc) * 17 + e % nc] = v[i];
+                        stage[(e / nc) * 17 + e % nc] = yc[17 * half + i];
                     }
                     __syncwarp();
 #pragma unroll
-                    for (int c = 0; c < 17; c++) y[c0 + c] = c < nc ? stage[lane * 17 + c] : 0.0f;
+                    for (int c = 0; c < 17; c++) y[17 * half + c] = c < nc ? stage[lane * 17 + c] : 0.0f;
                 }
             }
             if (!wait_done()) break;
@@ -1074,7 +1104,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                 tc::tmem_ld64(taddr, v);               // the 48 used of the 64 D columns, one round trip
 #pragma unroll
                 for (int j = 0; j < kN4; j++) dz[j] = v[j] + S.bias[3 * kHid + j];
-                float loss = 0.0f, mx = dz[0], W = 0.0f, se = 0.0f;
+                float kl = 0.0f, mx = dz[0], W = 0.0f, se = 0.0f;
 #pragma unroll
                 for (int b = 0; b < kBins; b++) {
                     mx = fmaxf(mx, dz[b]);
@@ -1088,12 +1118,12 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                 const float lse = mx + logf(se), wp = W / se, lw = W > 0.0f ? logf(W) : 0.0f;
 #pragma unroll
                 for (int b = 0; b < kBins; b++) {
-                    if (W > 0.0f && y[b] > 0.0f) loss += y[b] * ((logf(y[b]) - lw) - (dz[b] - lse));
+                    kl += fmaxf(y[b], 0.0f) * ((logf(fmaxf(y[b], 1e-37f)) - lw) - (dz[b] - lse));     // 0 where y is 0
                     dz[b] = W > 0.0f && valid ? (wp * v[b] - y[b]) * A.inv_n : 0.0f;
                 }
                 const float th = 1.0f / (1.0f + expf(-dz[kBins]));
                 const float dt = th - y[kBins];
-                loss += dt * dt;
+                const float loss = (W > 0.0f ? kl : 0.0f) + dt * dt;
                 dz[kBins] = valid ? 2.0f * dt * th * (1.0f - th) * A.inv_n : 0.0f;
 #pragma unroll
                 for (int j = kOutUsed; j < kN4; j++) dz[j] = 0.0f;
@@ -1118,11 +1148,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) tc_train_kernel(const TrainA
                         if ((h[i] & 0x7FFF0000u) == 0u) v[j0 + 2 * i + 1] = 0.0f;
                     }
                 }
+                // the weight gradient of layer l + 1 reads H_l
+                if (!wait_done_w()) break;
                 put_dz(H, v, t);
                 hand_over();
             }
             // the last step reads X and dZ1, which the next tile overwrites
-            if (!ok || !wait_done()) break;
+            if (!ok || !wait_done_w()) break;
         }
         if (!ok && t == 0) atomicOr(A.err, 1);
     }
@@ -1183,10 +1215,10 @@ __device__ __forceinline__ int operand_offset(int i) {
 
 // Sums the CTAs' partials: 32 parameters per block, eight threads on each
 // (every eighth partial, then a fixed order), so that the loads are whole lines
-// and eight chains of them run side by side (152 partials: 12.5 us with one
-// thread per parameter, RC_REDUCE_US). STEP: the Adam update (beta1 0.9, beta2
-// 0.999, eps 1e-8) of the FP32 parameters and their BF16 operands follows in
-// the same thread.
+// and eight chains of them run side by side (one thread per parameter took
+// 12.5 us for 152 partials). STEP: the Adam update (beta1 0.9, beta2 0.999, eps
+// 1e-8) of the FP32 parameters and their BF16 operands follows in the same
+// thread (a training step of 8192 rays 60 -> 25 us with the gradient kernel).
 template <bool STEP>
 __global__ void __launch_bounds__(256) reduce_grad_kernel(const float *partial, const float *loss_partial, int nblocks,
                                                           float inv_n, float *grad, float *loss, AdamArgs P) {
