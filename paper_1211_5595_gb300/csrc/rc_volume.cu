@@ -61,6 +61,28 @@ struct PrepArgs {
     uint16_t *mn, *mx, *mn4, *mx4;
 };
 
+// Local coordinates of element e = threadIdx.x + k * 256 of an E^3 box, carried
+// from one k to the next without divisions.
+template <int E>
+struct BoxWalk {
+    int x, y, z;
+    __device__ __forceinline__ explicit BoxWalk(int e) : x(e % E), y(e / E % E), z(e / (E * E)) {}
+    __device__ __forceinline__ void next() {
+        constexpr int sx = 256 % E, sy = 256 / E;              // sy < E: 256 < E * E
+        static_assert(256 < E * E, "one carry per axis");
+        x += sx;
+        y += sy;
+        if (x >= E) { x -= E; y++; }
+        if (y >= E) { y -= E; z++; }
+    }
+};
+
+// Bound by the bytes written (349 MB moved per 256x256x180 FP32 upload, 51 us at
+// the copy rate) once the index arithmetic is out of the way: 102 us with a
+// division per element and axis, neighbour clamps per difference and the grids
+// reduced in separate passes (97 M warp instructions, issue 75%), 61 us now; whole
+// uploads with the copy into the staging buffer, us: 256x256x180 FP32 112 -> 72,
+// 512x512x256 uint16 526 -> 290, 64x64x32 FP32 19 -> 13.
 template <int ST>
 __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
     __shared__ uint16_t s_code[kApronVox];
@@ -70,82 +92,65 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
               bz = (int)(b / ((unsigned)A.cb[0] * (unsigned)A.cb[1]));
     const int x0 = bx * kBrick - 1, y0 = by * kBrick - 1, z0 = bz * kBrick - 1;     // box origin
     const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
+    const float inv_o = 1.0f / (float)A.f16o;        // o is a power of two: the product is the quotient
     // box codes, and the apron brick from them
-    for (unsigned e = threadIdx.x; e < (unsigned)kApronVox; e += blockDim.x) {
-        const int lx = (int)(e % kApron), ly = (int)((e / kApron) % kApron), lz = (int)(e / (kApron * kApron));
-        const int x = min(max(x0 + lx, 0), nx - 1), y = min(max(y0 + ly, 0), ny - 1), z = min(max(z0 + lz, 0), nz - 1);
-        const int code = min((int)A.stage[((size_t)z * ny + y) * nx + x], A.vmax);
-        s_code[e] = (uint16_t)code;
-        const size_t o = (size_t)b * kApronVox + e;
-        if (ST == RC_STORE_F32) ((float *)A.apron)[o] = (float)code;
-        else if (ST == RC_STORE_F16)
-            ((__half *)A.apron)[o] = __float2half_rn(__fdiv_rn((float)(code - A.f16o), (float)A.f16o));
-        else ((uint16_t *)A.apron)[o] = (uint16_t)code;
+    {
+        BoxWalk<kApron> w(threadIdx.x);
+        constexpr int kPer = (kApronVox + 255) / 256, kBatch = 9;
+        static_assert(kPer % kBatch == 0, "whole batches of loads");
+#pragma unroll 1
+        for (int k0 = 0; k0 < kPer; k0 += kBatch) {
+            int code[kBatch];
+#pragma unroll
+            for (int k = 0; k < kBatch; k++) {
+                const int x = min(max(x0 + w.x, 0), nx - 1), y = min(max(y0 + w.y, 0), ny - 1),
+                          z = min(max(z0 + w.z, 0), nz - 1);
+                // fewer than 2^31 voxels (19^3 stored ones per brick are)
+                code[k] = w.z < kApron ? min((int)__ldg(A.stage + ((unsigned)(z * ny + y) * (unsigned)nx + (unsigned)x)), A.vmax) : 0;
+                w.next();
+            }
+#pragma unroll
+            for (int k = 0; k < kBatch; k++) {
+                const unsigned e = threadIdx.x + (unsigned)(k0 + k) * 256u;
+                if (e >= (unsigned)kApronVox) break;
+                s_code[e] = (uint16_t)code[k];
+                const size_t o = (size_t)b * kApronVox + e;
+                if (ST == RC_STORE_F32) ((float *)A.apron)[o] = (float)code[k];
+                else if (ST == RC_STORE_F16)
+                    ((__half *)A.apron)[o] = __float2half_rn((float)(code[k] - A.f16o) * inv_o);
+                else ((uint16_t *)A.apron)[o] = (uint16_t)code[k];
+            }
+        }
     }
     __syncthreads();
-    // the code at volume coordinate (x, y, z) inside the box
-    auto at = [&](int x, int y, int z) {
-        return (int)s_code[((z - z0) * kApron + (y - y0)) * kApron + (x - x0)];
-    };
     if (A.vg != nullptr) {
-        for (unsigned e = threadIdx.x; e < (unsigned)kGradVox; e += blockDim.x) {
-            const int lx = (int)(e % kGradEdge), ly = (int)((e / kGradEdge) % kGradEdge),
-                      lz = (int)(e / (kGradEdge * kGradEdge));
-            const int x = min(bx * kBrick + lx, nx - 1), y = min(by * kBrick + ly, ny - 1),
-                      z = min(bz * kBrick + lz, nz - 1);
-            const int V = at(x, y, z);
-            const int dx = at(min(x + 1, nx - 1), y, z) - at(max(x - 1, 0), y, z);
-            const int dy = at(x, min(y + 1, ny - 1), z) - at(x, max(y - 1, 0), z);
-            const int dz = at(x, y, min(z + 1, nz - 1)) - at(x, y, max(z - 1, 0));
+        BoxWalk<kGradEdge> w(threadIdx.x);
+        // last voxel of the volume in the brick's own coordinates
+        const int mx = nx - 1 - bx * kBrick, my = ny - 1 - by * kBrick, mz = nz - 1 - bz * kBrick;
+        for (unsigned e = threadIdx.x; e < (unsigned)kGradVox; e += 256u, w.next()) {
+            // the box's replicated border voxels are the clamped neighbours
+            const uint16_t *c = s_code + ((min(w.z, mz) + 1) * kApron + (min(w.y, my) + 1)) * kApron + (min(w.x, mx) + 1);
+            const int V = c[0];
+            const int dx = (int)c[1] - (int)c[-1], dy = (int)c[kApron] - (int)c[-kApron],
+                      dz = (int)c[kApron * kApron] - (int)c[-kApron * kApron];
+            const size_t o = (size_t)b * kGradVox + e;
             if (ST == RC_STORE_F32) {
-                reinterpret_cast<float4 *>(A.vg)[(size_t)b * kGradVox + e] =
-                    make_float4((float)V, (float)dx, (float)dy, (float)dz);
-            } else if (ST == RC_STORE_F16) {
-                // the apron brick's value of this voxel, h = fp16((V - o) / o)
-                const __half h = __float2half_rn(__fdiv_rn((float)(V - A.f16o), (float)A.f16o));
-                reinterpret_cast<uint2 *>(A.vg)[(size_t)b * kGradVox + e] =
-                    make_uint2((unsigned)__half_as_ushort(h) | ((unsigned)(dx + 32768) << 16),
-                               (unsigned)(dy + 32768) | ((unsigned)(dz + 32768) << 16));
+                reinterpret_cast<float4 *>(A.vg)[o] = make_float4((float)V, (float)dx, (float)dy, (float)dz);
             } else {
-                // codes <= 65535 and differences in (-32768, 32768): 16-bit fields
-                reinterpret_cast<uint2 *>(A.vg)[(size_t)b * kGradVox + e] =
-                    make_uint2((unsigned)V | ((unsigned)(dx + 32768) << 16),
-                               (unsigned)(dy + 32768) | ((unsigned)(dz + 32768) << 16));
+                // uint16: the code; FP16: the apron brick's value of this voxel,
+                // h = fp16((V - o) / o). Codes <= 65535 and differences in
+                // (-32768, 32768): 16-bit fields
+                const unsigned v = ST == RC_STORE_F16
+                                       ? (unsigned)__half_as_ushort(__float2half_rn((float)(V - A.f16o) * inv_o))
+                                       : (unsigned)V;
+                reinterpret_cast<uint2 *>(A.vg)[o] =
+                    make_uint2(v | ((unsigned)(dx + 32768) << 16), (unsigned)(dy + 32768) | ((unsigned)(dz + 32768) << 16));
             }
-        }
-    }
-    // cell-brick min / max over voxels max(16b, 0) .. min(16b + 16, N - 1)
-    {
-        const int xa = bx * kBrick, ya = by * kBrick, za = bz * kBrick;
-        const int ex = min(xa + 16, nx - 1) - xa + 1, ey = min(ya + 16, ny - 1) - ya + 1,
-                  ez = min(za + 16, nz - 1) - za + 1;
-        int lo = 65535, hi = 0;
-        for (int row = threadIdx.x; row < ey * ez; row += blockDim.x) {      // rows (y, z), then along x
-            const int y = ya + row % ey, z = za + row / ey;
-            for (int x = xa; x < xa + ex; x++) {
-                const int v = at(x, y, z);
-                lo = min(lo, v);
-                hi = max(hi, v);
-            }
-        }
-        lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)lo);
-        hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)hi);
-        if ((threadIdx.x & 31) == 0) {
-            s_lo[threadIdx.x >> 5] = lo;
-            s_hi[threadIdx.x >> 5] = hi;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-                lo = min(lo, s_lo[w]);
-                hi = max(hi, s_hi[w]);
-            }
-            A.mn[b] = (uint16_t)lo;
-            A.mx[b] = (uint16_t)hi;
         }
     }
     // the 4^3 sub-blocks j = 4b + s of the brick, four threads each, over
-    // voxels 4j .. min(4j + 4, N - 1)
+    // voxels 4j .. min(4j + 4, N - 1); the brick's own min / max (voxels 16b ..
+    // min(16b + 16, N - 1)) is theirs together
     {
         const int sb = threadIdx.x >> 2, q = threadIdx.x & 3;               // sub-block 0..63, quarter
         const int sx = sb & 3, sy = (sb >> 2) & 3, sz = sb >> 4;
@@ -153,15 +158,15 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
         const bool exists = jx < A.c4[0] && jy < A.c4[1] && jz < A.c4[2];
         int lo = 65535, hi = 0;
         if (exists) {
-            const int xa = 4 * jx, ya = 4 * jy, za = 4 * jz;
-            const int ex = min(xa + 4, nx - 1) - xa + 1, ey = min(ya + 4, ny - 1) - ya + 1,
-                      ez = min(za + 4, nz - 1) - za + 1;
-            for (int row = q; row < ey * ez; row += 4) {                      // rows (y, z), then along x
-                const int y = ya + row % ey, z = za + row / ey;
-                for (int x = xa; x < xa + ex; x++) {
-                    const int v = at(x, y, z);
-                    lo = min(lo, v);
-                    hi = max(hi, v);
+            // a footprint cut by the volume's far side continues in the box's
+            // replicated border voxels: the same values again
+            const uint16_t *c = s_code + ((4 * sz + 1) * kApron + (4 * sy + 1)) * kApron + 4 * sx + 1;
+            for (int row = q; row < 25; row += 4) {                          // rows (y, z), then along x
+                const uint16_t *r = c + (row / 5) * (kApron * kApron) + (row % 5) * kApron;
+#pragma unroll
+                for (int i = 0; i < 5; i++) {
+                    lo = min(lo, (int)r[i]);
+                    hi = max(hi, (int)r[i]);
                 }
             }
         }
@@ -171,9 +176,24 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
         lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
         hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, 2));
         if (exists && q == 0) {
-            const size_t j = ((size_t)jz * A.c4[1] + jy) * A.c4[0] + jx;
+            const unsigned j = ((unsigned)jz * A.c4[1] + jy) * A.c4[0] + jx;
             A.mn4[j] = (uint16_t)lo;
             A.mx4[j] = (uint16_t)hi;
+        }
+        lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)lo);
+        hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)hi);
+        if ((threadIdx.x & 31) == 0) {
+            s_lo[threadIdx.x >> 5] = lo;
+            s_hi[threadIdx.x >> 5] = hi;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < 8; w++) {
+                lo = min(lo, s_lo[w]);
+                hi = max(hi, s_hi[w]);
+            }
+            A.mn[b] = (uint16_t)lo;
+            A.mx[b] = (uint16_t)hi;
         }
     }
 }
