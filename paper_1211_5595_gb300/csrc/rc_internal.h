@@ -14,10 +14,12 @@ constexpr int kApron = 19;          // stored brick edge: cells 16b-1 .. 16b+17 
 constexpr int kApronVox = kApron * kApron * kApron;   // 6859
 constexpr int kGradEdge = 17;       // value+gradient brick edge: voxels 16b .. 16b+16 (the trilinear footprint)
 constexpr int kGradVox = kGradEdge * kGradEdge * kGradEdge;   // 4913
-// Pair bricks: per cell-brick the apron rows (lz, ly in 0..18) as 18
-// entries (V[16b-1+e], V[16b+e]), e = 0..17, in the storage type (two
-// elements, aligned to their size), so two x-adjacent voxels of any footprint
-// row arrive in one load.
+// Pair bricks: per cell-brick pairs of adjacent voxels in the storage type (two
+// elements, aligned to their size), so that two voxels of a footprint arrive in
+// one load. FP16: the apron rows (lz, ly in 0..18) as 18 entries
+// (V[16b-1+e], V[16b+e]) along x, e = 0..17. FP32 (the B-spline only): pairs
+// along y, entry ((lz * 18 + ly) * 19 + lx) = voxels ly and ly + 1 at lx, ly in
+// 0..17, lz and lx in 0..18.
 constexpr int kPairRow = 18;
 constexpr int kPairVox = kApron * kApron * kPairRow;          // 6498
 

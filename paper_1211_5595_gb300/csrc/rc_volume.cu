@@ -6,27 +6,33 @@
 
 namespace rc {
 
-// One thread per entry of the pair bricks: entry (lz, ly, e) of brick b is
-// the apron elements e and e + 1 of row (ly, lz), copied bit for bit (so the
-// pairs hold exactly the stored values of every storage type).
-template <typename T>
+// One thread per entry of the pair bricks, copied bit for bit from the apron
+// bricks (so the pairs hold exactly the stored values of every storage type):
+// pairs along x (ALONG_Y false; 16-bit types) or along y (FP32).
+template <typename T, bool ALONG_Y>
 __global__ void pairs_kernel(const T *__restrict__ apron, T *__restrict__ dst, long long total) {
     const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;     // fewer than 2^31 entries
     if ((long long)e >= total) return;
     const unsigned local = e % (unsigned)kPairVox, brick = e / (unsigned)kPairVox;
-    const unsigned ex = local % kPairRow, row = local / kPairRow;     // row = lz * 19 + ly
-    const T *src = apron + (size_t)brick * kApronVox + row * kApron + ex;
-    dst[2 * e] = src[0];
-    dst[2 * e + 1] = src[1];
+    unsigned at;
+    if (ALONG_Y) {
+        const unsigned lx = local % kApron, r = local / kApron;           // r = lz * 18 + ly
+        at = ((r / kPairRow) * kApron + r % kPairRow) * kApron + lx;
+    } else {
+        at = (local / kPairRow) * kApron + local % kPairRow;              // row lz * 19 + ly
+    }
+    const T *src = apron + (size_t)brick * kApronVox + at;
+    struct alignas(2 * sizeof(T)) Two { T a, b; };
+    reinterpret_cast<Two *>(dst)[e] = Two{src[0], src[ALONG_Y ? kApron : 1]};
 }
 
 cudaError_t launch_pairs(VolDev v, void *dst, cudaStream_t s) {
     const long long total = (long long)v.cb[0] * v.cb[1] * v.cb[2] * kPairVox;
     const unsigned blocks = (unsigned)((total + 255) / 256);
     if (v.storage == RC_STORE_F32)
-        pairs_kernel<float><<<blocks, 256, 0, s>>>((const float *)v.data, (float *)dst, total);
+        pairs_kernel<float, true><<<blocks, 256, 0, s>>>((const float *)v.data, (float *)dst, total);
     else
-        pairs_kernel<uint16_t><<<blocks, 256, 0, s>>>((const uint16_t *)v.data, (uint16_t *)dst, total);
+        pairs_kernel<uint16_t, false><<<blocks, 256, 0, s>>>((const uint16_t *)v.data, (uint16_t *)dst, total);
     return cudaGetLastError();
 }
 
