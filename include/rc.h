@@ -155,8 +155,8 @@ rc_status rc_context_destroy(rc_context *ctx);
  * grid over the cell-bricks (footprint voxels 16b..min(16b+16, N-1)). FP32
  * storage, uint16 storage with vmax < 32768 and FP16 storage with
  * vmax <= 4096 also hold value+gradient bricks (each voxel's stored value and
- * the central differences of its codes: 16 bytes per voxel for FP32, 8 for
- * the others) that shaded and 2-D-table samples read. */
+ * the central differences of its codes: 8 bytes per voxel, 16 for FP32
+ * storage with vmax >= 32768) that shaded and 2-D-table samples read. */
 rc_status rc_volume_create(rc_context *ctx, int nx, int ny, int nz,
                            float sx, float sy, float sz, uint16_t vmax,
                            rc_storage storage, rc_volume **out);

@@ -292,8 +292,10 @@ __device__ __forceinline__ void gradient_tile(const AdjointArgs &A, const float4
             position_at(R, sample_t(R, k), p);
             Cell c;
             cell_of(a.vol, p, c);
-            if (CUBIC) val = GRAD ? bspline_grad<ST>(a.vol, c, gr) : bspline<ST>(a.vol, c);
-            else val = GRAD ? value_grad<ST>(a.vol, c, gr) : trilinear<ST>(a.vol, c);
+            if constexpr (CUBIC && GRAD) val = bspline_grad<ST>(a.vol, c, gr);
+            else if constexpr (CUBIC) val = bspline<ST>(a.vol, c);
+            else if constexpr (GRAD) val = value_grad<ST>(a.vol, c, gr);
+            else val = trilinear<ST>(a.vol, c);
             float w, wb = 0.0f;
             float4 e;
             if (TF2) {
@@ -516,26 +518,22 @@ static cudaError_t launch_adj2(Kern kern, const AdjointArgs &a, int nviews, cons
 // and reconstruction filter.
 template <int RM, bool CUBIC>
 static cudaError_t launch_adj_rm(const AdjointArgs &a, int nviews, const float *absmax, cudaStream_t s) {
-    switch (a.m.vol.storage * 2 + (a.m.p.shade ? 1 : 0)) {
-        case RC_STORE_F32 * 2: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_F32, false, RM, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F32 * 2 + 1: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_F32, true, RM, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F16 * 2: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_F16, false, RM, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F16 * 2 + 1: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_F16, true, RM, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_U16 * 2: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_U16, false, RM, CUBIC>, a, nviews, absmax, s);
-        default: return launch_adj<CUBIC>(adjoint_kernel<RC_STORE_U16, true, RM, CUBIC>, a, nviews, absmax, s);
-    }
+    if (a.m.p.shade)
+        return by_storage<!CUBIC>(a.m.vol, [&](auto st) {
+            return launch_adj<CUBIC>(adjoint_kernel<decltype(st)::value, true, RM, CUBIC>, a, nviews, absmax, s);
+        });
+    return by_storage<false>(a.m.vol, [&](auto st) {
+        return launch_adj<CUBIC>(adjoint_kernel<decltype(st)::value, false, RM, CUBIC>, a, nviews, absmax, s);
+    });
 }
 
 template <bool CUBIC>
 static cudaError_t launch_adj_tf2(const AdjointArgs &a, int nviews, const float *absmax, cudaStream_t s) {
-    switch (a.m.vol.storage * 2 + (a.m.p.shade ? 1 : 0)) {
-        case RC_STORE_F32 * 2: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_F32, false, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F32 * 2 + 1: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_F32, true, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F16 * 2: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_F16, false, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_F16 * 2 + 1: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_F16, true, CUBIC>, a, nviews, absmax, s);
-        case RC_STORE_U16 * 2: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_U16, false, CUBIC>, a, nviews, absmax, s);
-        default: return launch_adj2<CUBIC>(adjoint2_kernel<RC_STORE_U16, true, CUBIC>, a, nviews, absmax, s);
-    }
+    return by_storage<!CUBIC>(a.m.vol, [&](auto st) {
+        constexpr int ST = decltype(st)::value;
+        return a.m.p.shade ? launch_adj2<CUBIC>(adjoint2_kernel<ST, true, CUBIC>, a, nviews, absmax, s)
+                           : launch_adj2<CUBIC>(adjoint2_kernel<ST, false, CUBIC>, a, nviews, absmax, s);
+    });
 }
 
 // 1-D tables: one instance per opacity-correction mode; 2-D tables: the mode

@@ -314,6 +314,11 @@ static void volume_free(rc_volume *v) {
     }
 }
 
+static size_t vg_entry_bytes(const rc_volume *v) {
+    if (v->storage == RC_STORE_F16 ? v->vmax <= 4096 : v->vmax < 32768) return sizeof(uint2);
+    return v->storage == RC_STORE_F32 ? sizeof(float4) : 0;
+}
+
 rc_status rc_volume_create(rc_context *ctx, int nx, int ny, int nz, float sx, float sy, float sz, uint16_t vmax,
                            rc_storage storage, rc_volume **out) {
     if (!ctx) return fail(nullptr, RC_ERR_INVALID_ARG, "rc_volume_create: ctx is NULL");
@@ -342,14 +347,12 @@ rc_status rc_volume_create(rc_context *ctx, int nx, int ny, int nz, float sx, fl
     v->nbricks = v->cb[0] * v->cb[1] * v->cb[2];
     size_t esz = storage == RC_STORE_F32 ? 4 : 2;
     size_t nvox = (size_t)nx * ny * nz;
-    // value+gradient bricks: FP32 storage; uint16 storage while the central
-    // differences fit 16 bits (vmax < 32768); FP16 storage while every stored
-    // value is exact (vmax <= 4096: offset o <= 2048), so that the differences
-    // of stored values are integer code differences / o
-    const size_t vg_bytes = storage == RC_STORE_F32 ? (size_t)v->nbricks * kGradVox * sizeof(float4)
-                            : (storage == RC_STORE_U16 && vmax < 32768) || (storage == RC_STORE_F16 && vmax <= 4096)
-                                ? (size_t)v->nbricks * kGradVox * sizeof(uint2)
-                                : 0;
+    // value+gradient bricks: 8-byte entries while the central differences fit
+    // 16 bits (vmax < 32768; FP16 storage while every stored value is exact,
+    // vmax <= 4096: offset o <= 2048, so that the differences of stored values
+    // are integer code differences / o); FP32 storage of wider codes 16-byte ones
+    const size_t entry = vg_entry_bytes(v);
+    const size_t vg_bytes = (size_t)v->nbricks * kGradVox * entry;
     const size_t n4 = (size_t)((nx - 1 + 3) / 4) * ((ny - 1 + 3) / 4) * ((nz - 1 + 3) / 4);
     if (dev_alloc(&v->d_data, (size_t)padded * esz) != cudaSuccess ||
         (vg_bytes && dev_alloc(&v->d_vg, vg_bytes) != cudaSuccess) ||
@@ -394,6 +397,7 @@ static VolDev vol_dev(const rc_volume *v) {
     VolDev d;
     d.data = v->d_data;
     d.vg = v->d_vg;
+    d.vg16 = vg_entry_bytes(v) == sizeof(uint2);
     d.pairs = v->pairs_data_version == v->data_version ? v->d_pairs : nullptr;
     d.storage = (int)v->storage;
     float smin = fminf(fminf(v->s[0], v->s[1]), v->s[2]);

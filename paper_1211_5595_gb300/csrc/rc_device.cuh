@@ -140,8 +140,34 @@ __device__ __forceinline__ unsigned cell_address(const VolDev &v, const Cell &c)
     return b * (unsigned)kApronVox + (lz * kApron + ly) * kApron + lx;
 }
 
+// Kernel instances are by storage (ST = rc_storage). An instance whose form
+// reads gradients expects 8-byte value+gradient entries; a volume without them
+// (codes too wide) takes the instance ST | kNoVg16. Choosing at launch instead
+// of per sample keeps the unused path's registers out of the march (12 shaded
+// views of 256x256x180 at 1024^2: 2.55 ms against 2.79 with the branch).
+constexpr int kNoVg16 = 4;
+template <int N> struct IntC { static constexpr int value = N; };
+
+// go(IntC<ST>) with the instance for volume v; GRAD: the form reads
+// value+gradient entries.
+template <bool GRAD, typename Go>
+static inline cudaError_t by_storage(const VolDev &v, Go go) {
+    if constexpr (GRAD) {
+        if (!v.vg16) switch (v.storage) {
+            case RC_STORE_F32: return go(IntC<RC_STORE_F32 | kNoVg16>{});
+            case RC_STORE_F16: return go(IntC<RC_STORE_F16 | kNoVg16>{});
+            default: return go(IntC<RC_STORE_U16 | kNoVg16>{});
+        }
+    }
+    switch (v.storage) {
+        case RC_STORE_F32: return go(IntC<RC_STORE_F32>{});
+        case RC_STORE_F16: return go(IntC<RC_STORE_F16>{});
+        default: return go(IntC<RC_STORE_U16>{});
+    }
+}
+
 // Element type of each storage.
-template <int ST> struct Voxel;
+template <int ST> struct Voxel : Voxel<(ST & 3)> {};
 template <> struct Voxel<RC_STORE_F32> { using T = float; };
 template <> struct Voxel<RC_STORE_F16> { using T = __half; };
 template <> struct Voxel<RC_STORE_U16> { using T = unsigned short; };
@@ -157,8 +183,8 @@ __device__ __forceinline__ const typename Voxel<ST>::T *cell_ptr(const VolDev &v
 
 template <int ST>
 __device__ __forceinline__ float ldv(const typename Voxel<ST>::T *p) {
-    if (ST == RC_STORE_F32) return __ldg(reinterpret_cast<const float *>(p));
-    if (ST == RC_STORE_F16) return __half2float(__ldg(reinterpret_cast<const __half *>(p)));
+    if ((ST & 3) == RC_STORE_F32) return __ldg(reinterpret_cast<const float *>(p));
+    if ((ST & 3) == RC_STORE_F16) return __half2float(__ldg(reinterpret_cast<const __half *>(p)));
     return (float)__ldg(reinterpret_cast<const unsigned short *>(p));
 }
 
@@ -231,7 +257,7 @@ __device__ __forceinline__ float trilinear(const VolDev &v, const Cell &c) {
 }
 
 // Pair entries by storage: two stored elements, aligned to their size.
-template <int ST> struct Pair;
+template <int ST> struct Pair : Pair<(ST & 3)> {};
 template <> struct Pair<RC_STORE_F32> { using T = float2; };
 template <> struct Pair<RC_STORE_F16> { using T = __half2; };
 template <> struct Pair<RC_STORE_U16> { using T = ushort2; };
@@ -249,8 +275,8 @@ __device__ __forceinline__ const typename Pair<ST>::T *pair_ptr(const VolDev &v,
 // The two voxels of a pair entry as FP32 (the stored values converted as ldv does).
 template <int ST>
 __device__ __forceinline__ float2 ld_pair(const typename Pair<ST>::T *q) {
-    if constexpr (ST == RC_STORE_F32) return __ldg(q);
-    else if constexpr (ST == RC_STORE_F16) return __half22float2(__ldg(q));
+    if constexpr ((ST & 3) == RC_STORE_F32) return __ldg(q);
+    else if constexpr ((ST & 3) == RC_STORE_F16) return __half22float2(__ldg(q));
     else {
         const ushort2 u = __ldg(q);
         return make_float2((float)u.x, (float)u.y);
@@ -260,8 +286,8 @@ __device__ __forceinline__ float2 ld_pair(const typename Pair<ST>::T *q) {
 template <int OY, int OZ, int OX>
 constexpr int pair_off() { return (OZ * kApron + OY) * kPairRow + OX; }
 
-// Value and world-space gradient from the value+gradient bricks (FP32
-// storage): each voxel holds (V, D_x, D_y, D_z) with D_a = V(+1 along a) -
+// Value and world-space gradient from value+gradient bricks of float4 entries
+// (FP32 storage of codes beyond 15 bits): each voxel holds (V, D_x, D_y, D_z) with D_a = V(+1 along a) -
 // V(-1 along a), neighbour indices clamped to the volume, all exact integers.
 // Central differences of the trilinear field are linear in the voxels, so
 // (f(p + e_a) - f(p - e_a)) / 2 equals the trilinear interpolation of D_a / 2
@@ -317,9 +343,8 @@ __device__ __forceinline__ ulonglong2 vg16_lerp(uint2 qa, uint2 qb, unsigned lon
     return make_ulonglong2(r0, r1);
 }
 
-// value_grad_vg for uint16 storage: the same integers from 8-byte entries
-// (half the bytes of the float4 entries), so the same operations give the
-// FP32 storage's result bit for bit.
+// value_grad_vg from 8-byte entries of the same integers: the same operations
+// give the same result bit for bit.
 __device__ __forceinline__ float value_grad_vg16(const VolDev &v, const Cell &c, float g[3]) {
     const unsigned idx = (unsigned)brick_of(v, c) * (unsigned)kGradVox +
                          (unsigned)(((c.i[2] & 15) * kGradEdge + (c.i[1] & 15)) * kGradEdge + (c.i[0] & 15));
@@ -449,17 +474,28 @@ __device__ __forceinline__ float value_grad_x(const VolDev &v, const Cell &c, fl
     return val;
 }
 
-// Value and gradient of the trilinear field: FP32 storage from the
-// value+gradient bricks, uint16 from its 8-byte value+gradient bricks when
-// the volume has them (vmax < 32768); FP16 from the pair bricks when the
-// volume has them (one uniform branch per sample), else from the apron brick.
+// Value and gradient of the trilinear field from the value+gradient bricks'
+// 8-byte entries; without them (kNoVg16) from float4 entries (FP32 storage), the
+// pair bricks when built (FP16) or the apron brick. FP32 storage reads the same
+// entries as uint16: the same integers, so the same result, from half the L1
+// bytes of float4 entries (12 shaded views of 256x256x180 at 1024^2 2.61 -> 2.55
+// ms, 4 views with a 2-D table at 768^2 1.29 -> 1.16, 6 proposal views 0.90 ->
+// 0.86, and half the bytes to write per upload).
 template <int ST>
 __device__ __forceinline__ float value_grad(const VolDev &v, const Cell &c, float g[3]) {
-    if (ST == RC_STORE_F32) return value_grad_vg(v, c, g);
-    if (ST == RC_STORE_U16 && v.vg != nullptr) return value_grad_vg16(v, c, g);
-    if (ST == RC_STORE_F16 && v.vg != nullptr) return value_grad_vg16h(v, c, g);
-    if (ST == RC_STORE_F16 && v.pairs != nullptr) return value_grad_x<ST, true>(v, c, g);
-    return value_grad_x<ST, false>(v, c, g);
+    if constexpr (ST == RC_STORE_F32 || ST == RC_STORE_U16) return value_grad_vg16(v, c, g);
+    else if constexpr (ST == RC_STORE_F16) return value_grad_vg16h(v, c, g);
+    else if constexpr ((ST & 3) == RC_STORE_F32) return value_grad_vg(v, c, g);
+    else {
+        if ((ST & 3) == RC_STORE_F16 && v.pairs != nullptr) return value_grad_x<ST & 3, true>(v, c, g);
+        return value_grad_x<ST & 3, false>(v, c, g);
+    }
+}
+
+// The same chosen at run time, for kernels that need it once per ray.
+template <int ST>
+__device__ __forceinline__ float value_grad_any(const VolDev &v, const Cell &c, float g[3]) {
+    return v.vg16 ? value_grad<ST>(v, c, g) : value_grad<ST | kNoVg16>(v, c, g);
 }
 
 // Uniform cubic B-spline reconstruction (Sec. 3.2's higher-order filter):
@@ -669,7 +705,7 @@ __device__ __forceinline__ float bspline_grad(const VolDev &v, const Cell &c, fl
 // makes skipping exact.
 template <int ST>
 __device__ __forceinline__ float tf_coord(float val, float ucoef) {
-    if (ST == RC_STORE_F16) return __fmaf_rn(val, ucoef, ucoef);
+    if ((ST & 3) == RC_STORE_F16) return __fmaf_rn(val, ucoef, ucoef);
     return __fmul_rn(val, ucoef);
 }
 
@@ -794,11 +830,11 @@ __device__ __forceinline__ float4 eval_sample_x(const VolDev &vol, const MarchPa
     constexpr bool SHADE = (F & kShade) != 0, CUBIC = (F & kCubic) != 0, TF2 = (F & kTF2) != 0;
     constexpr bool GRAD = SHADE || TF2;
     float val, g[3];
-    if (CUBIC) {
-        if (GRAD) val = bspline_grad<ST>(vol, c, g);
+    if constexpr (CUBIC) {
+        if constexpr (GRAD) val = bspline_grad<ST>(vol, c, g);
         else val = bspline<ST>(vol, c);
     } else {
-        if (GRAD) val = value_grad<ST>(vol, c, g);
+        if constexpr (GRAD) val = value_grad<ST>(vol, c, g);
         else val = trilinear<ST>(vol, c);
     }
     float4 e;

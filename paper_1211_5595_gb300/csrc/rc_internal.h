@@ -13,7 +13,7 @@ constexpr int kBrick = 16;          // cell-brick edge (trilinear cells)
 constexpr int kApron = 19;          // stored brick edge: cells 16b-1 .. 16b+17 (edges replicated)
 constexpr int kApronVox = kApron * kApron * kApron;   // 6859
 constexpr int kGradEdge = 17;       // value+gradient brick edge: voxels 16b .. 16b+16 (the trilinear footprint)
-constexpr int kGradVox = kGradEdge * kGradEdge * kGradEdge;   // 4913
+constexpr int kGradVox = kGradEdge * kGradEdge * kGradEdge + 1;   // 4913 and one to keep bricks 16-byte aligned
 // Pair bricks: per cell-brick pairs of adjacent voxels in the storage type (two
 // elements, aligned to their size), so that two voxels of a footprint arrive in
 // one load. FP16: the apron rows (lz, ly in 0..18) as 18 entries
@@ -36,9 +36,11 @@ struct VolDev {
     const void *data;      // [bz][by][bx][19][19][19] apron bricks, storage type
     const void *pairs;     // pair bricks (storage type) once a render needed them, else null
     // value+gradient bricks [bz][by][bx][17][17][17] of (value, central
-    // differences x2): F32 storage float4 entries, U16 storage uint2 entries
-    // (value | (D_x + 32768) << 16, (D_y + 32768) | (D_z + 32768) << 16); F16: null
+    // differences x2), or null: uint2 entries (value | (D_x + 32768) << 16,
+    // (D_y + 32768) | (D_z + 32768) << 16) where vg16, else float4 (F32 storage
+    // of codes beyond 15 bits); F16 storage: the stored value's bits for the value
     const void *vg;
+    int vg16;
     int storage;           // rc_storage
     int n[3];              // voxels per axis
     int cb[3];             // cell-bricks per axis: ceil((n-1)/16)

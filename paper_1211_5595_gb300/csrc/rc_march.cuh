@@ -55,6 +55,8 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, unsigned de
 // - one sample at a time else.
 // Lanes leave the loop one by one: holding the warp together by a vote per
 // turn took uint16 at 512x512x256, 2048^2, from 1.37 to 1.45 ms.
+constexpr bool reads_gradients(int F) { return (F & (kShade | kTF2)) != 0 && !(F & kCubic); }
+
 enum : int { kTurnOne = 0, kTurnPair = 1, kTurnAhead = 2 };
 
 template <int ST, int F, int RM>
@@ -390,7 +392,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
             }
             float g[3], sf, spec;
             if (CUBIC) bspline_grad<ST>(a.vol, c, g);
-            else value_grad<ST>(a.vol, c, g);
+            else value_grad_any<ST>(a.vol, c, g);
             shade_factor(a.p, a.vol, g, R.dir, sf, spec);
             out = make_float4(ts, fminf(1.0f, sf + spec), (float)hit_k, 1.0f);
         }
@@ -442,8 +444,9 @@ static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool ta
 //   256x256x180, 512^2: 172 142 135 161 / 135 105 99 131
 //   256x256x180, 724^2: 223 201 214 293 / 150 143 162 235
 //   256x256x180, 1024^2: 292 307 386 572 / 193 229 287 456
-// Forms whose samples take longer (FP32 shading, B-spline, 2-D table) gain
-// further up than the plain and the 16-bit ones.
+// Forms whose samples take longer (shading without 8-byte value+gradient
+// entries, which the FP32 shaded figures above are for; B-spline; 2-D table) gain
+// further up than the others.
 static int lanes_per_ray(const MarchArgs &a, int nviews) {
     // the box's corners bound the part of the image whose rays can meet it;
     // its silhouette fills about two thirds of that rectangle
@@ -476,7 +479,7 @@ static int lanes_per_ray(const MarchArgs &a, int nviews) {
     for (int i = 0; i < 3; i++) diag2 += (double)(a.vol.n[i] - 1) * a.vol.s[i] * (a.vol.n[i] - 1) * a.vol.s[i];
     const double hits = 0.65 * part * c.W * c.H * nviews;
     const double steps = sqrt(diag2) / ((double)a.p.step_vox * a.vol.smin);
-    const bool heavy = (a.p.shade && a.vol.storage == RC_STORE_F32) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2;
+    const bool heavy = (a.p.shade && !a.vol.vg16) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2;
     if (hits <= (heavy ? 22e3 : 7e3) && hits <= 70.0 * steps) return 8;
     if (hits <= 76e3 && hits <= 190.0 * steps) return 4;
     if (hits <= 155e3 && hits <= (heavy ? 390.0 : 190.0) * steps) return 2;
@@ -487,11 +490,9 @@ template <int F, int L>
 static cudaError_t launch_wide(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = !(F & kTF2);
     constexpr int W = kWarpsX * WideTile<L>::X, H = kWarpsY * WideTile<L>::Y;
-    switch (a.vol.storage) {
-        case RC_STORE_F32: return launch_kernel(wide_kernel<RC_STORE_F32, F, L>, a, nviews, smem, s, W, H);
-        case RC_STORE_F16: return launch_kernel(wide_kernel<RC_STORE_F16, F, L>, a, nviews, smem, s, W, H);
-        default: return launch_kernel(wide_kernel<RC_STORE_U16, F, L>, a, nviews, smem, s, W, H);
-    }
+    return by_storage<reads_gradients(F)>(a.vol, [&](auto st) {
+        return launch_kernel(wide_kernel<decltype(st)::value, F, L>, a, nviews, smem, s, W, H);
+    });
 }
 
 // Composite march with sample form F and opacity-correction mode RM for the
@@ -499,11 +500,9 @@ static cudaError_t launch_wide(const MarchArgs &a, int nviews, cudaStream_t s) {
 template <int F, int RM>
 static cudaError_t launch_composite_rm(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = !(F & kTF2);
-    switch (a.vol.storage) {
-        case RC_STORE_F32: return launch_kernel(composite_kernel<RC_STORE_F32, F, RM>, a, nviews, smem, s);
-        case RC_STORE_F16: return launch_kernel(composite_kernel<RC_STORE_F16, F, RM>, a, nviews, smem, s);
-        default: return launch_kernel(composite_kernel<RC_STORE_U16, F, RM>, a, nviews, smem, s);
-    }
+    return by_storage<reads_gradients(F)>(a.vol, [&](auto st) {
+        return launch_kernel(composite_kernel<decltype(st)::value, F, RM>, a, nviews, smem, s);
+    });
 }
 
 // The step ratios of the fixed modes (1, 1/2, 1/4) get their own instances.
@@ -525,11 +524,9 @@ static cudaError_t launch_composite(const MarchArgs &a, int nviews, cudaStream_t
 template <bool CUBIC, int FN>
 static cudaError_t launch_function_group(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = a.p.func == RC_FUNC_THRESHOLD;
-    switch (a.vol.storage) {
-        case RC_STORE_F32: return launch_kernel(function_kernel<RC_STORE_F32, CUBIC, FN>, a, nviews, smem, s);
-        case RC_STORE_F16: return launch_kernel(function_kernel<RC_STORE_F16, CUBIC, FN>, a, nviews, smem, s);
-        default: return launch_kernel(function_kernel<RC_STORE_U16, CUBIC, FN>, a, nviews, smem, s);
-    }
+    return by_storage<false>(a.vol, [&](auto st) {
+        return launch_kernel(function_kernel<decltype(st)::value, CUBIC, FN>, a, nviews, smem, s);
+    });
 }
 
 template <bool CUBIC>

@@ -5,7 +5,7 @@
 // (the smallest brick index any of its rays needs) until every ray is done.
 // The per-sample arithmetic is composite_kernel's (the same loads' values,
 // the same operations), so the images are identical. It is an alternative
-// kept for measurement: the staging of a whole 78.6 KB brick serves only the
+// kept for measurement: the staging of a whole 39 KB brick serves only the
 // thin pencil of it that a 16 x 8 pixel tile's rays cross, so it moves far
 // more bytes than the cached gathers of composite_kernel.
 #include "rc_march.cuh"
@@ -13,19 +13,19 @@
 
 namespace rc {
 
-constexpr unsigned kStagedBytes = (unsigned)kGradVox * 16u;     // 78,608 B: one value+gradient brick
+constexpr unsigned kStagedBytes = (unsigned)kGradVox * 8u;      // 39,312 B: one value+gradient brick
 
-// value_grad_vg on a brick in shared memory (same loads' values, same order).
-__device__ __forceinline__ float value_grad_staged(const ulonglong2 *brick, const VolDev &v, const Cell &c,
+// value_grad_vg16 on a brick in shared memory (same loads' values, same order).
+__device__ __forceinline__ float value_grad_staged(const uint2 *brick, const VolDev &v, const Cell &c,
                                                    float g[3]) {
     const unsigned idx = (unsigned)(((c.i[2] & 15) * kGradEdge + (c.i[1] & 15)) * kGradEdge + (c.i[0] & 15));
-    const ulonglong2 *p = brick + idx;
+    const uint2 *p = brick + idx;
     constexpr int DY = kGradEdge, DZ = kGradEdge * kGradEdge;
     const unsigned long long wx = pack2(c.w[0], c.w[0]), wy = pack2(c.w[1], c.w[1]), wz = pack2(c.w[2], c.w[2]);
-    const ulonglong2 c00 = lerp4p(p[0], p[1], wx);
-    const ulonglong2 c10 = lerp4p(p[DY], p[DY + 1], wx);
-    const ulonglong2 c01 = lerp4p(p[DZ], p[DZ + 1], wx);
-    const ulonglong2 c11 = lerp4p(p[DZ + DY], p[DZ + DY + 1], wx);
+    const ulonglong2 c00 = vg16_lerp(p[0], p[1], wx);
+    const ulonglong2 c10 = vg16_lerp(p[DY], p[DY + 1], wx);
+    const ulonglong2 c01 = vg16_lerp(p[DZ], p[DZ + 1], wx);
+    const ulonglong2 c11 = vg16_lerp(p[DZ + DY], p[DZ + DY + 1], wx);
     const float4 r = unpack4(lerp4p(lerp4p(c00, c10, wy), lerp4p(c01, c11, wy), wz));
     g[0] = r.y * v.inv2s[0];
     g[1] = r.z * v.inv2s[1];
@@ -36,7 +36,7 @@ __device__ __forceinline__ float value_grad_staged(const ulonglong2 *brick, cons
 template <int RM>
 __global__ void __launch_bounds__(kMarchThreads) staged_kernel(const MarchArgs a, int *err, long long budget) {
     extern __shared__ __align__(128) uint8_t smem[];
-    const ulonglong2 *s_vg = reinterpret_cast<const ulonglong2 *>(smem);
+    const uint2 *s_vg = reinterpret_cast<const uint2 *>(smem);
     float4 *s_tf = reinterpret_cast<float4 *>(smem + kStagedBytes);
     __shared__ __align__(8) unsigned long long bar;
     __shared__ unsigned s_min[kWarpsX * kWarpsY];
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kMarchThreads) staged_kernel(const MarchArgs a
         if (bmin != staged) {
             if (threadIdx.x == 0) {
                 tc::fence_async_smem();
-                tc::bulk_g2s(tc::smem_addr(smem), reinterpret_cast<const float4 *>(vol.vg) + (size_t)bmin * kGradVox,
+                tc::bulk_g2s(tc::smem_addr(smem), reinterpret_cast<const uint2 *>(vol.vg) + (size_t)bmin * kGradVox,
                              kStagedBytes, bar_a);
             }
             const bool ok = __syncthreads_and(tc::bar_wait(bar_a, phase, budget));
@@ -133,10 +133,10 @@ __global__ void __launch_bounds__(kMarchThreads) staged_kernel(const MarchArgs a
     if (a.stats) add_stats(a.stats, (unsigned)min(k, nsamp), evald, hit ? 1u : 0u, inimg ? 1u : 0u);
 }
 
-// The staged march for FP32 storage, shaded, trilinear, 1-D table, compositing;
+// The staged march for FP32 storage (8-byte entries), shaded, trilinear, 1-D table, compositing;
 // false when the form is another (the caller then runs composite_kernel).
 bool staged_eligible(const MarchArgs &a) {
-    return a.vol.storage == RC_STORE_F32 && a.vol.vg != nullptr && a.p.shade && a.p.skip &&
+    return a.vol.storage == RC_STORE_F32 && a.vol.vg != nullptr && a.vol.vg16 && a.p.shade && a.p.skip &&
            a.p.func == RC_FUNC_COMPOSITE && a.p.filter == RC_FILTER_TRILINEAR && a.tf.M < 2 && a.batch == nullptr;
 }
 

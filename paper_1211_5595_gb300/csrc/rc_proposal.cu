@@ -1312,11 +1312,7 @@ cudaError_t launch_profiles(const MarchArgs &a, float *out, cudaStream_t s) {
         kern<<<grid, 128, smem, s>>>(a, out);
         return cudaGetLastError();
     };
-    switch (a.vol.storage) {
-        case RC_STORE_F32: return go(profiles_kernel<RC_STORE_F32>);
-        case RC_STORE_F16: return go(profiles_kernel<RC_STORE_F16>);
-        default: return go(profiles_kernel<RC_STORE_U16>);
-    }
+    return by_storage<false>(a.vol, [&](auto st) { return go(profiles_kernel<decltype(st)::value>); });
 }
 
 cudaError_t launch_features(const MarchArgs &a, float *out, cudaStream_t s) {
@@ -1384,14 +1380,9 @@ static cudaError_t launch_imp_st(const ImportanceArgs &a, int nviews, cudaStream
 }
 
 cudaError_t launch_importance(const ImportanceArgs &a, int nviews, cudaStream_t s) {
-    switch (a.m.vol.storage * 2 + (a.m.p.shade ? 1 : 0)) {
-        case RC_STORE_F32 * 2: return launch_imp_st<RC_STORE_F32, false>(a, nviews, s);
-        case RC_STORE_F32 * 2 + 1: return launch_imp_st<RC_STORE_F32, true>(a, nviews, s);
-        case RC_STORE_F16 * 2: return launch_imp_st<RC_STORE_F16, false>(a, nviews, s);
-        case RC_STORE_F16 * 2 + 1: return launch_imp_st<RC_STORE_F16, true>(a, nviews, s);
-        case RC_STORE_U16 * 2: return launch_imp_st<RC_STORE_U16, false>(a, nviews, s);
-        default: return launch_imp_st<RC_STORE_U16, true>(a, nviews, s);
-    }
+    if (a.m.p.shade)
+        return by_storage<true>(a.m.vol, [&](auto st) { return launch_imp_st<decltype(st)::value, true>(a, nviews, s); });
+    return by_storage<false>(a.m.vol, [&](auto st) { return launch_imp_st<decltype(st)::value, false>(a, nviews, s); });
 }
 
 }  // namespace rc

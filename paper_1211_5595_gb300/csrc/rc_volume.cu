@@ -47,9 +47,9 @@ cudaError_t launch_pairs(VolDev v, void *dst, cudaStream_t s) {
 //     h is exact), U16 the code;
 //   - the 17^3 value+gradient entries of voxels 16b .. 16b+16 (clamped) as
 //     (V, V(x+1) - V(x-1), V(y+1) - V(y-1), V(z+1) - V(z-1)) of the codes,
-//     neighbour indices clamped to the volume: exact in FP32 (float4) for
-//     FP32 storage; for uint16 as 16-bit fields with the differences offset
-//     by 32768 (uint2: V | Dx << 16, Dy | Dz << 16); for FP16 the same with
+//     neighbour indices clamped to the volume: 16-bit fields with the
+//     differences offset by 32768 (uint2: V | Dx << 16, Dy | Dz << 16), or
+//     float4 for FP32 storage of wider codes; for FP16 the uint2 form with
 //     the bits of the stored FP16 value h in place of V (the differences of
 //     stored values are the code differences / o, exactly, when o <= 2048);
 //   - the trilinear cell-brick min / max over voxels max(16b, 0) .. min(16b+16, N-1);
@@ -63,7 +63,8 @@ struct PrepArgs {
     int vmax;
     int f16o;                    // FP16 storage: the offset o
     void *apron;
-    void *vg;                    // float4 (FP32 storage), uint2 (uint16, FP16 storage) or null
+    void *vg;                    // uint2 entries (vg16), float4 entries or null
+    int vg16;
     uint16_t *mn, *mx, *mn4, *mx4;
 };
 
@@ -133,14 +134,14 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
         BoxWalk<kGradEdge> w(threadIdx.x);
         // last voxel of the volume in the brick's own coordinates
         const int mx = nx - 1 - bx * kBrick, my = ny - 1 - by * kBrick, mz = nz - 1 - bz * kBrick;
-        for (unsigned e = threadIdx.x; e < (unsigned)kGradVox; e += 256u, w.next()) {
+        for (unsigned e = threadIdx.x; e < (unsigned)(kGradEdge * kGradEdge * kGradEdge); e += 256u, w.next()) {
             // the box's replicated border voxels are the clamped neighbours
             const uint16_t *c = s_code + ((min(w.z, mz) + 1) * kApron + (min(w.y, my) + 1)) * kApron + (min(w.x, mx) + 1);
             const int V = c[0];
             const int dx = (int)c[1] - (int)c[-1], dy = (int)c[kApron] - (int)c[-kApron],
                       dz = (int)c[kApron * kApron] - (int)c[-kApron * kApron];
             const size_t o = (size_t)b * kGradVox + e;
-            if (ST == RC_STORE_F32) {
+            if (ST == RC_STORE_F32 && !A.vg16) {
                 reinterpret_cast<float4 *>(A.vg)[o] = make_float4((float)V, (float)dx, (float)dy, (float)dz);
             } else {
                 // uint16: the code; FP16: the apron brick's value of this voxel,
@@ -217,6 +218,7 @@ cudaError_t launch_prep(const uint16_t *stage, VolDev v, void *apron, void *vg, 
     a.f16o = (int)v.f16o;
     a.apron = apron;
     a.vg = vg;
+    a.vg16 = v.vg16;
     a.mn = mn;
     a.mx = mx;
     a.mn4 = mn4;

@@ -79,3 +79,56 @@ def test_lanes_per_ray_change_nothing(rc, storage, form, size, views):
                 assert st["evaluated_samples"] > 0
     finally:
         r.close()
+
+
+# Codes on both sides of the line where value+gradient entries take 8 bytes
+# (vmax 32767 | 32768): every form that reads gradients, against the oracle.
+@pytest.mark.parametrize("storage", ["F32", "U16"])
+@pytest.mark.parametrize("vmax", [32767, 32768, 65535])
+def test_gradient_forms_by_code_width(rc, orc, storage, vmax):
+    import torch
+    dims, spacing, gmax = (38, 33, 29), (1.0, 0.9, 1.3), 20000.0
+    n = dims[0] * dims[1] * dims[2]
+    u = synth.uniform01(5, np.arange(n)).reshape(dims[2], dims[1], dims[0])
+    ph = synth.head_phantom(dims, spacing, seed=12, tumor_radius_vox=3).vol.astype(np.float64)
+    vol = np.clip(ph * (vmax / 4095.0) + 0.02 * vmax * u, 0, vmax).astype(np.uint16)
+    vol[10, 10, 8:20] = vmax                         # full-scale steps: the largest differences
+    vol[10, 12, 8:20] = 0
+    cam = synth.orbit_camera(dims, spacing, 140.0, width=61, height=45)
+    r = GPURenderer(rc, vol, spacing, getattr(rc, "RC_STORE_" + storage), vmax)
+    try:
+        tab, tab2 = synth.tf_table(200, vmax=vmax), synth.tf2d_table(64, 8, gmax=gmax, vmax=vmax)
+        for tf, kw in ((tab, dict(shade=True)), (tab2, dict(shade=False)), (tab2, dict(shade=True))):
+            two = tf.ndim == 3
+            if two:
+                rc.rc_tf2d_set(r.ctx, tf, gmax)
+            else:
+                r.set_tf(tf)
+            sc = orc.Scene(vol, spacing, tf, cam, step=0.5, term=0.99, vmax=vmax, gmax=gmax if two else None, **kw)
+            o = orc.render(sc)
+            compare(r.render(cam, step_vox=0.5, term=0.99, **kw), o, TOL_FP32)
+            keep = np.nonzero(~o["tie"].reshape(-1))[0]
+            g = np.zeros((61 * 45, 4))
+            g[keep] = 1.0
+            want, _ = orc.render_grad(sc, g[keep], pixels=keep)
+            got = torch.empty(tf.shape, device="cuda")
+            rc.rc_render_backward(r.ctx, r.vol, rc.RenderParams(step_vox=0.5, term=0.99, **kw),
+                                  torch.from_numpy(g.astype(np.float32).reshape(45, 61, 4)).cuda(), got)
+            torch.cuda.synchronize()
+            assert np.abs(got.cpu().numpy() - want).max() / np.abs(want).max() < 2e-4
+        r.set_tf(tab)
+        img = r.render(cam, step_vox=0.5, term=0.99, shade=True, func=rc.RC_FUNC_ISO, iso=0.4 * vmax)
+        o = orc.render(orc.Scene(vol, spacing, tab, cam, step=0.5, term=0.99, shade=True, vmax=vmax, func=orc.ISO,
+                                 iso=0.4 * vmax))
+        a, b = img.reshape(-1, 4).astype(np.float64), o["rgba"].reshape(-1, 4)
+        same = (a[:, 3] == b[:, 3]) & (a[:, 2] == b[:, 2])
+        assert same.mean() > 0.99 and b[:, 3].sum() > 100
+        np.testing.assert_allclose(a[same][:, 1], b[same][:, 1], atol=2e-4)
+        # the importance march over the whole chord reads the same entries
+        out = torch.empty((1, 45, 61, 4), device="cuda")
+        rc.rc_render_importance_views(r.ctx, r.vol, rc.RenderParams(step_vox=0.5, term=0.99, shade=True), [cam],
+                                      rc.RC_SAMPLING_INVCDF, 1.0, None, None, 64, 2.0, out)
+        torch.cuda.synchronize()
+        assert torch.isfinite(out).all() and out[..., 3].max() > 0.2
+    finally:
+        r.close()
