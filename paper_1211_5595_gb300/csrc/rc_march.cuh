@@ -47,12 +47,13 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, unsigned de
 // sample's chain (level, voxels, table) behind both. One turn of the loop is
 // - two samples for the plain trilinear form, whose 8 loads leave registers
 //   for a second sample in flight (4 FP16 views of 181x217x157 at 901x703:
-//   0.342 -> 0.327 ms; with shading the registers cost more warps than the
-//   overlap gains: 2.63 -> 2.78 ms for 12 views of 256x256x180 at 1024^2);
+//   0.342 -> 0.327 ms; 4 shaded views of 256x256x180 at 1024^2 0.875 -> 0.905:
+//   there the registers cost more warps than the overlap gains);
 // - one sample with the next one's cell and level fetched under it for the
-//   shaded FP32 form (2.635 -> 2.612 ms; uint16 1.373 -> 1.422, B-spline
-//   1.725 -> 1.762);
-// - one sample at a time else.
+//   forms that read gradients from FP32 and uint16 volumes (shaded 0.916 ->
+//   0.875, 512x512x256 at 2048^2, step 1/4, 1.320 -> 1.283, 2-D table 1.813 ->
+//   1.774; FP16, with its longer decode, 0.892 -> 0.898 and 1.283 -> 1.310);
+// - one sample at a time else (B-spline 1.725 -> 1.762 with the fetch).
 // Lanes leave the loop one by one: holding the warp together by a vote per
 // turn took uint16 at 512x512x256, 2048^2, from 1.37 to 1.45 ms.
 constexpr bool reads_gradients(int F) { return (F & (kShade | kTF2)) != 0 && !(F & kCubic); }
@@ -61,7 +62,8 @@ enum : int { kTurnOne = 0, kTurnPair = 1, kTurnAhead = 2 };
 
 template <int ST, int F, int RM>
 __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArgs a) {
-    constexpr int kTurn = F == 0 ? kTurnPair : F == kShade && ST == RC_STORE_F32 ? kTurnAhead : kTurnOne;
+    constexpr int kTurn = F == 0 ? kTurnPair
+                          : reads_gradients(F) && (ST & 3) != RC_STORE_F16 ? kTurnAhead : kTurnOne;
     extern __shared__ float4 s_tf[];
     if (!(F & kTF2)) {
         load_tf(a.tf, s_tf);
