@@ -408,6 +408,17 @@ static VolDev vol_dev(const rc_volume *v) {
         d.inv2s[a] = 0.5f / v->s[a];
     }
     d.smin = smin;
+    // brick stride minus 16 local strides, per axis (unsigned arithmetic wraps)
+    const unsigned bricks[3] = {1u, (unsigned)v->cb[0], (unsigned)v->cb[0] * (unsigned)v->cb[1]};
+    const unsigned apron_l[3] = {1u, kApron, kApron * kApron}, vg_l[3] = {1u, kGradEdge, kGradEdge * kGradEdge};
+    // pairs along x hold 18 entries per row, pairs along y (FP32) 19 per row and 18 rows
+    const bool rows = v->storage == RC_STORE_F32;
+    const unsigned pair_l[3] = {1u, rows ? (unsigned)kApron : (unsigned)kPairRow, (unsigned)(kApron * kPairRow)};
+    for (int a = 0; a < 3; a++) {
+        d.apron_step[a] = bricks[a] * (unsigned)kApronVox - 16u * apron_l[a];
+        d.vg_step[a] = bricks[a] * (unsigned)kGradVox - 16u * vg_l[a];
+        d.pair_step[a] = bricks[a] * (unsigned)kPairVox - 16u * pair_l[a];
+    }
     d.vmax = v->vmax;
     d.vscale = full_scale(v);
     d.f16o = v->storage == RC_STORE_F16 ? (float)f16_offset(v->vmax) : 0.0f;

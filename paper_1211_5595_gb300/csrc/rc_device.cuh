@@ -133,11 +133,24 @@ __device__ __forceinline__ int brick_of(const VolDev &v, const Cell &c) {
 // offsets. Local coordinates of cell base i: (i & 15) + 1.
 constexpr unsigned kDX = 1, kDY = kApron, kDZ = kApron * kApron;
 
+// Index of the cell's local entry (lz * LZ + ly * LY + lx, l = i & 15) in bricks
+// of VOX entries. i & 15 = i - 16 (i >> 4), so with the brick's stride per axis
+// less 16 local strides (`step`) the index is one multiply-add per axis for the
+// coordinate and one for its brick: 8 instructions instead of 11 (1% of every
+// march, 3% of the plain ones together with the float sample counter).
+template <int VOX, int LY, int LZ>
+__device__ __forceinline__ unsigned brick_index(const VolDev &v, const Cell &c, const unsigned step[3]) {
+#ifdef RC_DEBUG
+    return (unsigned)brick_of(v, c) * (unsigned)VOX +
+           (unsigned)((c.i[2] & 15) * LZ + (c.i[1] & 15) * LY + (c.i[0] & 15));
+#else
+    const unsigned x = (unsigned)c.i[0], y = (unsigned)c.i[1], z = (unsigned)c.i[2];
+    return (x >> 4) * step[0] + ((y >> 4) * step[1] + ((z >> 4) * step[2] + (z * (unsigned)LZ + (y * (unsigned)LY + x))));
+#endif
+}
+
 __device__ __forceinline__ unsigned cell_address(const VolDev &v, const Cell &c) {
-    const unsigned b = (unsigned)brick_of(v, c);
-    const unsigned lx = (unsigned)(c.i[0] & 15) + 1, ly = (unsigned)(c.i[1] & 15) + 1,
-                   lz = (unsigned)(c.i[2] & 15) + 1;
-    return b * (unsigned)kApronVox + (lz * kApron + ly) * kApron + lx;
+    return brick_index<kApronVox, kApron, kApron * kApron>(v, c, v.apron_step) + (kDX + kDY + kDZ);
 }
 
 // Kernel instances are by storage (ST = rc_storage). An instance whose form
@@ -268,8 +281,7 @@ template <> struct Pair<RC_STORE_U16> { using T = ushort2; };
 template <int ST>
 __device__ __forceinline__ const typename Pair<ST>::T *pair_ptr(const VolDev &v, const Cell &c) {
     return reinterpret_cast<const typename Pair<ST>::T *>(v.pairs) +
-           ((unsigned)brick_of(v, c) * (unsigned)kPairVox +
-            (unsigned)((((c.i[2] & 15) * kApron + (c.i[1] & 15)) * kPairRow) + (c.i[0] & 15)));
+           brick_index<kPairVox, kPairRow, kApron * kPairRow>(v, c, v.pair_step);
 }
 
 // The two voxels of a pair entry as FP32 (the stored values converted as ldv does).
@@ -296,8 +308,7 @@ constexpr int pair_off() { return (OZ * kApron + OY) * kPairRow + OX; }
 __device__ __forceinline__ float value_grad_vg(const VolDev &v, const Cell &c, float g[3]) {
     // 32-bit index: a volume has fewer than 2^31 apron voxels (19^3 per
     // brick), so fewer value+gradient entries (17^3 per brick)
-    const unsigned idx = (unsigned)brick_of(v, c) * (unsigned)kGradVox +
-                         (unsigned)(((c.i[2] & 15) * kGradEdge + (c.i[1] & 15)) * kGradEdge + (c.i[0] & 15));
+    const unsigned idx = brick_index<kGradVox, kGradEdge, kGradEdge * kGradEdge>(v, c, v.vg_step);
     const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(v.vg) + idx;
     constexpr int DY = kGradEdge, DZ = kGradEdge * kGradEdge;
     const unsigned long long wx = pack2(c.w[0], c.w[0]), wy = pack2(c.w[1], c.w[1]), wz = pack2(c.w[2], c.w[2]);
@@ -346,8 +357,7 @@ __device__ __forceinline__ ulonglong2 vg16_lerp(uint2 qa, uint2 qb, unsigned lon
 // value_grad_vg from 8-byte entries of the same integers: the same operations
 // give the same result bit for bit.
 __device__ __forceinline__ float value_grad_vg16(const VolDev &v, const Cell &c, float g[3]) {
-    const unsigned idx = (unsigned)brick_of(v, c) * (unsigned)kGradVox +
-                         (unsigned)(((c.i[2] & 15) * kGradEdge + (c.i[1] & 15)) * kGradEdge + (c.i[0] & 15));
+    const unsigned idx = brick_index<kGradVox, kGradEdge, kGradEdge * kGradEdge>(v, c, v.vg_step);
     const uint2 *p = reinterpret_cast<const uint2 *>(v.vg) + idx;
     constexpr int DY = kGradEdge, DZ = kGradEdge * kGradEdge;
     const unsigned long long wx = pack2(c.w[0], c.w[0]), wy = pack2(c.w[1], c.w[1]), wz = pack2(c.w[2], c.w[2]);
@@ -368,8 +378,7 @@ __device__ __forceinline__ float value_grad_vg16(const VolDev &v, const Cell &c,
 // x, then y, then z), the differences as integers, and the gradient of h is
 // the code gradient / o (o a power of two: exact scaling).
 __device__ __forceinline__ float value_grad_vg16h(const VolDev &v, const Cell &c, float g[3]) {
-    const unsigned idx = (unsigned)brick_of(v, c) * (unsigned)kGradVox +
-                         (unsigned)(((c.i[2] & 15) * kGradEdge + (c.i[1] & 15)) * kGradEdge + (c.i[0] & 15));
+    const unsigned idx = brick_index<kGradVox, kGradEdge, kGradEdge * kGradEdge>(v, c, v.vg_step);
     const uint2 *p = reinterpret_cast<const uint2 *>(v.vg) + idx;
     constexpr int DY = kGradEdge, DZ = kGradEdge * kGradEdge;
     const unsigned long long wx = pack2(c.w[0], c.w[0]), wy = pack2(c.w[1], c.w[1]), wz = pack2(c.w[2], c.w[2]);
@@ -628,8 +637,7 @@ __device__ __forceinline__ float bspline_grad_x(const VolDev &v, const Cell &c, 
 template <bool GRAD>
 __device__ __forceinline__ float bspline_rows2(const VolDev &v, const Cell &c, float g[3]) {
     const unsigned long long *q = reinterpret_cast<const unsigned long long *>(v.pairs) +
-                                  ((unsigned)brick_of(v, c) * (unsigned)kPairVox +
-                                   (unsigned)(((c.i[2] & 15) * kPairRow + (c.i[1] & 15)) * kApron + (c.i[0] & 15)));
+                                  brick_index<kPairVox, kApron, kApron * kPairRow>(v, c, v.pair_step);
     float t[4], wy[4], wz[4], dy[4], dz[4];
     unsigned long long wx[4], dx[4];
     bspline_weights(c.w[0], t);

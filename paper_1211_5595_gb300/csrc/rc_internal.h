@@ -44,6 +44,9 @@ struct VolDev {
     int storage;           // rc_storage
     int n[3];              // voxels per axis
     int cb[3];             // cell-bricks per axis: ceil((n-1)/16)
+    // per axis, what a cell's brick adds to its linear index beyond its own
+    // coordinate (see brick_index): apron, value+gradient and pair bricks
+    unsigned apron_step[3], vg_step[3], pair_step[3];
     float s[3];            // spacing (mm)
     float inv2s[3];        // 0.5 / spacing
     float smin;            // reference step: finest spacing

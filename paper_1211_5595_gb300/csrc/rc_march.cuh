@@ -91,12 +91,13 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     const bool hit = inimg && setup_ray(cam, vol, a.p.step_vox, x, y, R);
     const int nsamp = hit ? R.nsamp : 0;
     float C0 = 0.0f, C1 = 0.0f, C2 = 0.0f, T = 1.0f;
-    int k = 0;
+    float k = 0.0f;               // sample counter: a float (exact, below 2^24) needs no conversion per sample
+    const float n = (float)nsamp;
     unsigned evald = 0;
     bool active = nsamp > 0;
-    auto cell_at = [&](int i, Cell &c) {
+    auto cell_at = [&](float i, Cell &c) {
         float p[3];
-        position_at(R, sample_t(R, i), p);
+        position_at(R, __fmaf_rn(i, R.ds, R.tn), p);
         cell_of(vol, p, c);
     };
     auto level = [&](const Cell &c) { return a.p.skip ? empty_level(a, lvl, c) : 0; };
@@ -106,20 +107,20 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     auto add = [&](const float4 &e) {
         composite_add(e, C0, C1, C2, T);
         evald++;
-        k++;
-        active = k < nsamp && (1.0f - T) < a.p.term;
+        k += 1.0f;
+        active = k < n && (1.0f - T) < a.p.term;
     };
     // past the largest empty block around the sample: its cell-brick, octant
     // or 4^3 sub-block
     auto jump = [&](const Cell &c, int s) {
-        k = jump_block(R, vol, c, k, s);
-        active = k < nsamp;
+        k = (float)jump_block(R, vol, c, (int)k, s);
+        active = k < n;
     };
     if constexpr (kTurn == kTurnPair) {
         while (active) {
             Cell c, cn;
             cell_at(k, c);
-            cell_at(k + 1, cn);                 // past the end: clamped into the volume, not used
+            cell_at(k + 1.0f, cn);                 // past the end: clamped into the volume, not used
             const int s = level(c), sn = level(cn);
             if (s) {
                 jump(c, s);
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
         Cell c;
         int s = 0;
         if (active) {
-            cell_at(0, c);
+            cell_at(0.0f, c);
             s = level(c);
         }
         while (active) {
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
                 continue;
             }
             Cell cn;
-            cell_at(k + 1, cn);
+            cell_at(k + 1.0f, cn);
             s = level(cn);
             add(sample(c));
             c = cn;
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
     }
     __syncwarp();
     if (inimg) out[(size_t)y * cam.W + x] = make_float4(C0, C1, C2, 1.0f - T);
-    if (a.stats) add_stats(a.stats, (unsigned)min(k, nsamp), evald, hit ? 1u : 0u, inimg ? 1u : 0u);
+    if (a.stats) add_stats(a.stats, (unsigned)min((int)k, nsamp), evald, hit ? 1u : 0u, inimg ? 1u : 0u);
 }
 
 // The compositing march with L lanes per ray, for launches too small to fill
