@@ -251,17 +251,18 @@ __global__ void __launch_bounds__(kMarchThreads) wide_kernel(const MarchArgs a) 
 // Ray function groups: the functions of one group share a loop.
 enum : int { kFnMip = 0, kFnSum = 1, kFnFirst = 2 };    // MIP | average, x-ray | isosurface, threshold
 
-// The largest block around cell c (brick b) whose codes cannot matter to a
-// search for values above `need` (code units): 4 for the cell-brick, 2 for the
-// 4^3 sub-block, -1 when the sample has to be evaluated. A block's maximum
+// The largest block around cell c (brick b) whose codes cannot matter, none of
+// them above `need`: 4 for the cell-brick, 2 for the 4^3 sub-block, -1 when the
+// sample has to be evaluated. need is a threshold in code units less a.slack,
+// rounded down (the conversion takes infinities to the ends of int). A block's maximum
 // code bounds every value reconstructed in it up to FP32 rounding (and, for
 // FP16 storage of more than 12 bits, the rounding of the stored values);
 // a.slack covers both many times over, so a skipped sample is strictly below
 // `need`.
-__device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int b, float need) {
+__device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int b, int need) {
     const int j = ((c.i[2] >> 2) * a.c4[1] + (c.i[1] >> 2)) * a.c4[0] + (c.i[0] >> 2);
-    if ((float)__ldg(a.mx4 + j) + a.slack > need) return -1;
-    return (float)__ldg(a.mx + b) + a.slack > need ? 2 : 4;
+    if ((int)__ldg(a.mx4 + j) > need) return -1;
+    return (int)__ldg(a.mx + b) > need ? 2 : 4;
 }
 
 // The other ray functions of Sec. 4.1 (MIP, average, x-ray, isosurface,
@@ -280,11 +281,12 @@ __device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int 
 // The value before a first hit is reconstructed once, when the hit is found.
 // Average and x-ray sum every sample.
 // Instruction issue bounds it (76% with every sample evaluated, L1 54%, DRAM
-// 3%). 256x256x180 phantom at 1024^2: 4 isosurface views 0.725 -> 0.283 ms,
-// 8 MIP views 2.44 -> 2.15 ms (the noise around the head has block maxima
-// above any value reconstructed in it, so 60% of the samples stay; jumping
-// lane by lane instead of by warp 2.55, with samples four voxels apart first
-// 2.60).
+// 3%). 256x256x180 phantom at 1024^2: 4 isosurface views 0.725 -> 0.253 ms,
+// 8 MIP views 2.44 -> 2.00 ms (the noise around the head has block maxima
+// above any value reconstructed in it, so 60% of the samples stay). Of the MIP
+// forms tried when the rest of the march took 2.15: jumping lane by lane instead
+// of by warp 2.55, with samples four voxels apart first 2.60; a branch on a new
+// maximum instead of the plain update 2% slower.
 template <int ST, bool CUBIC, int FN>
 __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs a) {
     extern __shared__ float4 s_tf[];
@@ -309,7 +311,8 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
     auto value = [&](const Cell &c) { return CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c); };
     // thresholds in code units: FP16 storage holds h = code / o - 1
     auto in_codes = [&](float v) { return ST == RC_STORE_F16 ? (v + 1.0f) * a.vol.f16o : v; };
-    float need = FN == kFnFirst ? in_codes(a.p.iso) : acc;
+    auto bound = [&](float v) { return __float2int_rd(in_codes(v) - a.slack); };
+    int need = bound(FN == kFnFirst ? a.p.iso : acc);
     auto cell_at = [&](int j, Cell &c) {
         float p[3];
         position_at(R, sample_t(R, j), p);
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
             evald++;
             if (v > acc) {
                 acc = v;
-                need = in_codes(v);
+                need = bound(v);
             }
         }
     }
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
         if (FN == kFnMip) {
             acc = fmaxf(acc, v0);
             if (two) acc = fmaxf(acc, v1);
-            need = in_codes(acc);
+            need = bound(acc);
         } else if (v0 >= a.p.iso || (two && v1 >= a.p.iso)) {
             if (!(v0 >= a.p.iso)) {
                 k++;

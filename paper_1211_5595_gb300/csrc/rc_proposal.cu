@@ -121,6 +121,30 @@ __global__ void __launch_bounds__(128) profiles_kernel(const MarchArgs a, float 
 // features: entry point (normalised to the box) and world direction, their
 // sin/cos encodings at 6 octaves, 32 occupancy bits along the chord, 2 zeros
 // ---------------------------------------------------------------------------
+// A ray in units of cell-bricks (positions / 16), for occupancy lookups: scaling
+// by a power of two is exact, so the truncated coordinate is the base cell's
+// brick (min(i, n - 2) >> 4 = min(i >> 4, cb - 1)) without the shifts.
+struct BrickRay {
+    float o[3], d[3];
+    __device__ __forceinline__ explicit BrickRay(const Ray &R) {
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            o[a] = R.o[a] * 0.0625f;
+            d[a] = R.d[a] * 0.0625f;
+        }
+    }
+    __device__ __forceinline__ bool occupied(const VolDev &v, const uint8_t *occ, float t) const {
+        int b[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) b[a] = (int)min(__float2uint_rz(__fmaf_rn(t, d[a], o[a])), (unsigned)(v.cb[a] - 1));
+        int at = (b[2] * v.cb[1] + b[1]) * v.cb[0] + b[0];
+#ifdef RC_DEBUG
+        at = dbg_index(at + v.dbg_poison, v.cb[0] * v.cb[1] * v.cb[2], v.dbg_err, kSiteBrick);
+#endif
+        return __ldg(occ + at) != 0;
+    }
+};
+
 // Emits the 112 features in 14 chunks of 8 (emit(chunk, v) in chunk order) and
 // returns the occupancy bits at the bin centres as a mask (bit b = bin b).
 // Feature order: 0-5 entry point and direction; 6 + 12c + 2j and 7 + 12c + 2j
@@ -159,7 +183,7 @@ __device__ __forceinline__ uint32_t ray_features(const VolDev &v, const uint8_t 
 #pragma unroll
         for (int j = 0; j < 6; j++) {
             if (j == 0 || j == 3) {
-                sincospif(ldexpf(xs[c], j), &s, &co);
+                sincospif(j == 0 ? xs[c] : 8.0f * xs[c], &s, &co);
             } else {
                 const float s2 = 2.0f * s * co;
                 co = (co - s) * (co + s);
@@ -170,14 +194,11 @@ __device__ __forceinline__ uint32_t ray_features(const VolDev &v, const uint8_t 
         }
     }
     const float bw = __fdiv_rn(__fsub_rn(R.tf, R.tn), (float)kBins);
+    const BrickRay B(R);
     uint32_t mask = 0;
 #pragma unroll
     for (int b = 0; b < kBins; b++) {
-        float p[3];
-        position_at(R, __fmaf_rn((float)b + 0.5f, bw, R.tn), p);
-        Cell c;
-        cell_of(v, p, c);
-        const bool o = __ldg(occ + brick_of(v, c)) != 0;
+        const bool o = B.occupied(v, occ, __fmaf_rn((float)b + 0.5f, bw, R.tn));
         mask |= (uint32_t)o << b;
         put(o ? 1.0f : 0.0f);
     }
@@ -578,14 +599,6 @@ __device__ __forceinline__ void plain_ray(const MarchArgs &a, const float4 *s_tf
     }
 }
 
-__device__ __forceinline__ bool occupied_at(const VolDev &v, const uint8_t *occ, const Ray &R, float t) {
-    float p[3];
-    position_at(R, t, p);
-    Cell c;
-    cell_of(v, p, c);
-    return __ldg(occ + brick_of(v, c)) != 0;
-}
-
 // The PDF marks where the ray's contribution ends: b_end is one bin past the
 // first bin >= b_start where its running sum reaches 1 - 1/64 (a margin for
 // early predictions; at most 31, and 31 if never); b_start is the
@@ -598,15 +611,16 @@ __device__ __forceinline__ void range_of(const MarchArgs &a, const Ray &R, const
     // fma(k, bw, t_near)); its centre bit comes from the features when known
     b0 = -1;
     b1 = kBins - 1;
-    bool start = occupied_at(a.vol, a.occ, R, R.tn);
+    const BrickRay B(R);
+    bool start = B.occupied(a.vol, a.occ, R.tn);
     for (int b = 0; b < kBins && b0 < 0; b++) {
         const bool mid = have_centre ? ((centre >> b) & 1u) != 0
-                                     : occupied_at(a.vol, a.occ, R, __fmaf_rn((float)b + 0.5f, bw, R.tn));
+                                     : B.occupied(a.vol, a.occ, __fmaf_rn((float)b + 0.5f, bw, R.tn));
         if (start || mid) {
             b0 = b;
             break;
         }
-        const bool end = occupied_at(a.vol, a.occ, R, __fmaf_rn((float)(b + 1), bw, R.tn));
+        const bool end = B.occupied(a.vol, a.occ, __fmaf_rn((float)(b + 1), bw, R.tn));
         if (end) b0 = b;
         start = end;
     }
