@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kMarchThreads) composite_kernel(const MarchArg
 // sample latencies is L times shorter. Samples past a termination are
 // evaluated in vain and the shuffles cost issue slots: lanes_per_ray says
 // where that pays.
-template <int L> struct WideTile;
+template <int L> struct WideTile { static constexpr int X = 8, Y = 4; };
 template <> struct WideTile<2> { static constexpr int X = 4, Y = 4; };
 template <> struct WideTile<4> { static constexpr int X = 4, Y = 2; };
 template <> struct WideTile<8> { static constexpr int X = 2, Y = 2; };
@@ -248,8 +248,9 @@ __global__ void __launch_bounds__(kMarchThreads) wide_kernel(const MarchArgs a) 
     }
 }
 
-// Ray function groups: the functions of one group share a loop.
-enum : int { kFnMip = 0, kFnSum = 1, kFnFirst = 2 };    // MIP | average, x-ray | isosurface, threshold
+// Ray function groups of function_kernel: MIP | isosurface, threshold (average
+// and x-ray: sum_kernel).
+enum : int { kFnMip = 0, kFnFirst = 2 };
 
 // The largest block around cell c (brick b) whose codes cannot matter, none of
 // them above `need`: 4 for the cell-brick, 2 for the 4^3 sub-block, -1 when the
@@ -279,7 +280,6 @@ __device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int 
 // takes samples eight voxels apart and so starts from nearly the ray's
 // maximum, with the space in front of the brightest tissue to skip as well.
 // The value before a first hit is reconstructed once, when the hit is found.
-// Average and x-ray sum every sample.
 // Instruction issue bounds it (76% with every sample evaluated, L1 54%, DRAM
 // 3%). 256x256x180 phantom at 1024^2: 4 isosurface views 0.725 -> 0.253 ms,
 // 8 MIP views 2.44 -> 2.00 ms (the noise around the head has block maxima
@@ -332,16 +332,8 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
             }
         }
     }
-    if (FN == kFnSum) {
-        for (; k < nsamp; k++) {
-            Cell c;
-            cell_at(k, c);
-            acc += value(c);
-        }
-        evald = (unsigned)nsamp;
-    }
-    bool active = FN != kFnSum && nsamp > 0;
-    while (FN != kFnSum && __any_sync(kFull, active)) {
+    bool active = nsamp > 0;
+    while (__any_sync(kFull, active)) {
         Cell c0, c1;
         if (active) cell_at(k, c0);
         if (a.p.skip) {
@@ -404,24 +396,73 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
         }
     }
     k = min(k, nsamp);
-    if (FN != kFnFirst && nsamp > 0) {
+    if (FN == kFnMip && nsamp > 0) {
         // over full scale; FP16 values h = (code - o) / o are shifted by 1 first
         // (code / vmax = (h + 1) / vscale)
-        float m;
-        if (ST == RC_STORE_F16) {
-            if (FN == kFnMip) m = (acc + 1.0f) / a.vol.vscale;
-            else if (func == RC_FUNC_AVERAGE) m = (acc / (float)nsamp + 1.0f) / a.vol.vscale;
-            else m = (acc + (float)nsamp) * R.ds / a.vol.vscale;
-        } else {
-            if (FN == kFnMip) m = acc / a.vol.vscale;
-            else if (func == RC_FUNC_AVERAGE) m = acc / (float)nsamp / a.vol.vscale;
-            else m = acc * R.ds / a.vol.vscale;
-        }
+        const float m = (ST == RC_STORE_F16 ? acc + 1.0f : acc) / a.vol.vscale;
         out = make_float4(m, m, m, 1.0f);
     }
     if (inimg) outp[(size_t)y * cam.W + x] = out;
     // a sample that MIP took in its first pass too counts once
     if (a.stats) add_stats(a.stats, (unsigned)k, min(evald, (unsigned)k), hit ? 1u : 0u, inimg ? 1u : 0u);
+}
+
+// Average and x-ray: the sum of every sample, in sample order. L lanes per ray
+// as in wide_kernel: lane j reconstructs sample k + j and the
+// group adds the L values in order from shuffles (the same sum bit for bit; the
+// measured times stand at lanes_per_sum). Bound by instruction issue, for the
+// B-spline by its chain of gathers.
+template <int ST, bool CUBIC, int L>
+__global__ void __launch_bounds__(kMarchThreads) sum_kernel(const MarchArgs a) {
+    const CamRec cam = a.cams ? a.cams[blockIdx.z] : a.cam;
+    float4 *outp = a.out + (size_t)blockIdx.z * cam.W * cam.H;
+    constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane % L, ray = lane / L, first = lane - j;
+    const int x = blockIdx.x * (kWarpsX * TX) + (warp % kWarpsX) * TX + ray % TX;
+    const int y = blockIdx.y * (kWarpsY * TY) + (warp / kWarpsX) * TY + ray / TX;
+    const bool inimg = x < cam.W && y < cam.H;
+    Ray R;
+    const bool hit = inimg && setup_ray(cam, a.vol, a.p.step_vox, x, y, R);
+    const int nsamp = hit ? R.nsamp : 0;
+    float acc = 0.0f;
+    auto value = [&](int k) {
+        float p[3];
+        position_at(R, sample_t(R, k), p);
+        Cell c;
+        cell_of(a.vol, p, c);
+        return CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c);
+    };
+    if constexpr (L == 1) {
+#pragma unroll 1
+        for (int k = 0; k < nsamp; k++) acc += value(k);
+    } else {
+#pragma unroll 1
+        for (int k = 0; __any_sync(kFull, k < nsamp); k += L) {
+            const float v = k + j < nsamp ? value(k + j) : 0.0f;
+#pragma unroll
+            for (int i = 0; i < L; i++) {
+                const float q = __shfl_sync(kFull, v, first + i);
+                if (k + i < nsamp) acc += q;
+            }
+        }
+    }
+    // over full scale; FP16 values h = code / o - 1 are shifted by 1 per sample first
+    float4 out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (nsamp > 0) {
+        const float n = (float)nsamp;
+        float m;
+        if (ST == RC_STORE_F16)
+            m = a.p.func == RC_FUNC_AVERAGE ? (acc / n + 1.0f) / a.vol.vscale : (acc + n) * R.ds / a.vol.vscale;
+        else
+            m = a.p.func == RC_FUNC_AVERAGE ? acc / n / a.vol.vscale : acc * R.ds / a.vol.vscale;
+        out = make_float4(m, m, m, 1.0f);
+    }
+    const bool one = j == 0;
+    if (inimg && one) outp[(size_t)y * cam.W + x] = out;
+    if (a.stats) {
+        const unsigned n = one ? (unsigned)nsamp : 0u;
+        add_stats(a.stats, n, n, one && hit ? 1u : 0u, one && inimg ? 1u : 0u);
+    }
 }
 
 template <typename K>
@@ -435,6 +476,43 @@ static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool ta
     dim3 grid((a.cam.W + tile_w - 1) / tile_w, (a.cam.H + tile_h - 1) / tile_h, nviews);
     kern<<<grid, kMarchThreads, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+// About how many rays of a launch meet the volume: the box's corners bound the
+// part of the image (of the first view) whose rays can, and its silhouette fills
+// about two thirds of that rectangle.
+static double rays_that_hit(const MarchArgs &a, int nviews) {
+    const CamRec &c = a.cam;
+    double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0};
+    for (int q = 0; q < 8; q++) {
+        double z = 0.0, u[2] = {0.0, 0.0};
+        for (int i = 0; i < 3; i++) {
+            const double d = (((q >> i) & 1 ? a.vol.n[i] - 1 : 0) - (double)c.o[i]) * a.vol.s[i];
+            z += d * c.f[i];
+            u[0] += d * c.r[i];
+            u[1] += d * c.u[i];
+        }
+        if (!(z > 0.0)) return 0.65 * c.W * c.H * nviews;      // a corner behind the eye: the whole image
+        const double t[2] = {c.tx, c.ty};
+        for (int i = 0; i < 2; i++) {
+            const double e = u[i] / (z * t[i]);
+            lo[i] = e < lo[i] ? e : lo[i];
+            hi[i] = e > hi[i] ? e : hi[i];
+        }
+    }
+    double part = 0.65;
+    for (int i = 0; i < 2; i++) {
+        const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
+        part *= h > l ? (h - l) * 0.5 : 0.0;
+    }
+    return part * c.W * c.H * nviews;
+}
+
+// Samples across the box's diagonal.
+static double samples_across(const MarchArgs &a) {
+    double diag2 = 0.0;
+    for (int i = 0; i < 3; i++) diag2 += (double)(a.vol.n[i] - 1) * a.vol.s[i] * (a.vol.n[i] - 1) * a.vol.s[i];
+    return sqrt(diag2) / ((double)a.p.step_vox * a.vol.smin);
 }
 
 // Lanes per ray of a launch. A ray's samples are a serial chain (a few hundred
@@ -454,37 +532,8 @@ static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool ta
 // entries, which the FP32 shaded figures above are for; B-spline; 2-D table) gain
 // further up than the others.
 static int lanes_per_ray(const MarchArgs &a, int nviews) {
-    // the box's corners bound the part of the image whose rays can meet it;
-    // its silhouette fills about two thirds of that rectangle
-    const CamRec &c = a.cam;
-    double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0}, diag2 = 0.0;
-    bool behind = false;
-    for (int q = 0; q < 8; q++) {
-        double d[3], z = 0.0, u[2] = {0.0, 0.0};
-        for (int i = 0; i < 3; i++) {
-            d[i] = (((q >> i) & 1 ? a.vol.n[i] - 1 : 0) - (double)c.o[i]) * a.vol.s[i];
-            z += d[i] * c.f[i];
-            u[0] += d[i] * c.r[i];
-            u[1] += d[i] * c.u[i];
-        }
-        if (!(z > 0.0)) behind = true;
-        else {
-            const double t[2] = {c.tx, c.ty};
-            for (int i = 0; i < 2; i++) {
-                const double e = u[i] / (z * t[i]);
-                lo[i] = e < lo[i] ? e : lo[i];
-                hi[i] = e > hi[i] ? e : hi[i];
-            }
-        }
-    }
-    double part = 1.0;
-    for (int i = 0; i < 2 && !behind; i++) {
-        const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
-        part *= h > l ? (h - l) * 0.5 : 0.0;
-    }
-    for (int i = 0; i < 3; i++) diag2 += (double)(a.vol.n[i] - 1) * a.vol.s[i] * (a.vol.n[i] - 1) * a.vol.s[i];
-    const double hits = 0.65 * part * c.W * c.H * nviews;
-    const double steps = sqrt(diag2) / ((double)a.p.step_vox * a.vol.smin);
+    if (a.cam.H > 4 * 65535) return 1;     // the grid's y limit at 4 rows per CTA
+    const double hits = rays_that_hit(a, nviews), steps = samples_across(a);
     const bool heavy = (a.p.shade && !a.vol.vg16) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2;
     if (hits <= (heavy ? 22e3 : 7e3) && hits <= 70.0 * steps) return 8;
     if (hits <= 76e3 && hits <= 190.0 * steps) return 4;
@@ -492,7 +541,19 @@ static int lanes_per_ray(const MarchArgs &a, int nviews) {
     return 1;
 }
 
-template <int F, int L>
+// Lanes per ray of the sums: every ray marches its whole chord, so no sample is
+// in vain and more lanes pay further up, for the B-spline's long samples always
+// (us with 1, 2 and 4 lanes, FP32 trilinear / B-spline: one 600^2 view of
+// 256x256x180 322 201 131 / 1565 833 580, three 865x878 views of 51x302x86 222
+// 184 204 / 1085 720 672, four 1024^2 views of 256x256x180 1064 1051 1224 / 5592
+// 4842 5112).
+static int lanes_per_sum(const MarchArgs &a, int nviews) {
+    const double hits = rays_that_hit(a, nviews);
+    const bool cubic = a.p.filter == RC_FILTER_BSPLINE;
+    if (hits <= (cubic ? 600e3 : 200e3) && a.cam.H <= 4 * 65535) return 4;
+    return cubic || hits <= 600e3 ? 2 : 1;
+}
+ template <int F, int L>
 static cudaError_t launch_wide(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = !(F & kTF2);
     constexpr int W = kWarpsX * WideTile<L>::X, H = kWarpsY * WideTile<L>::Y;
@@ -535,12 +596,25 @@ static cudaError_t launch_function_group(const MarchArgs &a, int nviews, cudaStr
     });
 }
 
+template <bool CUBIC, int L>
+static cudaError_t launch_sum(const MarchArgs &a, int nviews, cudaStream_t s) {
+    constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
+    return by_storage<false>(a.vol, [&](auto st) {
+        return launch_kernel(sum_kernel<decltype(st)::value, CUBIC, L>, a, nviews, false, s, kWarpsX * TX, kWarpsY * TY);
+    });
+}
+
 template <bool CUBIC>
 static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t s) {
     switch (a.p.func) {
         case RC_FUNC_MIP: return launch_function_group<CUBIC, kFnMip>(a, nviews, s);
         case RC_FUNC_AVERAGE:
-        case RC_FUNC_XRAY: return launch_function_group<CUBIC, kFnSum>(a, nviews, s);
+        case RC_FUNC_XRAY:
+            switch (lanes_per_sum(a, nviews)) {
+                case 4: return launch_sum<CUBIC, 4>(a, nviews, s);
+                case 2: return launch_sum<CUBIC, 2>(a, nviews, s);
+                default: return launch_sum<CUBIC, CUBIC ? 2 : 1>(a, nviews, s);      // the B-spline: 2 at least
+            }
         default: return launch_function_group<CUBIC, kFnFirst>(a, nviews, s);
     }
 }

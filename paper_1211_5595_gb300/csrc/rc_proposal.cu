@@ -49,71 +49,75 @@ __global__ void __launch_bounds__(128) profiles_kernel(const MarchArgs a, float 
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = lane % kProfLanes, ray = lane / kProfLanes,
               first = lane - j;
-    const int x0 = blockIdx.x * kProfTileX + (warp & 1) * 4, y0 = blockIdx.y * kProfTileY + (warp >> 1) * 2;
-    const int x = x0 + (ray & 3), y = y0 + (ray >> 2);
-    Ray R;
-    const bool hit = x < a.cam.W && y < a.cam.H && setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
-    float *row = s_row[warp][ray];
-    for (int b = j; b < kBins; b += kProfLanes) row[b] = 0.0f;
-    __syncwarp();
-    float T = 1.0f;
-    if (__any_sync(0xffffffffu, hit)) {
-        constexpr int kPerBin = kProfSamples / kBins, kPerLane = kPerBin / kProfLanes;
-        const float delta = hit ? __fdiv_rn(__fsub_rn(R.tf, R.tn), (float)kProfSamples) : 0.0f;
-        const float ratio = __fdiv_rn(delta, a.vol.smin);
-        int b = hit ? 0 : kBins;
-        while (__any_sync(0xffffffffu, b < kBins)) {
-            const bool on = b < kBins;
-            float al[kPerLane];
-            Cell c;
-            int s = 0;
-            unsigned some = 0;
-#pragma unroll
-            for (int i = 0; i < kPerLane; i++) {
-                al[i] = 0.0f;
-                if (on) {
-                    float p[3];
-                    position_at(R, __fmaf_rn((float)(b * kPerBin + i * kProfLanes + j) + 0.5f, delta, R.tn), p);
-                    cell_of(a.vol, p, c);
-                    s = a.p.skip ? empty_level(a, a.lvl, c) : 0;
-                    if (!s) {
-                        al[i] = eval_sample<ST, false>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio).w;
-                        some = 1;
+    // more tile rows than the grid's y limit take further turns
+    for (int tile_y = blockIdx.y; tile_y * kProfTileY < a.cam.H; tile_y += gridDim.y) {
+        __syncwarp();
+        const int x0 = blockIdx.x * kProfTileX + (warp & 1) * 4, y0 = tile_y * kProfTileY + (warp >> 1) * 2;
+        const int x = x0 + (ray & 3), y = y0 + (ray >> 2);
+        Ray R;
+        const bool hit = x < a.cam.W && y < a.cam.H && setup_ray(a.cam, a.vol, a.p.step_vox, x, y, R);
+        float *row = s_row[warp][ray];
+        for (int b = j; b < kBins; b += kProfLanes) row[b] = 0.0f;
+        __syncwarp();
+        float T = 1.0f;
+        if (__any_sync(0xffffffffu, hit)) {
+            constexpr int kPerBin = kProfSamples / kBins, kPerLane = kPerBin / kProfLanes;
+            const float delta = hit ? __fdiv_rn(__fsub_rn(R.tf, R.tn), (float)kProfSamples) : 0.0f;
+            const float ratio = __fdiv_rn(delta, a.vol.smin);
+            int b = hit ? 0 : kBins;
+            while (__any_sync(0xffffffffu, b < kBins)) {
+                const bool on = b < kBins;
+                float al[kPerLane];
+                Cell c;
+                int s = 0;
+                unsigned some = 0;
+    #pragma unroll
+                for (int i = 0; i < kPerLane; i++) {
+                    al[i] = 0.0f;
+                    if (on) {
+                        float p[3];
+                        position_at(R, __fmaf_rn((float)(b * kPerBin + i * kProfLanes + j) + 0.5f, delta, R.tn), p);
+                        cell_of(a.vol, p, c);
+                        s = a.p.skip ? empty_level(a, a.lvl, c) : 0;
+                        if (!s) {
+                            al[i] = eval_sample<ST, false>(a.vol, a.p, s_tf, a.tf.K, a.tf.ucoef, R.dir, c, 3, ratio).w;
+                            some = 1;
+                        }
                     }
                 }
-            }
-            float acc = 0.0f;
-            if (__any_sync(0xffffffffu, some)) {
-#pragma unroll
-                for (int k = 0; k < kPerBin; k++) {
-                    const float w = __shfl_sync(0xffffffffu, al[k / kProfLanes], first + k % kProfLanes);
-                    acc = __fmaf_rn(T, w, acc);
-                    T = T * (1.0f - w);
+                float acc = 0.0f;
+                if (__any_sync(0xffffffffu, some)) {
+    #pragma unroll
+                    for (int k = 0; k < kPerBin; k++) {
+                        const float w = __shfl_sync(0xffffffffu, al[k / kProfLanes], first + k % kProfLanes);
+                        acc = __fmaf_rn(T, w, acc);
+                        T = T * (1.0f - w);
+                    }
+                }
+                const unsigned in_group = (__ballot_sync(0xffffffffu, some) >> first) & ((1u << kProfLanes) - 1u);
+                int next = b + 1;
+                if (on && in_group == 0) {
+                    // the sample after the block of each lane's last sample; the
+                    // bins wholly before the last lane's stay zero
+                    const int k = jump_block_grid(R, a.vol, c, b * kPerBin + kPerBin - kProfLanes + j, s, R.tn, delta, kProfSamples);
+                    next = max(next, k / kPerBin);
+                }
+                next = __shfl_sync(0xffffffffu, next, first + kProfLanes - 1);
+                if (on) {
+                    if (j == 0 && in_group) row[b] = acc;
+                    b = next;
                 }
             }
-            const unsigned in_group = (__ballot_sync(0xffffffffu, some) >> first) & ((1u << kProfLanes) - 1u);
-            int next = b + 1;
-            if (on && in_group == 0) {
-                // the sample after the block of each lane's last sample; the
-                // bins wholly before the last lane's stay zero
-                const int k = jump_block_grid(R, a.vol, c, b * kPerBin + kPerBin - kProfLanes + j, s, R.tn, delta, kProfSamples);
-                next = max(next, k / kPerBin);
-            }
-            next = __shfl_sync(0xffffffffu, next, first + kProfLanes - 1);
-            if (on) {
-                if (j == 0 && in_group) row[b] = acc;
-                b = next;
-            }
         }
-    }
-    if (j == 0) row[kBins] = T;
-    __syncwarp();
-    // two image rows of up to four rays, contiguous in the output
-    const int rays = min(4, a.cam.W - x0);
-    for (int r = 0; r < 2 && y0 + r < a.cam.H; r++) {
-        float *o = out + ((size_t)(y0 + r) * a.cam.W + x0) * kOutUsed;
-        const float *src = s_row[warp][4 * r];
-        for (int e = lane; e < rays * kOutUsed; e += 32) o[e] = src[e];
+        if (j == 0) row[kBins] = T;
+        __syncwarp();
+        // two image rows of up to four rays, contiguous in the output
+        const int rays = min(4, a.cam.W - x0);
+        for (int r = 0; r < 2 && y0 + r < a.cam.H; r++) {
+            float *o = out + ((size_t)(y0 + r) * a.cam.W + x0) * kOutUsed;
+            const float *src = s_row[warp][4 * r];
+            for (int e = lane; e < rays * kOutUsed; e += 32) o[e] = src[e];
+        }
     }
 }
 
@@ -1322,7 +1326,7 @@ cudaError_t launch_profiles(const MarchArgs &a, float *out, cudaStream_t s) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        const dim3 grid((a.cam.W + kProfTileX - 1) / kProfTileX, (a.cam.H + kProfTileY - 1) / kProfTileY);
+        const dim3 grid((a.cam.W + kProfTileX - 1) / kProfTileX, min(65535, (a.cam.H + kProfTileY - 1) / kProfTileY));
         kern<<<grid, 128, smem, s>>>(a, out);
         return cudaGetLastError();
     };

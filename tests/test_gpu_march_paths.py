@@ -132,3 +132,31 @@ def test_gradient_forms_by_code_width(rc, orc, storage, vmax):
         assert torch.isfinite(out).all() and out[..., 3].max() > 0.2
     finally:
         r.close()
+
+
+# Average and x-ray sums: a small launch (several lanes per ray) gives the sums
+# of a large one (one lane per ray) bit for bit, and matches the oracle.
+@pytest.mark.parametrize("storage", ["F32", "F16", "U16"])
+@pytest.mark.parametrize("filt", [0, 1])
+@pytest.mark.parametrize("size,views", [((37, 21), 1200), ((97, 75), 130), ((260, 201), 18)])
+def test_sums_by_lanes(rc, orc, storage, filt, size, views):
+    import torch
+    dims, spacing = (50, 41, 37), (1.0, 1.0, 1.5)
+    ph = synth.head_phantom(dims, spacing, seed=5, tumor_radius_vox=3)
+    tf = synth.tf_table(64)
+    r = GPURenderer(rc, ph.vol, spacing, getattr(rc, "RC_STORE_" + storage))
+    try:
+        r.set_tf(tf)
+        w, h = size
+        cam = synth.orbit_camera(dims, spacing, 77.0, width=w, height=h)
+        for func, name in ((rc.RC_FUNC_AVERAGE, "AVERAGE"), (rc.RC_FUNC_XRAY, "XRAY")):
+            P = dict(step_vox=0.4, func=func, filter=filt)
+            one, st = r.render(cam, stats=True, **P)
+            many = torch.empty((views, h, w, 4), device="cuda")
+            sm = rc.rc_render_views(r.ctx, r.vol, P, [cam] * views, many, stats=True)
+            assert (many == torch.from_numpy(one).cuda()[None]).all()
+            assert sm["dense_samples"] == sm["evaluated_samples"] == views * st["dense_samples"] == views * st["evaluated_samples"]
+            o = orc.render(orc.Scene(ph.vol, spacing, tf, cam, step=0.4, term=0.99, func=getattr(orc, name), filter=filt))
+            np.testing.assert_allclose(one.reshape(-1, 4), o["rgba"].reshape(-1, 4), rtol=2e-5, atol=1e-5)
+    finally:
+        r.close()
