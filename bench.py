@@ -38,7 +38,7 @@ import synth  # noqa: E402
 
 WORKLOAD = "shaded_256x256x180"
 METRIC = "Gsamples/s (dense-equivalent), 1024^2 of 256x256x180 u16, shaded, 36-view orbit"
-BYTES_PER_SAMPLE = 128          # 32 distinct FP32 voxels per shaded sample (8 value+gradient float4)
+BYTES_PER_SAMPLE = 128          # 32 distinct FP32 voxels per shaded sample (loaded as 8 8-byte value+gradient entries)
 TF2_GMAX = 1200.0               # gradient magnitude (codes per mm) of the 2-D table's last row
 L2_FLUSH_BYTES = 256 << 20      # > 129 MB L2
 
@@ -1068,7 +1068,7 @@ def main():
         "roofline": {"bound": "l1", "achieved": achieved, "peak": l1_peak, "unit": "GB/s",
                      "frac": achieved / l1_peak, "traffic": traffic,
                      "kernel": "composite_kernel<F32, shaded>, one launch per step for all views",
-                     "model": f"{BYTES_PER_SAMPLE} B per evaluated sample (32 distinct FP32 voxels = 8 value+gradient float4) / mean launch time",
+                     "model": f"{BYTES_PER_SAMPLE} B per evaluated sample (32 distinct FP32 voxels; loaded as 8 8-byte value+gradient entries) / mean launch time",
                      "peak_kind": "measured in this run: rc_probe_read_l1, coalesced 16-byte read-only loads of "
                                   "an L1-resident 32 KB buffer by 4 CTAs per SM",
                      "note": "95% of the gather sectors hit L1, so L1 is the memory level that serves the "

@@ -32,7 +32,7 @@ __device__ __forceinline__ void tile_pixel(int &x, int &y) {
 // opacity exactly 0 and changes nothing, so the values are those of one lane
 // marching alone). A ray's 512 samples are a serial chain and only the rays that
 // meet the volume have one, so one lane per ray left the GPU waiting on latency
-// (256x256x180, 256^2 view 240 us, 512^2 257, 1024^2 602; now 68, 136 and 398).
+// (256x256x180, 256^2 view 240 us, 512^2 257, 1024^2 602; now 69, 133 and 399).
 // When a whole bin is empty, the bins up to the exit of the last sample's block
 // are too. Rows are staged in shared memory and written 132 contiguous bytes
 // per ray.

@@ -84,12 +84,13 @@ struct BoxWalk {
     }
 };
 
-// Bound by the bytes written (349 MB moved per 256x256x180 FP32 upload, 51 us at
-// the copy rate) once the index arithmetic is out of the way: 102 us with a
-// division per element and axis, neighbour clamps per difference and the grids
-// reduced in separate passes (97 M warp instructions, issue 75%), 61 us now; whole
-// uploads with the copy into the staging buffer, us: 256x256x180 FP32 112 -> 72,
-// 512x512x256 uint16 526 -> 290, 64x64x32 FP32 19 -> 13.
+// Bound by index arithmetic and, once that is out of the way, by the bytes written.
+// With 16-byte FP32 entries (349 MB moved per 256x256x180 upload, 51 us at the copy
+// rate): 102 us with a division per element and axis, neighbour clamps per
+// difference and the grids reduced in separate passes (97 M warp instructions,
+// issue 75%), 61 us with the walk. 8-byte entries move 229 MB (34 us). Whole uploads
+// with the copy into the staging buffer, us: 256x256x180 FP32 112 -> 64,
+// 512x512x256 uint16 526 -> 292, 64x64x32 FP32 19 -> 13.
 template <int ST>
 __global__ void __launch_bounds__(256) prep_kernel(const PrepArgs A) {
     __shared__ uint16_t s_code[kApronVox];
