@@ -43,8 +43,11 @@ cudaError_t launch_absmax(const float *x, long long n, float *out, cudaStream_t 
     return cudaGetLastError();
 }
 
+// Fixed-point units per unit of gradient, finite for every dL/dI: the floor is
+// the smallest maximum whose scale does not overflow FP32 (2^32 / 1.3e-29 =
+// 3.30e38), so zeros stay zeros when they are scaled.
 __device__ __forceinline__ float fixed_scale(const float *absmax) {
-    return 4294967296.0f / fmaxf(*absmax, 1e-30f);
+    return 4294967296.0f / fmaxf(*absmax, 1.3e-29f);
 }
 
 __device__ __forceinline__ void acc_add(unsigned long long *acc, int idx, float v, float scale) {
@@ -236,8 +239,8 @@ __device__ __forceinline__ void gradient_tile(const AdjointArgs &A, const float4
     bool hit = inimg && setup_ray(cam, a.vol, a.p.step_vox, x, y, R);
     float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (hit) g = A.dimg[((size_t)view * cam.H + y) * cam.W + x];
-    if (TF2) g = make_float4(g.x * gscale, g.y * gscale, g.z * gscale, g.w * gscale);
     const bool has_g = hit && (g.x != 0.0f || g.y != 0.0f || g.z != 0.0f || g.w != 0.0f);
+    if (TF2) g = make_float4(g.x * gscale, g.y * gscale, g.z * gscale, g.w * gscale);
     // pass 1: the forward march, with exact empty-space skipping over empty
     // bricks, octants and 4^3 sub-blocks (identical result), for C_final,
     // T_final and the sample count n up to termination
