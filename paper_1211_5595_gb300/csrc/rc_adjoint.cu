@@ -24,6 +24,7 @@
 // on the order of the atomics, and no other sum depends on thread scheduling,
 // so the result is deterministic.
 #include "rc_device.cuh"
+#include "rc_rules.h"
 
 namespace rc {
 
@@ -511,9 +512,8 @@ static cudaError_t launch_adj2(Kern kern, const AdjointArgs &a, int nviews, cons
     if ((e = cudaMemsetAsync(a.next, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
     const int cx = (a.m.cam.W + 15) / 16, cy = (a.m.cam.H + 2 * kGroupWarps - 1) / (2 * kGroupWarps);
     const int nchunks = cx * cy * nviews;       // at most 2^31 pixels in all: fewer than 2^28
-    const int groups = group_count(CUBIC);
-    const int grid = sms < (nchunks + groups - 1) / groups ? sms : (nchunks + groups - 1) / groups;
-    kern<<<grid, 32 * kGroupWarps * groups, smem, s>>>(a, absmax, slots, tagged ? 1 : 0, cx, cy, nchunks);
+    const int grid = persistent_ctas(nchunks, sms);
+    kern<<<grid, 32 * kGroupWarps * group_count(CUBIC), smem, s>>>(a, absmax, slots, tagged ? 1 : 0, cx, cy, nchunks);
     return cudaGetLastError();
 }
 
