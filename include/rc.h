@@ -26,6 +26,9 @@
  *    Voxel arrays are x fastest, then y, then z.
  *  - Images are row-major H x W x 4 floats, y = 0 at the top, premultiplied
  *    RGBA on a black background.
+ *  - Device images (rendered, forward and dL/dI) and the feature matrix that the
+ *    network's forward, gradient and training calls read are accessed 16 bytes
+ *    at a time: their addresses must be multiples of 16 (RC_ERR_INVALID_ARG).
  */
 #ifndef RC_H
 #define RC_H

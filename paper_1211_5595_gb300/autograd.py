@@ -45,8 +45,11 @@ class RenderTF(torch.autograd.Function):
         tf, out = fctx.saved_tensors
         _set_table(fctx.handle, tf, fctx.gmax)
         dtf = torch.empty_like(tf)
-        rc_render_backward_views_with_forward(fctx.handle, fctx.vol, fctx.params, [fctx.camera], out,
-                                              gout.contiguous(), dtf)
+        gout = gout.contiguous()
+        if gout.data_ptr() % 16:          # a view into a larger gradient: the library wants whole 16-byte pixels
+            gout = gout.clone()
+        rc_render_backward_views_with_forward(fctx.handle, fctx.vol, fctx.params, [fctx.camera], out, gout,
+                                              dtf)
         return dtf, None, None, None, None, None
 
 

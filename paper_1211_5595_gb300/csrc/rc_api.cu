@@ -742,6 +742,14 @@ static rc_status check_render(rc_context *ctx, const rc_volume *v, const rc_rend
     return RC_OK;
 }
 
+// The kernels read and write image pixels and network features 16 bytes at a
+// time; a device address that is not a multiple of 16 would fault the context.
+static rc_status check_aligned(rc_context *ctx, const void *p, const char *what, const char *who) {
+    if ((reinterpret_cast<uintptr_t>(p) & 15u) != 0)
+        return fail(ctx, RC_ERR_INVALID_ARG, "%s: %s is not 16-byte aligned", who, what);
+    return RC_OK;
+}
+
 // A set of views: 1..65535 valid cameras of one image size, at most 2^31
 // pixels in all.
 static rc_status check_views(rc_context *ctx, const rc_camera *cams, int nviews, const char *who) {
@@ -981,6 +989,7 @@ static MarchArgs march_args(rc_context *ctx, const rc_volume *v, const rc_render
 rc_status rc_render(rc_context *ctx, const rc_volume *vol, const rc_render_params *p, float *out_rgba,
                     rc_stats *stats) {
     rc_status st = check_render(ctx, vol, p, out_rgba, "rc_render");
+    if (st == RC_OK) st = check_aligned(ctx, out_rgba, "out_rgba", "rc_render");
     if (st != RC_OK) return st;
     DeviceScope ds(ctx->device);
     rc_volume *v = const_cast<rc_volume *>(vol);
@@ -1004,6 +1013,7 @@ rc_status rc_render_views(rc_context *ctx, const rc_volume *vol, const rc_render
     if (!ctx) return fail(nullptr, RC_ERR_INVALID_ARG, "%s: ctx is NULL", who);
     rc_status st = check_views(ctx, cams, nviews, who);
     if (st == RC_OK) st = check_render_views(ctx, vol, p, cams, out_rgba, who);
+    if (st == RC_OK) st = check_aligned(ctx, out_rgba, "out_rgba", who);
     if (st != RC_OK) return st;
     DeviceScope ds(ctx->device);
     rc_volume *v = const_cast<rc_volume *>(vol);
@@ -1149,6 +1159,8 @@ rc_status rc_render_batch(rc_context *ctx, const rc_volume *const *vols, int nvo
             return fail(ctx, RC_ERR_INVALID_ARG, "%s: volume %d differs from volume 0 in shape, spacing, vmax or "
                         "storage", who, i);
     }
+    st = check_aligned(ctx, out_rgba, "out_rgba", who);
+    if (st != RC_OK) return st;
     if (p->func != RC_FUNC_COMPOSITE) return fail(ctx, RC_ERR_UNSUPPORTED, "%s: compositing function only", who);
     DeviceScope ds(ctx->device);
     for (int i = 0; i < nvols; i++) {
@@ -1194,6 +1206,8 @@ rc_status rc_render_backward(rc_context *ctx, const rc_volume *vol, const rc_ren
     rc_status st = check_render(ctx, vol, p, dL_dtf, "rc_render_backward");
     if (st != RC_OK) return st;
     if (!dL_dimage) return fail(ctx, RC_ERR_INVALID_ARG, "rc_render_backward: dL_dimage is NULL");
+    st = check_aligned(ctx, dL_dimage, "dL_dimage", "rc_render_backward");
+    if (st != RC_OK) return st;
     if (p->func != RC_FUNC_COMPOSITE)
         return fail(ctx, RC_ERR_UNSUPPORTED, "rc_render_backward: compositing function only");
     DeviceScope ds(ctx->device);
@@ -1239,6 +1253,9 @@ static rc_status backward_views(rc_context *ctx, const rc_volume *vol, const rc_
     if (st == RC_OK) st = check_render_views(ctx, vol, p, cams, dL_dtf, who);
     if (st != RC_OK) return st;
     if (!dL_dimages) return fail(ctx, RC_ERR_INVALID_ARG, "%s: dL_dimages is NULL", who);
+    st = check_aligned(ctx, dL_dimages, "dL_dimages", who);
+    if (st == RC_OK) st = check_aligned(ctx, images, "images", who);
+    if (st != RC_OK) return st;
     if (p->func != RC_FUNC_COMPOSITE) return fail(ctx, RC_ERR_UNSUPPORTED, "%s: compositing function only", who);
     DeviceScope ds(ctx->device);
     st = ensure_grad_scratch(ctx);
@@ -1306,6 +1323,8 @@ rc_status rc_render_backward_noalloc(rc_context *ctx, const rc_volume *vol, cons
     rc_status st = check_render(ctx, vol, p, dL_dtf, "rc_render_backward_noalloc");
     if (st != RC_OK) return st;
     if (!dL_dimage) return fail(ctx, RC_ERR_INVALID_ARG, "rc_render_backward_noalloc: dL_dimage is NULL");
+    st = check_aligned(ctx, dL_dimage, "dL_dimage", "rc_render_backward_noalloc");
+    if (st != RC_OK) return st;
     if (p->func != RC_FUNC_COMPOSITE)
         return fail(ctx, RC_ERR_UNSUPPORTED, "rc_render_backward_noalloc: compositing function only");
     if (tf_entries(ctx) > (size_t)kNoAllocMaxEntries)
@@ -1499,12 +1518,12 @@ rc_status rc_proposal_features(rc_context *ctx, const rc_volume *vol, const rc_r
     return RC_OK;
 }
 
-static rc_status check_net(rc_context *ctx, const void *a, const void *b, int64_t n, const char *who) {
+static rc_status check_net(rc_context *ctx, const void *features, const void *b, int64_t n, const char *who) {
     if (!ctx) return fail(nullptr, RC_ERR_INVALID_ARG, "%s: ctx is NULL", who);
-    if (!a || !b) return fail(ctx, RC_ERR_INVALID_ARG, "%s: NULL buffer", who);
+    if (!features || !b) return fail(ctx, RC_ERR_INVALID_ARG, "%s: NULL buffer", who);
     if (n < 1 || n > (1ll << 31)) return fail(ctx, RC_ERR_INVALID_ARG, "%s: n = %lld", who, (long long)n);
     if (!ctx->net_loaded) return fail(ctx, RC_ERR_STATE, "%s: no network (call rc_proposal_load)", who);
-    return RC_OK;
+    return check_aligned(ctx, features, "features", who);
 }
 
 rc_status rc_proposal_forward(rc_context *ctx, const float *features, int64_t n, float *out) {
@@ -1589,7 +1608,7 @@ static rc_status check_importance(rc_context *ctx, const rc_volume *vol, const r
     if (p->func != RC_FUNC_COMPOSITE) return fail(ctx, RC_ERR_UNSUPPORTED, "%s: compositing function only", who);
     if (nimp < 1 || nimp > 4096) return fail(ctx, RC_ERR_INVALID_ARG, "%s: nimp %d", who, nimp);
     if (!(eps >= 0.0f)) return fail(ctx, RC_ERR_INVALID_ARG, "%s: eps %g", who, (double)eps);
-    return RC_OK;
+    return check_aligned(ctx, out, "out_rgba", who);
 }
 
 static ImportanceArgs importance_args(rc_context *ctx, rc_volume *v, const rc_render_params *p, int nimp, float eps,
