@@ -767,10 +767,35 @@ static rc_status check_views(rc_context *ctx, const rc_camera *cams, int nviews,
     return RC_OK;
 }
 
+static LaunchSizer launch_sizer(const rc_volume *v, const rc_render_params *p) {
+    BoxGeom b;
+    for (int a = 0; a < 3; a++) {
+        b.n[a] = v->n[a];
+        b.s[a] = v->s[a];
+    }
+    return LaunchSizer(b, (double)p->step_vox * fminf(fminf(v->s[0], v->s[1]), v->s[2]));
+}
+
+static ViewGeom view_geom(const CamRec &c) {
+    ViewGeom g;
+    for (int a = 0; a < 3; a++) {
+        g.o[a] = c.o[a];
+        g.f[a] = c.f[a];
+        g.r[a] = c.r[a];
+        g.u[a] = c.u[a];
+    }
+    g.tx = c.tx;
+    g.ty = c.ty;
+    g.W = c.W;
+    g.H = c.H;
+    return g;
+}
+
 // Copies the views' camera records (for volume v) to the context's device
-// array, growing it when needed; *first receives record 0.
+// array, growing it when needed; *first receives record 0, *sizer (or null) the
+// views a launch over all of them is sized by.
 static rc_status upload_views(rc_context *ctx, const rc_volume *v, const rc_camera *cams, int nviews, CamRec *first,
-                              const char *who) {
+                              const char *who, LaunchSizer *sizer = nullptr) {
     if (ctx->cams_cap < nviews) {
         CamRec *buf = nullptr;
         RC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));   // queued kernels may still read the old records
@@ -782,6 +807,7 @@ static rc_status upload_views(rc_context *ctx, const rc_volume *v, const rc_came
     CamRec *recs = new (std::nothrow) CamRec[nviews];
     if (!recs) return fail(ctx, RC_ERR_OOM, "%s: host allocation", who);
     for (int i = 0; i < nviews; i++) recs[i] = camera_record(cams[i], v->s);
+    for (int i = 0; sizer && i < nviews; i += sized_stride(nviews)) sizer->add(view_geom(recs[i]));
     // pageable source: the copy is staged before the call returns
     cudaError_t ce = cudaMemcpyAsync(ctx->d_cams, recs, (size_t)nviews * sizeof(CamRec), cudaMemcpyHostToDevice,
                                      ctx->stream);
@@ -998,6 +1024,9 @@ rc_status rc_render(rc_context *ctx, const rc_volume *vol, const rc_render_param
     st = prepare_filter(ctx, v, p);
     if (st != RC_OK) return st;
     MarchArgs a = march_args(ctx, v, p, out_rgba);
+    LaunchSizer sizer = launch_sizer(v, p);
+    sizer.add(view_geom(a.cam));
+    a.size = sizer.size(1);
     if (stats) {
         RC_CUDA(ctx, stats_begin(ctx));
         a.stats = ctx->d_stats;
@@ -1022,11 +1051,13 @@ rc_status rc_render_views(rc_context *ctx, const rc_volume *vol, const rc_render
     st = prepare_filter(ctx, v, p);
     if (st != RC_OK) return st;
     CamRec first;
-    st = upload_views(ctx, v, cams, nviews, &first, who);
+    LaunchSizer sizer = launch_sizer(v, p);
+    st = upload_views(ctx, v, cams, nviews, &first, who, &sizer);
     if (st != RC_OK) return st;
     MarchArgs a = march_args(ctx, v, p, out_rgba);
     a.cam = first;
     a.cams = ctx->d_cams;
+    a.size = sizer.size(nviews);
     if (stats) {
         RC_CUDA(ctx, stats_begin(ctx));
         a.stats = ctx->d_stats;
@@ -1068,8 +1099,8 @@ constexpr long long kHostGroupPixels = 1ll << 21;
 // render stream (each with its own image buffer), so a group starts while the
 // previous one drains; each group is copied to the host on the copy stream.
 // The context's stream continues after the last copy.
-static rc_status render_groups_to_host(rc_context *ctx, MarchArgs a, int nviews, int g, long long px,
-                                       float *host_rgba) {
+static rc_status render_groups_to_host(rc_context *ctx, MarchArgs a, const rc_volume *v, const rc_render_params *p,
+                                       const rc_camera *cams, int nviews, int g, long long px, float *host_rgba) {
     // the second stream starts after the work queued so far
     RC_CUDA(ctx, cudaEventRecord(ctx->ev_start, ctx->stream));
     RC_CUDA(ctx, cudaStreamWaitEvent(ctx->aux_stream, ctx->ev_start, 0));
@@ -1081,6 +1112,9 @@ static rc_status render_groups_to_host(rc_context *ctx, MarchArgs a, int nviews,
         if (j >= 2) RC_CUDA(ctx, cudaStreamWaitEvent(rs, ctx->ev_copied[b], 0));
         a.cams = ctx->d_cams + v0;
         a.out = ctx->d_img[b];
+        LaunchSizer sizer = launch_sizer(v, p);
+        for (int i = 0; i < nv; i += sized_stride(nv)) sizer.add(view_geom(camera_record(cams[v0 + i], v->s)));
+        a.size = sizer.size(nv);
         RC_CUDA(ctx, launch_march(a, nv, rs));
         RC_CUDA(ctx, cudaEventRecord(ctx->ev_rendered[b], rs));
         RC_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_rendered[b], 0));
@@ -1127,7 +1161,7 @@ rc_status rc_render_views_host(rc_context *ctx, const rc_volume *vol, const rc_r
         RC_CUDA(ctx, stats_begin(ctx));
         a.stats = ctx->d_stats;
     }
-    st = render_groups_to_host(ctx, a, nviews, g, px, host_rgba);
+    st = render_groups_to_host(ctx, a, v, p, cams, nviews, g, px, host_rgba);
     if (st != RC_OK) {
         // no copy into the caller's memory may outlive the call
         cudaStreamSynchronize(ctx->stream);
@@ -1169,7 +1203,8 @@ rc_status rc_render_batch(rc_context *ctx, const rc_volume *const *vols, int nvo
         if (st != RC_OK) return st;
     }
     CamRec first;
-    st = upload_views(ctx, vols[0], cams, nviews, &first, who);
+    LaunchSizer sizer = launch_sizer(vols[0], p);
+    st = upload_views(ctx, vols[0], cams, nviews, &first, who, &sizer);
     if (st != RC_OK) return st;
     if (ctx->batch_cap < nvols) {
         BatchVol *buf = nullptr;
@@ -1192,6 +1227,7 @@ rc_status rc_render_batch(rc_context *ctx, const rc_volume *const *vols, int nvo
     a.cams = ctx->d_cams;
     a.batch = ctx->d_batch;
     a.views = nviews;
+    a.size = sizer.size((double)nvols * nviews);
     if (stats) {
         RC_CUDA(ctx, stats_begin(ctx));
         a.stats = ctx->d_stats;

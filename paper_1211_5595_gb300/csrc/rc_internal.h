@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "rc.h"
+#include "rc_rules.h"
 
 namespace rc {
 
@@ -123,6 +124,7 @@ struct MarchArgs {
     const CamRec *cams;            // one record per view (blockIdx.z), or null: cam
     const BatchVol *batch;         // compositing: blockIdx.z = volume * views + view (or null)
     int views;                     // views per volume of a batch
+    LaunchSize size;               // read on the host: the launch's form is chosen by it
 };
 
 // Adjoint arguments (compositing function only).

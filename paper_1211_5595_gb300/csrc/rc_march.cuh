@@ -6,8 +6,6 @@
 // (rc_march.cu, rc_march_cubic.cu, rc_march_tf2.cu) so they compile in parallel.
 #pragma once
 
-#include <math.h>
-
 #include "rc_device.cuh"
 
 namespace rc {
@@ -478,82 +476,17 @@ static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool ta
     return cudaGetLastError();
 }
 
-// About how many rays of a launch meet the volume: the box's corners bound the
-// part of the image (of the first view) whose rays can, and its silhouette fills
-// about two thirds of that rectangle.
-static double rays_that_hit(const MarchArgs &a, int nviews) {
-    const CamRec &c = a.cam;
-    double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0};
-    for (int q = 0; q < 8; q++) {
-        double z = 0.0, u[2] = {0.0, 0.0};
-        for (int i = 0; i < 3; i++) {
-            const double d = (((q >> i) & 1 ? a.vol.n[i] - 1 : 0) - (double)c.o[i]) * a.vol.s[i];
-            z += d * c.f[i];
-            u[0] += d * c.r[i];
-            u[1] += d * c.u[i];
-        }
-        if (!(z > 0.0)) return 0.65 * c.W * c.H * nviews;      // a corner behind the eye: the whole image
-        const double t[2] = {c.tx, c.ty};
-        for (int i = 0; i < 2; i++) {
-            const double e = u[i] / (z * t[i]);
-            lo[i] = e < lo[i] ? e : lo[i];
-            hi[i] = e > hi[i] ? e : hi[i];
-        }
-    }
-    double part = 0.65;
-    for (int i = 0; i < 2; i++) {
-        const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
-        part *= h > l ? (h - l) * 0.5 : 0.0;
-    }
-    return part * c.W * c.H * nviews;
-}
-
-// Samples across the box's diagonal.
-static double samples_across(const MarchArgs &a) {
-    double diag2 = 0.0;
-    for (int i = 0; i < 3; i++) diag2 += (double)(a.vol.n[i] - 1) * a.vol.s[i] * (a.vol.n[i] - 1) * a.vol.s[i];
-    return sqrt(diag2) / ((double)a.p.step_vox * a.vol.smin);
-}
-
-// Lanes per ray of a launch. A ray's samples are a serial chain (a few hundred
-// of them, 0.3 us each), so a launch with few rays takes the time of its
-// longest ray however few there are; more lanes shorten the chain until the
-// shuffles and the samples past termination fill the GPU. The lines lie where
-// the measured times cross, in rays that meet the volume (`hits`, 0.27 of the
-// pixels there) and per sample across the box (`steps`); us per view with
-// 1, 2, 4 and 8 lanes, FP32 shaded / FP32 plain:
-//   64x64x32, 256^2:    79 58 46 42 / 68 44 35 40
-//   128x128x96, 384^2: 118 107 74 88 / 102 65 66 73
-//   256x256x180, 256^2: 147 102 72 61 / 162 84 58 56
-//   256x256x180, 512^2: 172 142 135 161 / 135 105 99 131
-//   256x256x180, 724^2: 223 201 214 293 / 150 143 162 235
-//   256x256x180, 1024^2: 292 307 386 572 / 193 229 287 456
-// Forms whose samples take longer (shading without 8-byte value+gradient
-// entries, which the FP32 shaded figures above are for; B-spline; 2-D table) gain
-// further up than the others.
-static int lanes_per_ray(const MarchArgs &a, int nviews) {
+static int lanes_per_ray(const MarchArgs &a) {
     if (a.cam.H > 4 * 65535) return 1;     // the grid's y limit at 4 rows per CTA
-    const double hits = rays_that_hit(a, nviews), steps = samples_across(a);
-    const bool heavy = (a.p.shade && !a.vol.vg16) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2;
-    if (hits <= (heavy ? 22e3 : 7e3) && hits <= 70.0 * steps) return 8;
-    if (hits <= 76e3 && hits <= 190.0 * steps) return 4;
-    if (hits <= 155e3 && hits <= (heavy ? 390.0 : 190.0) * steps) return 2;
-    return 1;
+    return lanes_per_ray(a.size, (a.p.shade && !a.vol.vg16) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2);
 }
 
-// Lanes per ray of the sums: every ray marches its whole chord, so no sample is
-// in vain and more lanes pay further up, for the B-spline's long samples always
-// (us with 1, 2 and 4 lanes, FP32 trilinear / B-spline: one 600^2 view of
-// 256x256x180 322 201 131 / 1565 833 580, three 865x878 views of 51x302x86 222
-// 184 204 / 1085 720 672, four 1024^2 views of 256x256x180 1064 1051 1224 / 5592
-// 4842 5112).
-static int lanes_per_sum(const MarchArgs &a, int nviews) {
-    const double hits = rays_that_hit(a, nviews);
-    const bool cubic = a.p.filter == RC_FILTER_BSPLINE;
-    if (hits <= (cubic ? 600e3 : 200e3) && a.cam.H <= 4 * 65535) return 4;
-    return cubic || hits <= 600e3 ? 2 : 1;
+static int lanes_per_sum(const MarchArgs &a) {
+    const int lanes = lanes_per_sum(a.size, a.p.filter == RC_FILTER_BSPLINE);
+    return lanes == 4 && a.cam.H > 4 * 65535 ? 2 : lanes;
 }
- template <int F, int L>
+
+template <int F, int L>
 static cudaError_t launch_wide(const MarchArgs &a, int nviews, cudaStream_t s) {
     const bool smem = !(F & kTF2);
     constexpr int W = kWarpsX * WideTile<L>::X, H = kWarpsY * WideTile<L>::Y;
@@ -575,7 +508,7 @@ static cudaError_t launch_composite_rm(const MarchArgs &a, int nviews, cudaStrea
 // The step ratios of the fixed modes (1, 1/2, 1/4) get their own instances.
 template <int F>
 static cudaError_t launch_composite(const MarchArgs &a, int nviews, cudaStream_t s) {
-    switch (lanes_per_ray(a, nviews)) {
+    switch (lanes_per_ray(a)) {
         case 8: return launch_wide<F, 8>(a, nviews, s);
         case 4: return launch_wide<F, 4>(a, nviews, s);
         case 2: return launch_wide<F, 2>(a, nviews, s);
@@ -610,7 +543,7 @@ static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t 
         case RC_FUNC_MIP: return launch_function_group<CUBIC, kFnMip>(a, nviews, s);
         case RC_FUNC_AVERAGE:
         case RC_FUNC_XRAY:
-            switch (lanes_per_sum(a, nviews)) {
+            switch (lanes_per_sum(a)) {
                 case 4: return launch_sum<CUBIC, 4>(a, nviews, s);
                 case 2: return launch_sum<CUBIC, 2>(a, nviews, s);
                 default: return launch_sum<CUBIC, CUBIC ? 2 : 1>(a, nviews, s);      // the B-spline: 2 at least

@@ -2,6 +2,8 @@
 // without CUDA types, so that they can be compiled and tested by themselves.
 #pragma once
 
+#include <math.h>
+
 namespace rc {
 
 // CTAs of a persistent launch that takes `chunks` pieces of work from a queue,
@@ -10,5 +12,116 @@ namespace rc {
 // each chunk comes first (128x128x96, 32 x 256 table, one 128^2 view of 64
 // chunks: 748 us packed three to a CTA, 674 spread; 2 x 2 table 735 and 615).
 inline int persistent_ctas(int chunks, int sms) { return chunks < sms ? chunks : sms; }
+
+// The camera record's fields that say where the volume's box lies in an image.
+struct ViewGeom {
+    double o[3], f[3], r[3], u[3];     // eye (index space), view basis (world)
+    double tx, ty;                     // tangents of the half angles
+    int W, H;
+};
+
+struct BoxGeom {
+    int n[3];                          // voxels
+    double s[3];                       // spacing
+};
+
+// About how many rays of a view meet the volume: the box's corners bound the
+// part of the image whose rays can, and its silhouette fills about two thirds
+// of that rectangle.
+inline double view_rays(const ViewGeom &c, const BoxGeom &b) {
+    double hits = 0.65 * c.W * c.H;
+    double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0};
+    for (int q = 0; q < 8; q++) {
+        double z = 0.0, e[2] = {0.0, 0.0};
+        for (int i = 0; i < 3; i++) {
+            const double d = (((q >> i) & 1 ? b.n[i] - 1 : 0) - c.o[i]) * b.s[i];
+            z += d * c.f[i];
+            e[0] += d * c.r[i];
+            e[1] += d * c.u[i];
+        }
+        if (!(z > 0.0)) return hits;                       // a corner behind the eye: the whole image
+        e[0] /= z * c.tx;
+        e[1] /= z * c.ty;
+        for (int i = 0; i < 2; i++) {
+            lo[i] = e[i] < lo[i] ? e[i] : lo[i];
+            hi[i] = e[i] > hi[i] ? e[i] : hi[i];
+        }
+    }
+    for (int i = 0; i < 2; i++) {
+        const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
+        hits *= h > l ? (h - l) * 0.5 : 0.0;
+    }
+    return hits;
+}
+
+// The size of a march launch over all its views: rays that meet the volume and
+// samples across the box's diagonal. The views are summed (up to kSizedViews of them,
+// evenly spread): the first one alone says nothing about the others. Eight
+// 1024^2 views of 256x256x180, unshaded, took 3.37 ms instead of 1.14 when the
+// first of them looked past the volume, and 2.07 when it was far away.
+struct LaunchSize {
+    double hits = 0.0, steps = 0.0;
+};
+constexpr int kSizedViews = 32;
+inline int sized_stride(int views) { return (views + kSizedViews - 1) / kSizedViews; }
+
+class LaunchSizer {
+  public:
+    LaunchSizer(const BoxGeom &b, double step) : box(b) {      // step: sample distance (world)
+        double diag2 = 0.0;
+        for (int i = 0; i < 3; i++) diag2 += (b.n[i] - 1) * b.s[i] * (b.n[i] - 1) * b.s[i];
+        across = sqrt(diag2) / step;
+    }
+    void add(const ViewGeom &c) {
+        hits += view_rays(c, box);
+        added++;
+    }
+    // for `views` views of which the added ones are a sample
+    LaunchSize size(double views) const {
+        LaunchSize z;
+        z.hits = added ? hits * views / added : 0.0;
+        z.steps = across;
+        return z;
+    }
+
+  private:
+    BoxGeom box;
+    double across, hits = 0.0;
+    int added = 0;
+};
+
+// Lanes per ray of a compositing launch. A ray's samples are a serial chain (a
+// few hundred of them, 0.3 us each), so a launch with few rays takes the time of
+// its longest ray however few there are; more lanes shorten the chain until the
+// shuffles and the samples past termination fill the GPU. The lines lie where
+// the measured times cross, in rays that meet the volume (`hits`, 0.27 of the
+// pixels there) and per sample across the box (`steps`); us per view with
+// 1, 2, 4 and 8 lanes, FP32 shaded / FP32 plain:
+//   64x64x32, 256^2:    79 58 46 42 / 68 44 35 40
+//   128x128x96, 384^2: 118 107 74 88 / 102 65 66 73
+//   256x256x180, 256^2: 147 102 72 61 / 162 84 58 56
+//   256x256x180, 512^2: 172 142 135 161 / 135 105 99 131
+//   256x256x180, 724^2: 223 201 214 293 / 150 143 162 235
+//   256x256x180, 1024^2: 292 307 386 572 / 193 229 287 456
+// `heavy`: forms whose samples take longer (shading without 8-byte
+// value+gradient entries, which the FP32 shaded figures above are for;
+// B-spline; 2-D table) gain further up than the others.
+inline int lanes_per_ray(const LaunchSize &z, bool heavy) {
+    if (z.hits <= (heavy ? 22e3 : 7e3) && z.hits <= 70.0 * z.steps) return 8;
+    if (z.hits <= 76e3 && z.hits <= 190.0 * z.steps) return 4;
+    if (z.hits <= 155e3 && z.hits <= (heavy ? 390.0 : 190.0) * z.steps) return 2;
+    return 1;
+}
+
+// Lanes per ray of the sums: every ray marches its whole chord, so no sample is
+// in vain and more lanes pay further up, for the B-spline's long samples always
+// (us with 1, 2 and 4 lanes, FP32 trilinear / B-spline: one 600^2 view of
+// 256x256x180 322 201 131 / 1565 833 580, three 865x878 views of 51x302x86 222
+// 184 204 / 1085 720 672, four 1024^2 views of 256x256x180 1064 1051 1224 / 5592
+// 4842 5112).
+inline int lanes_per_sum(const LaunchSize &z, bool cubic) {
+    if (z.hits <= (cubic ? 600e3 : 200e3)) return 4;
+    return cubic || z.hits <= 600e3 ? 2 : 1;
+}
 
 }  // namespace rc

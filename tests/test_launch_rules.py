@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1211_5595_gb300", "csrc")
@@ -12,6 +13,34 @@ SHIM = r"""
 #include "rc_rules.h"
 extern "C" {
 int persistent_ctas(int chunks, int sms) { return rc::persistent_ctas(chunks, sms); }
+// rays and samples of `n` views (records of 16 doubles: eye, basis, tangents, size)
+void launch_size(const int *dims, const double *spacing, double step, const double *views, int n, double *out) {
+    rc::BoxGeom b;
+    for (int i = 0; i < 3; i++) { b.n[i] = dims[i]; b.s[i] = spacing[i]; }
+    rc::LaunchSizer z(b, step);
+    for (int i = 0; i < n; i += rc::sized_stride(n)) {
+        const double *q = views + 16 * i;
+        rc::ViewGeom c;
+        for (int a = 0; a < 3; a++) { c.o[a] = q[a]; c.f[a] = q[3 + a]; c.r[a] = q[6 + a]; c.u[a] = q[9 + a]; }
+        c.tx = q[12]; c.ty = q[13]; c.W = (int)q[14]; c.H = (int)q[15];
+        z.add(c);
+    }
+    const rc::LaunchSize s = z.size(n);
+    out[0] = s.hits;
+    out[1] = s.steps;
+}
+int lanes_per_ray(double hits, double steps, int heavy) {
+    rc::LaunchSize z;
+    z.hits = hits;
+    z.steps = steps;
+    return rc::lanes_per_ray(z, heavy != 0);
+}
+int lanes_per_sum(double hits, double steps, int cubic) {
+    rc::LaunchSize z;
+    z.hits = hits;
+    z.steps = steps;
+    return rc::lanes_per_sum(z, cubic != 0);
+}
 }
 """
 
@@ -25,7 +54,35 @@ def rules(tmp_path_factory):
     (d / "shim.cpp").write_text(SHIM)
     subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC,
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
-    return C.CDLL(str(d / "shim.so"))
+    lib = C.CDLL(str(d / "shim.so"))
+    lib.lanes_per_ray.argtypes = lib.lanes_per_sum.argtypes = [C.c_double, C.c_double, C.c_int]
+    return lib
+
+
+def view(dims, spacing, eye, target, size, fovy=30.0, up=(0.0, 0.0, 1.0)):
+    f = np.subtract(target, eye)
+    f = f / np.linalg.norm(f)
+    r = np.cross(f, up)
+    r = r / np.linalg.norm(r)
+    th = np.tan(np.radians(fovy) / 2)
+    return np.concatenate([np.divide(eye, spacing), f, r, np.cross(r, f), [th * size[0] / size[1], th, *size]])
+
+
+def launch_size(rules, dims, spacing, step, views):
+    v = np.ascontiguousarray(np.stack(views), dtype=np.float64)
+    out = (C.c_double * 2)()
+    rules.launch_size((C.c_int * 3)(*dims), (C.c_double * 3)(*spacing), C.c_double(step),
+                      v.ctypes.data_as(C.POINTER(C.c_double)), len(views), out)
+    return out[0], out[1]
+
+
+DIMS, ONES = (256, 256, 180), (1.0, 1.0, 1.0)
+CENTRE = (127.5, 127.5, 89.5)
+
+
+def orbit(n, size, dist=800.0):
+    a = np.radians(12.0 + 360.0 * np.arange(n) / n)
+    return [view(DIMS, ONES, (127.5 + dist * np.cos(x), 127.5 + dist * np.sin(x), 89.5 + 0.35 * dist), CENTRE, size) for x in a]
 
 
 # a chunk gets an SM of its own before two share one
@@ -33,3 +90,27 @@ def rules(tmp_path_factory):
                                          (1 << 27, 152)])
 def test_a_small_image_spreads_over_the_sms(rules, chunks, ctas):
     assert rules.persistent_ctas(chunks, 152) == ctas
+
+
+# a view that looks past the volume or stands far from it changes a launch's
+# size by its own rays only, wherever it stands among the views
+@pytest.mark.parametrize("other", [view(DIMS, ONES, (827.5, 127.5, 89.5), (327.5, 1027.5, 89.5), (1024, 1024)),
+                                   view(DIMS, ONES, (9127.5, 127.5, 89.5), CENTRE, (1024, 1024))])
+def test_every_view_counts(rules, other):
+    views = orbit(7, (1024, 1024))
+    base, steps = launch_size(rules, DIMS, ONES, 0.5, views)
+    assert 150e3 * 7 < base < 600e3 * 7
+    for at in (0, 3, 7):
+        hits, s = launch_size(rules, DIMS, ONES, 0.5, views[:at] + [other] + views[at:])
+        assert abs(hits - base) < 5e3 and s == steps
+        assert rules.lanes_per_ray(hits, s, 0) == 1 and rules.lanes_per_sum(hits, s, 0) == 1
+    alone, s = launch_size(rules, DIMS, ONES, 0.5, [other])
+    assert alone < 5e3 and rules.lanes_per_ray(alone, s, 0) == 8
+
+
+# many views are sized by a spread sample of them
+def test_many_views_are_sampled(rules):
+    one, steps = launch_size(rules, DIMS, ONES, 0.5, orbit(1, (64, 64)))
+    for n in (32, 33, 1000, 65535):
+        hits, s = launch_size(rules, DIMS, ONES, 0.5, orbit(n, (64, 64)))
+        assert s == steps and 0.7 * n * one < hits < 1.4 * n * one
