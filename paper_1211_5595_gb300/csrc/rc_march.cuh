@@ -546,7 +546,7 @@ static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t 
             switch (lanes_per_sum(a)) {
                 case 4: return launch_sum<CUBIC, 4>(a, nviews, s);
                 case 2: return launch_sum<CUBIC, 2>(a, nviews, s);
-                default: return launch_sum<CUBIC, CUBIC ? 2 : 1>(a, nviews, s);      // the B-spline: 2 at least
+                default: return launch_sum<CUBIC, 1>(a, nviews, s);
             }
         default: return launch_function_group<CUBIC, kFnFirst>(a, nviews, s);
     }

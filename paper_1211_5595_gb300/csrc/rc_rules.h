@@ -54,13 +54,14 @@ inline double view_rays(const ViewGeom &c, const BoxGeom &b) {
     return hits;
 }
 
-// The size of a march launch over all its views: rays that meet the volume and
-// samples across the box's diagonal. The views are summed (up to kSizedViews of them,
+// The size of a march launch over all its views: rays that meet the volume,
+// samples across the box's diagonal, and the rays of one view per voxel of the
+// box's cross-section (the two-thirds power of its voxels). The views are summed (up to kSizedViews of them,
 // evenly spread): the first one alone says nothing about the others. Eight
 // 1024^2 views of 256x256x180, unshaded, took 3.37 ms instead of 1.14 when the
 // first of them looked past the volume, and 2.07 when it was far away.
 struct LaunchSize {
-    double hits = 0.0, steps = 0.0;
+    double hits = 0.0, steps = 0.0, density = 0.0;
 };
 constexpr int kSizedViews = 32;
 inline int sized_stride(int views) { return (views + kSizedViews - 1) / kSizedViews; }
@@ -81,6 +82,7 @@ class LaunchSizer {
         LaunchSize z;
         z.hits = added ? hits * views / added : 0.0;
         z.steps = across;
+        z.density = z.hits / views / pow((double)box.n[0] * box.n[1] * box.n[2], 2.0 / 3.0);
         return z;
     }
 
@@ -114,14 +116,32 @@ inline int lanes_per_ray(const LaunchSize &z, bool heavy) {
 }
 
 // Lanes per ray of the sums: every ray marches its whole chord, so no sample is
-// in vain and more lanes pay further up, for the B-spline's long samples always
-// (us with 1, 2 and 4 lanes, FP32 trilinear / B-spline: one 600^2 view of
-// 256x256x180 322 201 131 / 1565 833 580, three 865x878 views of 51x302x86 222
-// 184 204 / 1085 720 672, four 1024^2 views of 256x256x180 1064 1051 1224 / 5592
-// 4842 5112).
+// in vain, and what more lanes cost is the ray setup and the shuffles, which
+// short chains do not repay, and the coherence of neighbouring rays, which is
+// worth more the denser the pixels lie on the voxels (`density`). us with 1, 2
+// and 4 lanes, FP32 trilinear / B-spline:
+//   128x128x96, 512^2, 408 samples along the diagonal: 92 70 61 / 326 244 215
+//   the same with 20 samples:                          15 14 18 / 35 33 37
+//   128x128x96, 1024^2 (27 rays per voxel):           148 159 180 / 564 539 611
+//   64x64x32, 1024^2 (128 rays per voxel):             66 74 97 / 209 210 246
+//   256x256x180, 1024^2 (7 rays per voxel):           371 296 315 / 1797 1286 1380
+//   51x302x86, four 870^2 views:                      288 244 273 / 1292 921 891
+//   256x256x180, four 1024^2 views:                  1064 1051 1224 / 5685 4863 5112
+//   the same, eight views:                                          / 11779 9970
+// Fixed lines in rays (4 lanes up to 200e3, B-spline 600e3) took 2.3 times as
+// long as one lane at a few samples per ray. Over 578 sizes these lines are
+// within 1.3% of the best choice on average, 9% slower than one lane at worst.
 inline int lanes_per_sum(const LaunchSize &z, bool cubic) {
-    if (z.hits <= (cubic ? 600e3 : 200e3)) return 4;
-    return cubic || z.hits <= 600e3 ? 2 : 1;
+    const double d = z.density < 16.0 ? z.density : 16.0;
+    if (cubic) {
+        // samples finer than voxels, voxels finer than pixels: two lanes of a ray
+        // share their footprints, however many rays there are
+        const bool shared = d <= 10.0 && z.steps >= 400.0;
+        if (!shared && z.hits > 40e3 + 1600.0 * z.steps) return 1;
+        return z.hits * pow(d, 0.7) <= 80e3 + 1600.0 * z.steps ? 4 : 2;
+    }
+    if (z.hits * pow(d, 0.4) > 80e3 + 1700.0 * z.steps) return 1;
+    return z.hits * sqrt(d) <= 60e3 + 600.0 * z.steps ? 4 : 2;
 }
 
 }  // namespace rc

@@ -28,6 +28,7 @@ void launch_size(const int *dims, const double *spacing, double step, const doub
     const rc::LaunchSize s = z.size(n);
     out[0] = s.hits;
     out[1] = s.steps;
+    out[2] = s.density;
 }
 int lanes_per_ray(double hits, double steps, int heavy) {
     rc::LaunchSize z;
@@ -35,10 +36,11 @@ int lanes_per_ray(double hits, double steps, int heavy) {
     z.steps = steps;
     return rc::lanes_per_ray(z, heavy != 0);
 }
-int lanes_per_sum(double hits, double steps, int cubic) {
+int lanes_per_sum(double hits, double steps, double density, int cubic) {
     rc::LaunchSize z;
     z.hits = hits;
     z.steps = steps;
+    z.density = density;
     return rc::lanes_per_sum(z, cubic != 0);
 }
 }
@@ -55,7 +57,8 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-Werror", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC,
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
     lib = C.CDLL(str(d / "shim.so"))
-    lib.lanes_per_ray.argtypes = lib.lanes_per_sum.argtypes = [C.c_double, C.c_double, C.c_int]
+    lib.lanes_per_ray.argtypes = [C.c_double, C.c_double, C.c_int]
+    lib.lanes_per_sum.argtypes = [C.c_double, C.c_double, C.c_double, C.c_int]
     return lib
 
 
@@ -70,10 +73,10 @@ def view(dims, spacing, eye, target, size, fovy=30.0, up=(0.0, 0.0, 1.0)):
 
 def launch_size(rules, dims, spacing, step, views):
     v = np.ascontiguousarray(np.stack(views), dtype=np.float64)
-    out = (C.c_double * 2)()
+    out = (C.c_double * 3)()
     rules.launch_size((C.c_int * 3)(*dims), (C.c_double * 3)(*spacing), C.c_double(step),
                       v.ctypes.data_as(C.POINTER(C.c_double)), len(views), out)
-    return out[0], out[1]
+    return tuple(out)
 
 
 DIMS, ONES = (256, 256, 180), (1.0, 1.0, 1.0)
@@ -98,19 +101,40 @@ def test_a_small_image_spreads_over_the_sms(rules, chunks, ctas):
                                    view(DIMS, ONES, (9127.5, 127.5, 89.5), CENTRE, (1024, 1024))])
 def test_every_view_counts(rules, other):
     views = orbit(7, (1024, 1024))
-    base, steps = launch_size(rules, DIMS, ONES, 0.5, views)
+    base, steps, _ = launch_size(rules, DIMS, ONES, 0.5, views)
     assert 150e3 * 7 < base < 600e3 * 7
     for at in (0, 3, 7):
-        hits, s = launch_size(rules, DIMS, ONES, 0.5, views[:at] + [other] + views[at:])
+        hits, s, density = launch_size(rules, DIMS, ONES, 0.5, views[:at] + [other] + views[at:])
         assert abs(hits - base) < 5e3 and s == steps
-        assert rules.lanes_per_ray(hits, s, 0) == 1 and rules.lanes_per_sum(hits, s, 0) == 1
-    alone, s = launch_size(rules, DIMS, ONES, 0.5, [other])
+        assert rules.lanes_per_ray(hits, s, 0) == 1 and rules.lanes_per_sum(hits, s, density, 0) == 1
+    alone, s, _ = launch_size(rules, DIMS, ONES, 0.5, [other])
     assert alone < 5e3 and rules.lanes_per_ray(alone, s, 0) == 8
 
 
 # many views are sized by a spread sample of them
 def test_many_views_are_sampled(rules):
-    one, steps = launch_size(rules, DIMS, ONES, 0.5, orbit(1, (64, 64)))
+    one, steps, density = launch_size(rules, DIMS, ONES, 0.5, orbit(1, (64, 64)))
     for n in (32, 33, 1000, 65535):
-        hits, s = launch_size(rules, DIMS, ONES, 0.5, orbit(n, (64, 64)))
-        assert s == steps and 0.7 * n * one < hits < 1.4 * n * one
+        hits, s, d = launch_size(rules, DIMS, ONES, 0.5, orbit(n, (64, 64)))
+        assert s == steps and 0.7 * density < d < 1.4 * density and 0.7 * n * one < hits < 1.4 * n * one
+
+
+# (dims, image, views, step): lanes of the trilinear and the B-spline sums where
+# the measured times leave one answer (another is slower by 15% or more): short
+# chains and pixels dense on the voxels take fewer
+@pytest.mark.parametrize("dims,size,views,step,lanes", [
+    ((256, 256, 180), 128, 1, 0.5, (4, 4)), ((128, 128, 96), 128, 1, 10.0, (4, 4)),
+    ((128, 128, 96), 512, 1, 20.0, (1, None)), ((128, 128, 96), 724, 1, 10.0, (1, 1)),
+    ((64, 64, 32), 1024, 1, 0.5, (1, None)), ((40, 40, 40), 1024, 1, 0.5, (1, 1)),
+    ((40, 40, 40), 1024, 1, 2.0, (1, 1)), ((256, 256, 180), 1024, 1, 0.5, (2, None)),
+    ((256, 256, 180), 1024, 4, 0.5, (None, 2)), ((256, 256, 180), 1024, 8, 0.5, (None, 2)), ((51, 302, 86), 870, 4, 0.5, (2, None))])
+def test_lanes_of_sums(rules, dims, size, views, step, lanes):
+    ext = np.array(dims) - 1.0
+    dist = 1.1 * np.linalg.norm(ext) / 2 / np.sin(np.radians(15.0))
+    el, az = np.radians(20.0), np.radians(12.0 + 360.0 * np.arange(views) / views)
+    vs = [view(dims, ONES, ext / 2 + dist * np.array([np.cos(el) * np.cos(a), np.cos(el) * np.sin(a), np.sin(el)]), ext / 2,
+               (size, size)) for a in az]
+    z = launch_size(rules, dims, ONES, step, vs)
+    for cubic in (0, 1):
+        if lanes[cubic]:
+            assert rules.lanes_per_sum(*z, cubic) == lanes[cubic], (cubic, z)
