@@ -111,8 +111,9 @@ typedef struct {
     float ka, kd, ks;   /* shading weights; specular exponent 16 */
     int32_t func;       /* rc_ray_function */
     float iso;          /* iso-value / threshold, in the volume's code units */
-    int32_t skip;       /* 1: skip bricks the occupancy mask marks empty (exact); MIP, ISO and
-                           THRESHOLD skip blocks whose largest code cannot matter (exact) */
+    int32_t skip;       /* 1: skip bricks the occupancy mask marks empty (exact); ISO and
+                           THRESHOLD skip blocks whose largest code is below iso (exact);
+                           no effect on the others */
     int32_t filter;     /* rc_filter (0: trilinear) */
 } rc_render_params;
 

@@ -924,10 +924,11 @@ static rc_status ensure_occupancy(rc_context *ctx, rc_volume *v, int f) {
 }
 
 // What a render's empty-space skipping reads: the occupancy masks for
-// compositing, the block maxima for MIP and the first-hit functions.
+// compositing, the block maxima for the first-hit functions.
 static rc_status ensure_skip(rc_context *ctx, rc_volume *v, const rc_render_params *p) {
-    if (!p->skip || p->func == RC_FUNC_AVERAGE || p->func == RC_FUNC_XRAY) return RC_OK;
-    return p->func == RC_FUNC_COMPOSITE ? ensure_occupancy(ctx, v, p->filter) : ensure_grid(ctx, v, p->filter);
+    if (!p->skip) return RC_OK;
+    if (p->func == RC_FUNC_COMPOSITE) return ensure_occupancy(ctx, v, p->filter);
+    return p->func == RC_FUNC_ISO || p->func == RC_FUNC_THRESHOLD ? ensure_grid(ctx, v, p->filter) : RC_OK;
 }
 
 // Copies the device counters into *stats (synchronises the stream). The

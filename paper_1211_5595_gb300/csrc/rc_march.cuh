@@ -246,10 +246,6 @@ __global__ void __launch_bounds__(kMarchThreads) wide_kernel(const MarchArgs a) 
     }
 }
 
-// Ray function groups of function_kernel: MIP | isosurface, threshold (average
-// and x-ray: sum_kernel).
-enum : int { kFnMip = 0, kFnFirst = 2 };
-
 // The largest block around cell c (brick b) whose codes cannot matter, none of
 // them above `need`: 4 for the cell-brick, 2 for the 4^3 sub-block, -1 when the
 // sample has to be evaluated. need is a threshold in code units less a.slack,
@@ -264,32 +260,23 @@ __device__ __forceinline__ int low_block(const MarchArgs &a, const Cell &c, int 
     return (int)__ldg(a.mx + b) > need ? 2 : 4;
 }
 
-// The other ray functions of Sec. 4.1 (MIP, average, x-ray, isosurface,
-// threshold); output channels as documented in rc.h. CUBIC: B-spline values
-// and analytic gradient instead of trilinear values and central differences.
+// The first-hit functions of Sec. 4.1 (isosurface, threshold); output channels
+// as documented in rc.h. CUBIC: B-spline values and analytic gradient instead
+// of trilinear values and central differences.
 //
-// MIP and the first-hit functions march the block maxima instead of every
-// sample: a sample in a 4^3 sub-block or cell-brick whose largest code cannot
-// exceed the ray's maximum so far (or reach the iso-value) changes nothing, so
-// the ray jumps over the block (the compositing march's exact jump, verified
-// on the sample grid). A warp jumps only when none of its lanes has to
+// They march the block maxima instead of every sample: a sample in a 4^3
+// sub-block or cell-brick whose largest code cannot reach the iso-value changes
+// nothing, so the ray jumps over the block (the compositing march's exact jump,
+// verified on the sample grid). A warp jumps only when none of its lanes has to
 // evaluate: in noise the lanes' blocks alternate, and a jump costs more than
-// the sample it saves. The maximum does not depend on the order, so MIP first
-// takes samples eight voxels apart and so starts from nearly the ray's
-// maximum, with the space in front of the brightest tissue to skip as well.
-// The value before a first hit is reconstructed once, when the hit is found.
-// Instruction issue bounds it (76% with every sample evaluated, L1 54%, DRAM
-// 3%). 256x256x180 phantom at 1024^2: 4 isosurface views 0.725 -> 0.253 ms,
-// 8 MIP views 2.44 -> 2.00 ms (the noise around the head has block maxima
-// above any value reconstructed in it, so 60% of the samples stay). Of the MIP
-// forms tried when the rest of the march took 2.15: jumping lane by lane instead
-// of by warp 2.55, with samples four voxels apart first 2.60; a branch on a new
-// maximum instead of the plain update 2% slower.
-template <int ST, bool CUBIC, int FN>
+// the sample it saves. The value before a hit is reconstructed once, when the
+// hit is found. Instruction issue bounds it. 256x256x180 phantom at 1024^2, 4
+// isosurface views: 0.725 -> 0.253 ms.
+template <int ST, bool CUBIC>
 __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs a) {
     extern __shared__ float4 s_tf[];
     const int func = a.p.func;
-    if (FN == kFnFirst && func == RC_FUNC_THRESHOLD) {   // the only one that classifies (1-D table)
+    if (func == RC_FUNC_THRESHOLD) {   // the only one that classifies (1-D table)
         load_tf(a.tf, s_tf);
         __syncthreads();
     }
@@ -302,34 +289,17 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
     const bool hit = inimg && setup_ray(cam, a.vol, a.p.step_vox, x, y, R);
     const int nsamp = hit ? R.nsamp : 0;
     float4 out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float acc = FN == kFnMip ? -__int_as_float(0x7f800000) : 0.0f;
     int k = 0;
     unsigned evald = 0;
     int hit_k = -1;
     auto value = [&](const Cell &c) { return CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c); };
-    // thresholds in code units: FP16 storage holds h = code / o - 1
-    auto in_codes = [&](float v) { return ST == RC_STORE_F16 ? (v + 1.0f) * a.vol.f16o : v; };
-    auto bound = [&](float v) { return __float2int_rd(in_codes(v) - a.slack); };
-    int need = bound(FN == kFnFirst ? a.p.iso : acc);
+    // the threshold in code units (FP16 storage holds h = code / o - 1)
+    const int need = __float2int_rd((ST == RC_STORE_F16 ? (a.p.iso + 1.0f) * a.vol.f16o : a.p.iso) - a.slack);
     auto cell_at = [&](int j, Cell &c) {
         float p[3];
         position_at(R, sample_t(R, j), p);
         cell_of(a.vol, p, c);
     };
-    if (FN == kFnMip && a.p.skip) {
-        const int stride = (int)fminf(8.0f / a.p.step_vox, 4096.0f);
-        for (int j = stride >> 1; stride > 1 && j < nsamp; j += stride) {
-            Cell c;
-            cell_at(j, c);
-            if (low_block(a, c, brick_of(a.vol, c), need) >= 0) continue;
-            const float v = value(c);
-            evald++;
-            if (v > acc) {
-                acc = v;
-                need = bound(v);
-            }
-        }
-    }
     bool active = nsamp > 0;
     while (__any_sync(kFull, active)) {
         Cell c0, c1;
@@ -350,11 +320,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
         cell_at(k + 1, c1);
         const float v0 = value(c0), v1 = value(c1);
         const bool two = k + 1 < nsamp;
-        if (FN == kFnMip) {
-            acc = fmaxf(acc, v0);
-            if (two) acc = fmaxf(acc, v1);
-            need = bound(acc);
-        } else if (v0 >= a.p.iso || (two && v1 >= a.p.iso)) {
+        if (v0 >= a.p.iso || (two && v1 >= a.p.iso)) {
             if (!(v0 >= a.p.iso)) {
                 k++;
                 evald++;
@@ -368,7 +334,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
         evald += two ? 2 : 1;
         active = k < nsamp;
     }
-    if (FN == kFnFirst && hit_k >= 0) {
+    if (hit_k >= 0) {
         // the hit's value again, and for an isosurface the value before it
         const float t = sample_t(R, hit_k);
         Cell c;
@@ -394,24 +360,23 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
         }
     }
     k = min(k, nsamp);
-    if (FN == kFnMip && nsamp > 0) {
-        // over full scale; FP16 values h = (code - o) / o are shifted by 1 first
-        // (code / vmax = (h + 1) / vscale)
-        const float m = (ST == RC_STORE_F16 ? acc + 1.0f : acc) / a.vol.vscale;
-        out = make_float4(m, m, m, 1.0f);
-    }
     if (inimg) outp[(size_t)y * cam.W + x] = out;
-    // a sample that MIP took in its first pass too counts once
-    if (a.stats) add_stats(a.stats, (unsigned)k, min(evald, (unsigned)k), hit ? 1u : 0u, inimg ? 1u : 0u);
+    if (a.stats) add_stats(a.stats, (unsigned)k, evald, hit ? 1u : 0u, inimg ? 1u : 0u);
 }
 
-// Average and x-ray: the sum of every sample, in sample order. L lanes per ray
-// as in wide_kernel: lane j reconstructs sample k + j and the
-// group adds the L values in order from shuffles (the same sum bit for bit; the
-// measured times stand at lanes_per_sum). Bound by instruction issue, for the
-// B-spline by its chain of gathers.
-template <int ST, bool CUBIC, int L>
-__global__ void __launch_bounds__(kMarchThreads) sum_kernel(const MarchArgs a) {
+// Average, x-ray and (MAX) MIP: the sum or the maximum of every sample. L lanes
+// per ray as in wide_kernel: lane j reconstructs sample k + j and the group adds
+// the L values in sample order from shuffles (the same sum bit for bit); a
+// maximum does not depend on the order, so each lane keeps its own to the end.
+// The measured times stand at lanes_per_sum and lanes_per_max. Bound by
+// instruction issue, for the B-spline by its chain of gathers.
+// MIP takes every sample: in noise the maxima of 4^3 blocks lie above any value
+// reconstructed in them, so skipping by them (as function_kernel does) left 60%
+// of the samples of a head phantom and a longer chain per sample. One 128^2 view
+// of 256x256x180, us: 304 with skipping, 171 with one lane and every sample, 43
+// with the lanes; eight 1024^2 views 1992, 2188 and 1984.
+template <int ST, bool CUBIC, int L, bool MAX>
+__global__ void __launch_bounds__(kMarchThreads) reduce_kernel(const MarchArgs a) {
     const CamRec cam = a.cams ? a.cams[blockIdx.z] : a.cam;
     float4 *outp = a.out + (size_t)blockIdx.z * cam.W * cam.H;
     constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
@@ -422,7 +387,7 @@ __global__ void __launch_bounds__(kMarchThreads) sum_kernel(const MarchArgs a) {
     Ray R;
     const bool hit = inimg && setup_ray(cam, a.vol, a.p.step_vox, x, y, R);
     const int nsamp = hit ? R.nsamp : 0;
-    float acc = 0.0f;
+    float acc = MAX ? -__int_as_float(0x7f800000) : 0.0f;
     auto value = [&](int k) {
         float p[3];
         position_at(R, sample_t(R, k), p);
@@ -430,7 +395,13 @@ __global__ void __launch_bounds__(kMarchThreads) sum_kernel(const MarchArgs a) {
         cell_of(a.vol, p, c);
         return CUBIC ? bspline<ST>(a.vol, c) : trilinear<ST>(a.vol, c);
     };
-    if constexpr (L == 1) {
+    if constexpr (MAX) {
+#pragma unroll 1
+        for (int k = j; k < nsamp; k += L) acc = fmaxf(acc, value(k));
+        __syncwarp();
+#pragma unroll
+        for (int i = 1; i < L; i <<= 1) acc = fmaxf(acc, __shfl_xor_sync(kFull, acc, i));
+    } else if constexpr (L == 1) {
 #pragma unroll 1
         for (int k = 0; k < nsamp; k++) acc += value(k);
     } else {
@@ -444,12 +415,15 @@ __global__ void __launch_bounds__(kMarchThreads) sum_kernel(const MarchArgs a) {
             }
         }
     }
-    // over full scale; FP16 values h = code / o - 1 are shifted by 1 per sample first
+    // over full scale; FP16 values h = code / o - 1 are shifted by 1 (a sum's by 1
+    // per sample) first
     float4 out = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (nsamp > 0) {
         const float n = (float)nsamp;
         float m;
-        if (ST == RC_STORE_F16)
+        if (MAX)
+            m = (ST == RC_STORE_F16 ? acc + 1.0f : acc) / a.vol.vscale;
+        else if (ST == RC_STORE_F16)
             m = a.p.func == RC_FUNC_AVERAGE ? (acc / n + 1.0f) / a.vol.vscale : (acc + n) * R.ds / a.vol.vscale;
         else
             m = a.p.func == RC_FUNC_AVERAGE ? acc / n / a.vol.vscale : acc * R.ds / a.vol.vscale;
@@ -479,11 +453,6 @@ static cudaError_t launch_kernel(K kern, const MarchArgs &a, int nviews, bool ta
 static int lanes_per_ray(const MarchArgs &a) {
     if (a.cam.H > 4 * 65535) return 1;     // the grid's y limit at 4 rows per CTA
     return lanes_per_ray(a.size, (a.p.shade && !a.vol.vg16) || a.p.filter == RC_FILTER_BSPLINE || a.tf.M >= 2);
-}
-
-static int lanes_per_sum(const MarchArgs &a) {
-    const int lanes = lanes_per_sum(a.size, a.p.filter == RC_FILTER_BSPLINE);
-    return lanes == 4 && a.cam.H > 4 * 65535 ? 2 : lanes;
 }
 
 template <int F, int L>
@@ -521,34 +490,37 @@ static cudaError_t launch_composite(const MarchArgs &a, int nviews, cudaStream_t
     }
 }
 
-template <bool CUBIC, int FN>
-static cudaError_t launch_function_group(const MarchArgs &a, int nviews, cudaStream_t s) {
-    const bool smem = a.p.func == RC_FUNC_THRESHOLD;
+template <bool CUBIC, bool MAX, int L>
+static cudaError_t launch_reduce_lanes(const MarchArgs &a, int nviews, cudaStream_t s) {
+    constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
     return by_storage<false>(a.vol, [&](auto st) {
-        return launch_kernel(function_kernel<decltype(st)::value, CUBIC, FN>, a, nviews, smem, s);
+        return launch_kernel(reduce_kernel<decltype(st)::value, CUBIC, L, MAX>, a, nviews, false, s, kWarpsX * TX,
+                             kWarpsY * TY);
     });
 }
 
-template <bool CUBIC, int L>
-static cudaError_t launch_sum(const MarchArgs &a, int nviews, cudaStream_t s) {
-    constexpr int TX = WideTile<L>::X, TY = WideTile<L>::Y;
-    return by_storage<false>(a.vol, [&](auto st) {
-        return launch_kernel(sum_kernel<decltype(st)::value, CUBIC, L>, a, nviews, false, s, kWarpsX * TX, kWarpsY * TY);
-    });
+template <bool CUBIC, bool MAX>
+static cudaError_t launch_reduce(const MarchArgs &a, int nviews, cudaStream_t s) {
+    int lanes = MAX ? lanes_per_max(a.size, CUBIC) : lanes_per_sum(a.size, CUBIC);
+    if (lanes == 4 && a.cam.H > 4 * 65535) lanes = 2;      // the grid's y limit at 4 rows per CTA
+    switch (lanes) {
+        case 4: return launch_reduce_lanes<CUBIC, MAX, 4>(a, nviews, s);
+        case 2: return launch_reduce_lanes<CUBIC, MAX, 2>(a, nviews, s);
+        default: return launch_reduce_lanes<CUBIC, MAX, 1>(a, nviews, s);
+    }
 }
 
 template <bool CUBIC>
 static cudaError_t launch_function(const MarchArgs &a, int nviews, cudaStream_t s) {
     switch (a.p.func) {
-        case RC_FUNC_MIP: return launch_function_group<CUBIC, kFnMip>(a, nviews, s);
+        case RC_FUNC_MIP: return launch_reduce<CUBIC, true>(a, nviews, s);
         case RC_FUNC_AVERAGE:
-        case RC_FUNC_XRAY:
-            switch (lanes_per_sum(a)) {
-                case 4: return launch_sum<CUBIC, 4>(a, nviews, s);
-                case 2: return launch_sum<CUBIC, 2>(a, nviews, s);
-                default: return launch_sum<CUBIC, 1>(a, nviews, s);
-            }
-        default: return launch_function_group<CUBIC, kFnFirst>(a, nviews, s);
+        case RC_FUNC_XRAY: return launch_reduce<CUBIC, false>(a, nviews, s);
+        default:
+            return by_storage<false>(a.vol, [&](auto st) {
+                return launch_kernel(function_kernel<decltype(st)::value, CUBIC>, a, nviews,
+                                     a.p.func == RC_FUNC_THRESHOLD, s);
+            });
     }
 }
 

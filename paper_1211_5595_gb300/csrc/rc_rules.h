@@ -115,6 +115,13 @@ inline int lanes_per_ray(const LaunchSize &z, bool heavy) {
     return 1;
 }
 
+// Rays of a view per voxel of the cross-section, as far as it matters.
+inline double pixel_density(const LaunchSize &z) { return z.density < 16.0 ? z.density : 16.0; }
+
+// Samples finer than voxels and voxels not much coarser than pixels: two lanes
+// of a ray share their footprints, and pay however many rays there are.
+inline bool shared_footprints(const LaunchSize &z) { return z.density <= 10.0 && z.steps >= 400.0; }
+
 // Lanes per ray of the sums: every ray marches its whole chord, so no sample is
 // in vain, and what more lanes cost is the ray setup and the shuffles, which
 // short chains do not repay, and the coherence of neighbouring rays, which is
@@ -132,16 +139,28 @@ inline int lanes_per_ray(const LaunchSize &z, bool heavy) {
 // long as one lane at a few samples per ray. Over 578 sizes these lines are
 // within 1.3% of the best choice on average, 9% slower than one lane at worst.
 inline int lanes_per_sum(const LaunchSize &z, bool cubic) {
-    const double d = z.density < 16.0 ? z.density : 16.0;
+    const double d = pixel_density(z);
     if (cubic) {
-        // samples finer than voxels, voxels finer than pixels: two lanes of a ray
-        // share their footprints, however many rays there are
-        const bool shared = d <= 10.0 && z.steps >= 400.0;
-        if (!shared && z.hits > 40e3 + 1600.0 * z.steps) return 1;
+        if (!shared_footprints(z) && z.hits > 40e3 + 1600.0 * z.steps) return 1;
         return z.hits * pow(d, 0.7) <= 80e3 + 1600.0 * z.steps ? 4 : 2;
     }
     if (z.hits * pow(d, 0.4) > 80e3 + 1700.0 * z.steps) return 1;
     return z.hits * sqrt(d) <= 60e3 + 600.0 * z.steps ? 4 : 2;
+}
+
+// Lanes per ray of a maximum: as for the sums, with no shuffle per sample. us
+// with 1, 2 and 4 lanes, FP32 trilinear / B-spline:
+//   256x256x180, 256^2:              278 145 78 / 1172 644 347
+//   128x128x96, 512^2:                92 65 50 / 331 242 208
+//   128x128x96, four 1024^2 views:    475 499 571 / 2057 2089 2398
+//   256x256x180, eight 1024^2 views: 2188 1984 2035
+//   51x302x86, four 870^2 views:      287 230 245 / 1277 917 868
+// Within 1% of the best choice on average over 510 sizes, 16% slower than one
+// lane at worst.
+inline int lanes_per_max(const LaunchSize &z, bool cubic) {
+    const double d = pixel_density(z), x = z.hits * pow(d, cubic ? 0.25 : 0.7);
+    if (!shared_footprints(z) && x > (cubic ? 60e3 + 4000.0 * z.steps : 40e3 + 6000.0 * z.steps)) return 1;
+    return (cubic ? z.hits * sqrt(d) <= 120e3 + 1000.0 * z.steps : x <= 120e3 + 1600.0 * z.steps) ? 4 : 2;
 }
 
 }  // namespace rc

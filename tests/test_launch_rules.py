@@ -43,6 +43,13 @@ int lanes_per_sum(double hits, double steps, double density, int cubic) {
     z.density = density;
     return rc::lanes_per_sum(z, cubic != 0);
 }
+int lanes_per_max(double hits, double steps, double density, int cubic) {
+    rc::LaunchSize z;
+    z.hits = hits;
+    z.steps = steps;
+    z.density = density;
+    return rc::lanes_per_max(z, cubic != 0);
+}
 }
 """
 
@@ -58,7 +65,7 @@ def rules(tmp_path_factory):
                     "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
     lib = C.CDLL(str(d / "shim.so"))
     lib.lanes_per_ray.argtypes = [C.c_double, C.c_double, C.c_int]
-    lib.lanes_per_sum.argtypes = [C.c_double, C.c_double, C.c_double, C.c_int]
+    lib.lanes_per_sum.argtypes = lib.lanes_per_max.argtypes = [C.c_double, C.c_double, C.c_double, C.c_int]
     return lib
 
 
@@ -95,6 +102,16 @@ def test_a_small_image_spreads_over_the_sms(rules, chunks, ctas):
     assert rules.persistent_ctas(chunks, 152) == ctas
 
 
+def orbit_size(rules, dims, size, views, step):
+    """Size of a launch of `views` square views on the orbit that just holds the box."""
+    ext = np.array(dims) - 1.0
+    dist = 1.1 * np.linalg.norm(ext) / 2 / np.sin(np.radians(15.0))
+    el, az = np.radians(20.0), np.radians(12.0 + 360.0 * np.arange(views) / views)
+    return launch_size(rules, dims, ONES, step, [
+        view(dims, ONES, ext / 2 + dist * np.array([np.cos(el) * np.cos(a), np.cos(el) * np.sin(a), np.sin(el)]), ext / 2,
+             (size, size)) for a in az])
+
+
 # a view that looks past the volume or stands far from it changes a launch's
 # size by its own rays only, wherever it stands among the views
 @pytest.mark.parametrize("other", [view(DIMS, ONES, (827.5, 127.5, 89.5), (327.5, 1027.5, 89.5), (1024, 1024)),
@@ -129,12 +146,20 @@ def test_many_views_are_sampled(rules):
     ((40, 40, 40), 1024, 1, 2.0, (1, 1)), ((256, 256, 180), 1024, 1, 0.5, (2, None)),
     ((256, 256, 180), 1024, 4, 0.5, (None, 2)), ((256, 256, 180), 1024, 8, 0.5, (None, 2)), ((51, 302, 86), 870, 4, 0.5, (2, None))])
 def test_lanes_of_sums(rules, dims, size, views, step, lanes):
-    ext = np.array(dims) - 1.0
-    dist = 1.1 * np.linalg.norm(ext) / 2 / np.sin(np.radians(15.0))
-    el, az = np.radians(20.0), np.radians(12.0 + 360.0 * np.arange(views) / views)
-    vs = [view(dims, ONES, ext / 2 + dist * np.array([np.cos(el) * np.cos(a), np.cos(el) * np.sin(a), np.sin(el)]), ext / 2,
-               (size, size)) for a in az]
-    z = launch_size(rules, dims, ONES, step, vs)
+    z = orbit_size(rules, dims, size, views, step)
     for cubic in (0, 1):
         if lanes[cubic]:
             assert rules.lanes_per_sum(*z, cubic) == lanes[cubic], (cubic, z)
+
+
+# the same for maxima
+@pytest.mark.parametrize("dims,size,views,step,lanes", [
+    ((256, 256, 180), 128, 1, 0.5, (4, 4)), ((256, 256, 180), 256, 1, 0.5, (4, 4)),
+    ((512, 512, 256), 512, 2, 0.5, (4, 4)), ((128, 128, 96), 1024, 8, 0.5, (1, None)),
+    ((64, 64, 32), 1448, 1, 0.5, (1, None)), ((256, 256, 180), 1024, 8, 0.5, (2, 2)),
+    ((51, 302, 86), 1024, 4, 0.5, (None, 2))])
+def test_lanes_of_maxima(rules, dims, size, views, step, lanes):
+    z = orbit_size(rules, dims, size, views, step)
+    for cubic in (0, 1):
+        if lanes[cubic]:
+            assert rules.lanes_per_max(*z, cubic) == lanes[cubic], (cubic, z)
