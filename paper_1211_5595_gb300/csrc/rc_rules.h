@@ -25,11 +25,17 @@ struct BoxGeom {
     double s[3];                       // spacing
 };
 
-// About how many rays of a view meet the volume: the box's corners bound the
-// part of the image whose rays can, and its silhouette fills about two thirds
-// of that rectangle.
-inline double view_rays(const ViewGeom &c, const BoxGeom &b) {
-    double hits = 0.65 * c.W * c.H;
+// About how many rays of a view meet the volume, and what part of the box's
+// diagonal they cross: the box's corners bound the part of the image whose rays
+// can, and its silhouette fills about two thirds of that rectangle. From inside
+// the box every ray meets it, and leaves it after about a third of the diagonal.
+inline void view_rays(const ViewGeom &c, const BoxGeom &b, double &hits, double &chord) {
+    const double pixels = (double)c.W * c.H;
+    bool inside = true;
+    for (int i = 0; i < 3; i++) inside = inside && c.o[i] >= 0.0 && c.o[i] <= b.n[i] - 1;
+    chord = inside ? 0.35 : 1.0;
+    hits = inside ? pixels : 0.65 * pixels;
+    if (inside) return;
     double lo[2] = {1.0, 1.0}, hi[2] = {-1.0, -1.0};
     for (int q = 0; q < 8; q++) {
         double z = 0.0, e[2] = {0.0, 0.0};
@@ -39,7 +45,7 @@ inline double view_rays(const ViewGeom &c, const BoxGeom &b) {
             e[0] += d * c.r[i];
             e[1] += d * c.u[i];
         }
-        if (!(z > 0.0)) return hits;                       // a corner behind the eye: the whole image
+        if (!(z > 0.0)) return;                            // a corner behind the eye: the whole image
         e[0] /= z * c.tx;
         e[1] /= z * c.ty;
         for (int i = 0; i < 2; i++) {
@@ -51,15 +57,15 @@ inline double view_rays(const ViewGeom &c, const BoxGeom &b) {
         const double l = lo[i] > -1.0 ? lo[i] : -1.0, h = hi[i] < 1.0 ? hi[i] : 1.0;
         hits *= h > l ? (h - l) * 0.5 : 0.0;
     }
-    return hits;
 }
 
 // The size of a march launch over all its views: rays that meet the volume,
-// samples across the box's diagonal, and the rays of one view per voxel of the
-// box's cross-section (the two-thirds power of its voxels). The views are summed (up to kSizedViews of them,
-// evenly spread): the first one alone says nothing about the others. Eight
-// 1024^2 views of 256x256x180, unshaded, took 3.37 ms instead of 1.14 when the
-// first of them looked past the volume, and 2.07 when it was far away.
+// samples along the diagonal (from inside the box, along their shorter chords),
+// and the rays of one view per voxel of the box's cross-section (the two-thirds
+// power of its voxels). The views are summed (up to kSizedViews of them, evenly
+// spread): the first one alone says nothing about the others. Eight 1024^2 views
+// of 256x256x180, unshaded, took 3.37 ms instead of 1.14 when the first of them
+// looked past the volume, and 2.07 when it was far away.
 struct LaunchSize {
     double hits = 0.0, steps = 0.0, density = 0.0;
 };
@@ -74,21 +80,24 @@ class LaunchSizer {
         across = sqrt(diag2) / step;
     }
     void add(const ViewGeom &c) {
-        hits += view_rays(c, box);
+        double h, part;
+        view_rays(c, box, h, part);
+        hits += h;
+        chords += h * part;
         added++;
     }
     // for `views` views of which the added ones are a sample
     LaunchSize size(double views) const {
         LaunchSize z;
         z.hits = added ? hits * views / added : 0.0;
-        z.steps = across;
+        z.steps = hits > 0.0 ? across * (chords / hits) : across;
         z.density = z.hits / views / pow((double)box.n[0] * box.n[1] * box.n[2], 2.0 / 3.0);
         return z;
     }
 
   private:
     BoxGeom box;
-    double across, hits = 0.0;
+    double across, hits = 0.0, chords = 0.0;
     int added = 0;
 };
 
@@ -97,7 +106,7 @@ class LaunchSizer {
 // its longest ray however few there are; more lanes shorten the chain until the
 // shuffles and the samples past termination fill the GPU. The lines lie where
 // the measured times cross, in rays that meet the volume (`hits`, 0.27 of the
-// pixels there) and per sample across the box (`steps`); us per view with
+// pixels there) and per sample along the diagonal (`steps`); us per view with
 // 1, 2, 4 and 8 lanes, FP32 shaded / FP32 plain:
 //   64x64x32, 256^2:    79 58 46 42 / 68 44 35 40
 //   128x128x96, 384^2: 118 107 74 88 / 102 65 66 73
@@ -105,6 +114,9 @@ class LaunchSizer {
 //   256x256x180, 512^2: 172 142 135 161 / 135 105 99 131
 //   256x256x180, 724^2: 223 201 214 293 / 150 143 162 235
 //   256x256x180, 1024^2: 292 307 386 572 / 193 229 287 456
+// From inside the box the chains are short and every pixel has one, so the
+// lines come sooner: 256x256x180, 128^2 74 61 45 44 / 52 45 35 35, 181^2 76 70 68
+// 79 / 51 51 48 60, 256^2 94 103 116 136 / 57 67 78 102.
 // `heavy`: forms whose samples take longer (shading without 8-byte
 // value+gradient entries, which the FP32 shaded figures above are for;
 // B-spline; 2-D table) gain further up than the others.

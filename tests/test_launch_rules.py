@@ -163,3 +163,15 @@ def test_lanes_of_maxima(rules, dims, size, views, step, lanes):
     for cubic in (0, 1):
         if lanes[cubic]:
             assert rules.lanes_per_max(*z, cubic) == lanes[cubic], (cubic, z)
+
+
+# from inside the box every pixel has a ray, and its chain is short
+@pytest.mark.parametrize("size,lanes", [(64, 8), (128, 4), (256, 1), (1024, 1)])
+def test_lanes_inside_the_box(rules, size, lanes):
+    eye, target = (102.4, 115.2, 90.0), (230.4, 128.0, 108.0)
+    hits, steps, density = launch_size(rules, DIMS, ONES, 0.5, [view(DIMS, ONES, eye, target, (size, size), fovy=60.0)])
+    assert hits == size * size
+    outside = launch_size(rules, DIMS, ONES, 0.5, orbit(1, (size, size)))[1]
+    assert 0.3 * outside < steps < 0.4 * outside
+    assert rules.lanes_per_ray(hits, steps, 0) == lanes
+    assert rules.lanes_per_sum(hits, steps, density, 0) == {64: 4, 128: 4, 256: 4, 1024: 1}[size]
