@@ -420,6 +420,7 @@ __device__ __forceinline__ float value_grad_vg16h(const VolDev &v, const Cell &c
 // voxels give the clamped coordinates.
 template <int ST, bool PAIRS>
 __device__ __forceinline__ float value_grad_x(const VolDev &v, const Cell &c, float g[3]) {
+    static_assert(!PAIRS || (ST & 3) != RC_STORE_F32, "FP32 pairs lie along y: bspline_rows2 reads them");
     const float wx = c.w[0], wy = c.w[1], wz = c.w[2];
     // rows along x at (y, z) = (j-1+oy, k-1+oz): L the centre cell's x edge,
     // M and P those of the -x and +x cells
@@ -560,6 +561,7 @@ __device__ __forceinline__ void bspline_row(const typename Voxel<ST>::T *a, cons
 
 template <int ST, bool PAIRS>
 __device__ __forceinline__ float bspline_x(const VolDev &v, const Cell &c) {
+    static_assert(!PAIRS || (ST & 3) != RC_STORE_F32, "FP32 pairs lie along y: bspline_rows2 reads them");
     const auto *a = cell_ptr<ST>(v, c) - (int)(kDX + kDY + kDZ);     // voxel (i-1, j-1, k-1)
     const typename Pair<ST>::T *pp = PAIRS ? pair_ptr<ST>(v, c) : nullptr;
     float wx[4], wy[4], wz[4];
@@ -590,6 +592,7 @@ __device__ __forceinline__ float bspline_x(const VolDev &v, const Cell &c) {
 // their derivatives; 1/s = 2 * (0.5/s) exactly.
 template <int ST, bool PAIRS>
 __device__ __forceinline__ float bspline_grad_x(const VolDev &v, const Cell &c, float g[3]) {
+    static_assert(!PAIRS || (ST & 3) != RC_STORE_F32, "FP32 pairs lie along y: bspline_rows2 reads them");
     const auto *a = cell_ptr<ST>(v, c) - (int)(kDX + kDY + kDZ);     // voxel (i-1, j-1, k-1)
     const typename Pair<ST>::T *pp = PAIRS ? pair_ptr<ST>(v, c) : nullptr;
     float wx[4], wy[4], wz[4], dx[4], dy[4], dz[4];
@@ -693,18 +696,22 @@ __device__ __forceinline__ float bspline_rows2(const VolDev &v, const Cell &c, f
 // sample), else from the apron brick; both read the same stored values.
 template <int ST>
 __device__ __forceinline__ float bspline(const VolDev &v, const Cell &c) {
-    if (ST == RC_STORE_F32 && v.pairs != nullptr) {
+    if constexpr ((ST & 3) == RC_STORE_F32) {
         float g[3];
-        return bspline_rows2<false>(v, c, g);
+        if (v.pairs != nullptr) return bspline_rows2<false>(v, c, g);
+    } else if constexpr ((ST & 3) == RC_STORE_F16) {
+        if (v.pairs != nullptr) return bspline_x<ST, true>(v, c);
     }
-    if (ST == RC_STORE_F16 && v.pairs != nullptr) return bspline_x<ST, true>(v, c);
     return bspline_x<ST, false>(v, c);
 }
 
 template <int ST>
 __device__ __forceinline__ float bspline_grad(const VolDev &v, const Cell &c, float g[3]) {
-    if (ST == RC_STORE_F32 && v.pairs != nullptr) return bspline_rows2<true>(v, c, g);
-    if (ST == RC_STORE_F16 && v.pairs != nullptr) return bspline_grad_x<ST, true>(v, c, g);
+    if constexpr ((ST & 3) == RC_STORE_F32) {
+        if (v.pairs != nullptr) return bspline_rows2<true>(v, c, g);
+    } else if constexpr ((ST & 3) == RC_STORE_F16) {
+        if (v.pairs != nullptr) return bspline_grad_x<ST, true>(v, c, g);
+    }
     return bspline_grad_x<ST, false>(v, c, g);
 }
 
