@@ -83,7 +83,7 @@ typedef enum {
  * V * b(dx) b(dy) b(dz), b(x) = (4 - 6x^2 + 3|x|^3)/6 for |x| < 1,
  * (2 - |x|)^3/6 for 1 <= |x| < 2; indices outside the volume take the
  * nearest border voxel. Gradient: the analytic derivative of that sum. Every
- * ray function supports it; the table gradient and the learned proposal do
+ * ray function and the table gradient support it; the learned proposal does
  * not (RC_ERR_UNSUPPORTED). */
 typedef enum { RC_FILTER_TRILINEAR = 0, RC_FILTER_BSPLINE = 1 } rc_filter;
 

@@ -890,12 +890,14 @@ static rc_status ensure_grid(rc_context *ctx, rc_volume *v, int f) {
     return RC_OK;
 }
 
-// The pair bricks of FP32 and FP16 volumes, allocated on the first render
-// that reads them and rebuilt after new data: B-spline renders, and
-// trilinear renders of FP16 volumes that need the gradient footprint
-// (shading, a 2-D table, the isosurface's shading). FP32 trilinear renders
-// read the value+gradient bricks; uint16 volumes read the apron bricks
-// (widening 16-bit integer pairs cost more than the loads they save).
+// The pair bricks of FP32 and FP16 volumes, allocated and built on the first
+// render of a form that may read them and rebuilt after new data: B-spline
+// renders, and trilinear renders of FP16 volumes that need the gradient
+// footprint (shading, a 2-D table, the isosurface's shading). Trilinear
+// gradients come from the value+gradient bricks where a volume has them, so of
+// the latter only volumes with vmax > 4096 read the pairs built here. uint16
+// volumes read the apron bricks (widening 16-bit integer pairs cost more than
+// the loads they save).
 static rc_status prepare_filter(rc_context *ctx, rc_volume *v, const rc_render_params *p) {
     const bool grad = p->shade || ctx->M >= 2 || p->func == RC_FUNC_ISO;
     const bool need = v->storage != RC_STORE_U16 &&
@@ -908,15 +910,17 @@ static rc_status prepare_filter(rc_context *ctx, rc_volume *v, const rc_render_p
     return RC_OK;
 }
 
-// The occupancy mask of filter f under the current table, rebuilt when the
-// table or the data changed since it was last built.
+// What skips empty space under the current table with filter f, rebuilt when the
+// table or the data changed since it was last built: the cell-brick mask (read
+// by the proposal's features and ranges and by rc_skip_mask_get) and the empty
+// levels (read by the marches and gradients).
 static rc_status ensure_occupancy(rc_context *ctx, rc_volume *v, int f) {
     if (v->occ_tf_version[f] == ctx->tf_version && v->occ_data_version[f] == v->data_version) return RC_OK;
     rc_status st = ensure_grid(ctx, v, f);
     if (st != RC_OK) return st;
     TFDev tf = tf_dev(ctx, v);
     const int f16o = v->storage == RC_STORE_F16 ? f16_offset(v->vmax) : 0;
-    RC_CUDA(ctx, launch_occupancy(v->d_mn[f], v->d_mx[f], v->nbricks, v->vmax, f16o, tf, v->d_occ[f], ctx->stream));
+    RC_CUDA(ctx, launch_occupancy(v->d_mn[f], v->d_mx[f], v->nbricks, f16o, tf, v->d_occ[f], ctx->stream));
     RC_CUDA(ctx, launch_levels(v->d_mn4[f], v->d_mx4[f], v->n, v->cb, f16o, tf, v->d_lvl[f], ctx->stream));
     v->occ_tf_version[f] = ctx->tf_version;
     v->occ_data_version[f] = v->data_version;

@@ -227,8 +227,8 @@ cudaError_t launch_prep(const uint16_t *stage, VolDev v, void *apron, void *vg, 
 cudaError_t launch_minmax(const uint16_t *stage, const int n[3], const int cb[3], int vmax, int filter,
                           uint16_t *mn, uint16_t *mx, cudaStream_t s);
 // f16o: 0 for raw codes; for FP16 storage the offset o of its values.
-cudaError_t launch_occupancy(const uint16_t *mn, const uint16_t *mx, int nbricks, int vmax,
-                             int f16o, TFDev tf, uint8_t *occ, cudaStream_t s);
+cudaError_t launch_occupancy(const uint16_t *mn, const uint16_t *mx, int nbricks, int f16o, TFDev tf, uint8_t *occ,
+                             cudaStream_t s);
 // 4^3 sub-block min/max grid of a filter (cells 4j..4j+3; footprint voxels
 // 4j..4j+4, or 4j-1..4j+5 for the B-spline, clamped) and the empty
 // levels built from it: one byte per sub-block.

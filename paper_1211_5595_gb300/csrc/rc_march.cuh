@@ -1,8 +1,8 @@
 // Forward march kernels (Sec. 4.1-4.2): one thread per ray, warps on 8 x 4
-// pixel tiles, bricked volume gathers through the read-only path, transfer
-// function in shared memory (1-D) or global memory (2-D), exact empty-space
-// skipping over the cell-brick occupancy mask and warp-vote early ray
-// termination. The instances are spread over several translation units
+// pixel tiles (several lanes per ray in small launches), bricked volume gathers
+// through the read-only path, transfer function in shared memory (1-D) or global
+// memory (2-D), exact empty-space skipping by one empty level per 4^3 sub-block
+// and early ray termination lane by lane. The instances are spread over several translation units
 // (rc_march.cu, rc_march_cubic.cu, rc_march_tf2.cu) so they compile in parallel.
 #pragma once
 
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kMarchThreads) function_kernel(const MarchArgs
 // MIP takes every sample: in noise the maxima of 4^3 blocks lie above any value
 // reconstructed in them, so skipping by them (as function_kernel does) left 60%
 // of the samples of a head phantom and a longer chain per sample. One 128^2 view
-// of 256x256x180, us: 304 with skipping, 171 with one lane and every sample, 43
+// of 256x256x180, us: 304 with skipping, 171 with one lane and every sample, 65
 // with the lanes; eight 1024^2 views 1992, 2188 and 1984.
 template <int ST, bool CUBIC, int L, bool MAX>
 __global__ void __launch_bounds__(kMarchThreads) reduce_kernel(const MarchArgs a) {

@@ -397,9 +397,8 @@ __global__ void occupancy_kernel(const uint16_t *mn, const uint16_t *mx, int nbr
     occ[b] = any;
 }
 
-cudaError_t launch_occupancy(const uint16_t *mn, const uint16_t *mx, int nbricks, int vmax, int f16o,
-                             TFDev tf, uint8_t *occ, cudaStream_t s) {
-    (void)vmax;
+cudaError_t launch_occupancy(const uint16_t *mn, const uint16_t *mx, int nbricks, int f16o, TFDev tf, uint8_t *occ,
+                             cudaStream_t s) {
     occupancy_kernel<<<(nbricks + 127) / 128, 128, 0, s>>>(mn, mx, nbricks, f16o, tf, occ);
     return cudaGetLastError();
 }
