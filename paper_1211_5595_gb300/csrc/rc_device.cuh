@@ -325,18 +325,26 @@ __device__ __forceinline__ float value_grad_vg(const VolDev &v, const Cell &c, f
     return r.x;
 }
 
+// 2^23 plus the upper 16 bits of x, as the bits of that float. On the FMA pipe:
+// the ALU pipe, with the lower halves' byte permutes, is the busier one (50%
+// against 34% with all four fields permuted). Shaded FP32 at 1024^2, us: a view
+// from inside 256x256x180 993 -> 968, 128x128x96 942 -> 918, 12 orbit views of
+// 256x256x180 2567 -> 2521 (both halves on the FMA pipe, or a dot product of
+// bytes instead of the multiply: 990 and 986 for the first).
+__device__ __forceinline__ unsigned high_field(unsigned x) {
+    unsigned r;
+    asm("mad.hi.u32 %0, %1, 65536, 0x4B000000;" : "=r"(r) : "r"(x));
+    return r;
+}
+
 // A uint16 value+gradient entry as biased FP32 pairs (V + m0, D_x + m1) and
-// (D_y + m1, D_z + m1), exactly: a byte permute places each 16-bit field in
-// the mantissa of 2^23, so m0 = 2^23 for the value and m1 = 2^23 + 32768 for
-// the offset differences.
+// (D_y + m1, D_z + m1), exactly: each 16-bit field placed in the mantissa of
+// 2^23, so m0 = 2^23 for the value and m1 = 2^23 + 32768 for the offset
+// differences.
 __device__ __forceinline__ ulonglong2 vg16_biased(uint2 q) {
     unsigned long long a, b;
-    asm("mov.b64 %0, {%1, %2};"
-        : "=l"(a)
-        : "r"(__byte_perm(q.x, 0x4B000000u, 0x7610)), "r"(__byte_perm(q.x, 0x4B000000u, 0x7632)));
-    asm("mov.b64 %0, {%1, %2};"
-        : "=l"(b)
-        : "r"(__byte_perm(q.y, 0x4B000000u, 0x7610)), "r"(__byte_perm(q.y, 0x4B000000u, 0x7632)));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "r"(__byte_perm(q.x, 0x4B000000u, 0x7610)), "r"(high_field(q.x)));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "r"(__byte_perm(q.y, 0x4B000000u, 0x7610)), "r"(high_field(q.y)));
     return make_ulonglong2(a, b);
 }
 
