@@ -325,12 +325,13 @@ __device__ __forceinline__ float value_grad_vg(const VolDev &v, const Cell &c, f
     return r.x;
 }
 
-// 2^23 plus the upper 16 bits of x, as the bits of that float. On the FMA pipe:
-// the ALU pipe, with the lower halves' byte permutes, is the busier one (50%
-// against 34% with all four fields permuted). Shaded FP32 at 1024^2, us: a view
-// from inside 256x256x180 993 -> 968, 128x128x96 942 -> 918, 12 orbit views of
-// 256x256x180 2567 -> 2521 (both halves on the FMA pipe, or a dot product of
-// bytes instead of the multiply: 990 and 986 for the first).
+// 2^23 plus the upper 16 bits of x, as the bits of that float. A multiply-add
+// instead of a byte permute like the lower fields': the same number of
+// instructions, but fewer of them held back at dispatch (0.51 instead of 0.59
+// per issue, issue 79% instead of 77.5%). Shaded at 1024^2, us: a view from
+// inside 256x256x180 993 -> 968, 128x128x96 942 -> 918, 12 orbit views of
+// 256x256x180 2567 -> 2521. (Lower fields by multiplies too 990 for the first,
+// upper ones by a dot product of bytes 986, all by dot products 1076.)
 __device__ __forceinline__ unsigned high_field(unsigned x) {
     unsigned r;
     asm("mad.hi.u32 %0, %1, 65536, 0x4B000000;" : "=r"(r) : "r"(x));
@@ -500,7 +501,8 @@ __device__ __forceinline__ float value_grad_x(const VolDev &v, const Cell &c, fl
 // entries as uint16: the same integers, so the same result, from half the L1
 // bytes of float4 entries (12 shaded views of 256x256x180 at 1024^2 2.61 -> 2.55
 // ms, 4 views with a 2-D table at 768^2 1.29 -> 1.16, 6 proposal views 0.90 ->
-// 0.86, and half the bytes to write per upload).
+// 0.86, and half the bytes to write per upload; where every sample is evaluated,
+// as in views from inside the volume, the decode costs 3-4%: 930 -> 968 us).
 template <int ST>
 __device__ __forceinline__ float value_grad(const VolDev &v, const Cell &c, float g[3]) {
     if constexpr (ST == RC_STORE_F32 || ST == RC_STORE_U16) return value_grad_vg16(v, c, g);
